@@ -194,6 +194,16 @@ csaw_status launch_walk_host(const CdfView& c, const uint64_t* off, const uint32
 csaw_status walk_batch_cached(const csaw_graph* g, int kind, const uint32_t* d_starts, uint64_t n,
                               const WalkSegments& seg, uint32_t max_len, uint32_t* d_path, cudaStream_t s);
 
+// node2vec walks by list intersection (csaw_walk_n2v.cu), over an index of
+// the rows and weight summaries built in the call.  *done = false without an error when
+// their memory cannot be had: the caller then streams the rows.  next_walker:
+// a zeroed device counter.
+csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,
+                     uint32_t length, uint64_t rng_seed, uint32_t tele, uint32_t tele_q32, uint32_t* path,
+                     unsigned long long* next_walker, cudaStream_t s, bool* done);
+// Whether a call of n walks of `length` steps is large enough for it.
+bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length);
+
 // Whether selection/walks of this kind can use a cached cumulative array:
 // uniform always (implicit), edge weight / neighbour degree when built and
 // no bias of the kind is zero.

@@ -1072,7 +1072,11 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
             max_bias = (uint64_t)g->max_weight * m;
         }
         timer.mark(1, s);
-        st = launch_walk(kind, max_bias, p, g->sm_count, s);
+        bool done = false;
+        if (kind == CSAW_BIAS_NODE2VEC && n2v_index_pays(g, n_walkers, length))
+            st = walk_n2v(g, bias, max_bias, d_starts, n_walkers, length, rng_seed, p.tele, p.tele_q32, d_path,
+                          p.next_walker, s, &done);
+        if (st == CSAW_OK && !done) st = launch_walk(kind, max_bias, p, g->sm_count, s);
         timer.mark(2, s);
     }
     dfree(counter, s);
