@@ -131,7 +131,9 @@ csaw_status csaw_graph_get_info(const csaw_graph* g, csaw_graph_info* out);
  * (CSAW_BIAS_EDGE_WEIGHT or CSAW_BIAS_NEIGHBOR_DEGREE): per edge e of row v,
  * the inclusive uint64 prefix sum of the row's biases up to e -- the CTPS of
  * Sec. II-B computed once instead of at every selection -- and a summary of
- * every 8th sum (9 bytes per edge in all).
+ * every 8th sum (9.1 bytes per edge in all), and for walks, where the biases
+ * are below 2^26 and memory allows, the biases packed beside their columns
+ * with running sums (8.6 bytes per edge + 16 per vertex).
  * Afterwards csaw_walk, csaw_sample and plans created later use it for that
  * kind: a walk step or a draw is a binary search (O(log d)) instead of a pass
  * over the row.  Picks are identical (same prefix sums, same draws).  Graphs
@@ -181,7 +183,11 @@ csaw_status csaw_graph_set_allocator(csaw_graph* g, csaw_alloc_fn alloc, csaw_fr
  * >= n_vertices for host inputs, n_walkers >= 2^32), CSAW_ERR_OVERFLOW
  * (node2vec: max weight * max multiplier >= 2^32), CSAW_ERR_NOMEM,
  * CSAW_ERR_CUDA.  With device inputs an out-of-range start is caught on the
- * device: its row is filled with CSAW_NONE. */
+ * device: its row is filled with CSAW_NONE.  A call with enough steps for it
+ * builds search structures of the whole graph into stream-ordered temporaries
+ * (static biases: as for build_cdf below; node2vec: an index of the rows, 4
+ * bytes per edge + 40 per vertex, and the weights' summaries); where they do
+ * not fit in memory, the rows are streamed. */
 csaw_status csaw_walk(csaw_graph* g, const uint32_t* starts, uint64_t n_walkers, uint32_t length,
                       const csaw_bias* bias, uint64_t rng_seed, uint32_t* path, int mem_kind,
                       void* stream);
@@ -196,23 +202,22 @@ csaw_status csaw_walk(csaw_graph* g, const uint32_t* starts, uint64_t n_walkers,
  * draw of attempt 2 (jump), instead of to a neighbour.  A walker at a vertex
  * with no neighbour of positive bias teleports the same way instead of
  * stopping.  After a teleport a node2vec walk has no previous vertex (its
- * next step uses the weights alone).  Teleporting walks always stream the
- * biases (a cached cumulative array is not used).
+ * next step uses the weights alone).
  * build_cdf = 1 (no teleport, static bias whose biases are all positive, no
- * cached array of the kind on g): the call first builds the cumulative array
- * of the kind over the whole graph, as csaw_graph_build_cdf does, into a
- * temporary of 9 bytes per edge (stream-ordered, freed by the call), and
- * every step is then a search of it instead of a pass over the row: the
- * same paths, with the array's construction inside the call.  Ignored
- * otherwise.  For edge weights the temporary holds only the summaries of the
- * prefix sums (every 8th and 64th) and per-vertex records {start, end,
- * total}, about 1.14 bytes per edge + 32 per vertex, and a step forms its
- * 8-edge group's sums from the weights; for neighbour degree it holds the
- * whole array (9 bytes per edge + 32 per vertex).
+ * cached array of the kind on g): the call first builds a search array of the
+ * kind over the whole graph into a temporary (stream-ordered, freed by the
+ * call), and every step is then a search of it instead of a pass over the row:
+ * the same paths, with the array's construction inside the call.  Ignored
+ * otherwise.  Biases below 2^26: the packed array (8.6 bytes per edge + 16 per
+ * vertex).  Larger ones: for edge weights the summaries of the prefix sums
+ * (every 8th and 64th) and per-vertex records {start, end, total}, about 1.14
+ * bytes per edge + 32 per vertex, and a step forms its 8-edge group's sums
+ * from the weights; for neighbour degree the whole cumulative array (9 bytes
+ * per edge + 32 per vertex).
  * phase_ms (not NULL): the call records CUDA events on `stream` around its
  * phases, waits for the stream, and stores the device time of the array's
- * construction in phase_ms[0] (0 when nothing is built) and of the walk
- * kernels in phase_ms[1].  Errors: those of csaw_walk, and CSAW_ERR_INVALID
+ * construction in phase_ms[0] (0 without build_cdf; what a plain call builds
+ * by itself counts as walking) and of the walk kernels in phase_ms[1].  Errors: those of csaw_walk, and CSAW_ERR_INVALID
  * for an unknown teleport mode. */
 #define CSAW_TELEPORT_NONE 0
 #define CSAW_TELEPORT_RESTART 1

@@ -243,7 +243,10 @@ extern "C" csaw_status csaw_graph_destroy(csaw_graph* g)
 {
     clear_error();
     if (!g) return CSAW_OK;
-    for (int k = 0; k < 4; ++k) free_with(g->cdf_alloc[k], g->cdf[k], nullptr);
+    for (int k = 0; k < 4; ++k) {
+        free_with(g->cdf_alloc[k], g->cdf[k], nullptr);
+        free_with(g->cdf_alloc[k], g->pack[k], nullptr);
+    }
     cudaFree(g->off);
     cudaFree(g->col);
     cudaFree(g->w);
@@ -720,6 +723,16 @@ extern "C" csaw_status csaw_graph_build_cdf(csaw_graph* g, int32_t bias_kind, vo
     const size_t bytes = sizeof(uint64_t) * cdf_words(g->E, g->V);
     CSAW_TRY(alloc_with(&g->allocator, (void**)&cdf, bytes, s));
     csaw_status st = enqueue_cdf_build(g, bias_kind, cdf, s);
+    // the packed array for walks, where the biases fit it and memory allows
+    // (without it they search the cumulative array)
+    uint64_t* pack = nullptr;
+    const size_t pack_bytes = sizeof(uint64_t) * pack_layout(g->E, g->V).words;
+    if (st == CSAW_OK && pack_fits(g, bias_kind)) {
+        if (alloc_with(&g->allocator, (void**)&pack, pack_bytes, s) == CSAW_OK)
+            st = enqueue_pack_build(g, bias_kind, pack, s);
+        else
+            clear_error();
+    }
     if (st == CSAW_OK) {
         const cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_fail(e, "build cumulative array");
@@ -727,11 +740,13 @@ extern "C" csaw_status csaw_graph_build_cdf(csaw_graph* g, int32_t bias_kind, vo
     if (st != CSAW_OK) {
         cudaStreamSynchronize(s);
         free_with(g->allocator, cdf, s);
+        free_with(g->allocator, pack, s);
         return st;
     }
     g->cdf[bias_kind] = cdf;
+    g->pack[bias_kind] = pack;
     g->cdf_alloc[bias_kind] = g->allocator;
-    g->device_bytes += bytes;
+    g->device_bytes += bytes + (pack ? pack_bytes : 0);
     return CSAW_OK;
 }
 
@@ -758,6 +773,11 @@ extern "C" csaw_status csaw_graph_drop_cdf(csaw_graph* g, int32_t bias_kind)
         free_with(g->cdf_alloc[bias_kind], g->cdf[bias_kind], nullptr);
         g->cdf[bias_kind] = nullptr;
         g->device_bytes -= sizeof(uint64_t) * cdf_words(g->E, g->V);
+        if (g->pack[bias_kind]) {
+            free_with(g->cdf_alloc[bias_kind], g->pack[bias_kind], nullptr);
+            g->pack[bias_kind] = nullptr;
+            g->device_bytes -= sizeof(uint64_t) * pack_layout(g->E, g->V).words;
+        }
     }
     return CSAW_OK;
 }

@@ -40,6 +40,8 @@ struct csaw_graph {
     // cached per-edge inclusive prefix sums of a static bias kind (or null):
     // cdf[kind][e] = b(row start) + ... + b(e) within e's row
     uint64_t* cdf[4] = {nullptr, nullptr, nullptr, nullptr};
+    // beside it the packed search array that walks use (PackView), or null
+    uint64_t* pack[4] = {nullptr, nullptr, nullptr, nullptr};
     // selection launch shape per bias kind (0 = default): warp-item degree
     // threshold and resident blocks per SM
     uint32_t tune_theta_w[4] = {0, 0, 0, 0};
@@ -163,26 +165,6 @@ bool host_register(void* p, size_t bytes);
 void launch_partition_check(uint32_t* col, uint32_t* w, uint64_t ne, uint32_t V, const uint32_t* deg,
                             uint32_t* err, cudaStream_t s);
 
-// Walks that read a cached cumulative array (or, for uniform bias, none):
-// one thread per walker.  Defined in csaw_walk.cu.
-// cdf: the kind's cumulative array (cdf_words(E, V) words; ignored for
-// uniform); leaf = false: summaries and records only, the leaf level formed
-// from the edge weights (edge-weight bias).  Walkers w0 .. w0+n-1 of the
-// call: starts and path point at walker w0's entries, and walker w0 + i
-// draws as walker w0 + i.  Defined in csaw_walk_cdf.cu.
-csaw_status launch_walk_cached(const csaw_graph* g, int kind, const uint64_t* cdf, bool leaf,
-                               const uint32_t* starts, uint64_t w0, uint64_t n, uint32_t length, uint64_t rng_seed,
-                               uint32_t* path, cudaStream_t s);
-// The same walks with the path matrix copied to host memory h_path: the
-// walkers run in a few chunks on s, and each chunk's rows are copied out on
-// a second stream while the next chunk walks.  Returns after the copies.
-// The host starts h_starts (the source of d_starts) are checked while the
-// walks run: CSAW_ERR_INVALID for a start that is not a vertex.
-// walked (or null) is recorded on s after the last walk kernel.
-csaw_status walk_cached_to_host(const csaw_graph* g, int kind, const uint64_t* cdf, bool leaf,
-                                const uint32_t* h_starts, const uint32_t* d_starts, uint64_t n, uint32_t length,
-                                uint64_t rng_seed, uint32_t* d_path, uint32_t* h_path, cudaStream_t s,
-                                cudaEvent_t walked);
 // Walks over CSR arrays in host memory, read in place (coherent access to
 // host memory): off, col and w (null: uniform) are host arrays, c holds
 // device summaries and records of the weights (no leaf level).
@@ -250,6 +232,77 @@ __host__ __device__ inline CdfView cdf_view(const uint64_t* base, uint64_t E, ui
     c.rec = base + L.rec;
     return c;
 }
+// The packed search array of a static bias.  P[e] is the sum of the biases of
+// edges 0 .. e, over all rows; a row's own prefix sums are P[e] - P[start - 1].
+//   pack[g][16]  per 8-edge group its biases, then its columns (64 bytes)
+//   s1[g]        P at the group's end less P at its 64-edge block's start, 32 bits
+//   s2[h]        P at the end of block h
+//   rec[v]       {off[v], P before off[v]}, v <= V
+// Edges are padded with zero biases to whole chunks.
+constexpr uint64_t PACK_CHUNK = 8192;
+struct PackLayout {
+    uint64_t chunks, s1, s2, rec, words;   // word (8-byte) offsets and the total; pack at word 0
+};
+__host__ __device__ inline PackLayout pack_layout(uint64_t E, uint64_t V)
+{
+    PackLayout L;
+    L.chunks = (E + PACK_CHUNK - 1) / PACK_CHUNK;
+    L.s1 = L.chunks * PACK_CHUNK;
+    L.s2 = L.s1 + L.chunks * (PACK_CHUNK / 16);
+    L.rec = L.s2 + L.chunks * (PACK_CHUNK / 64);
+    L.words = L.rec + 2 * (V + 1);
+    return L;
+}
+struct PackView {
+    const uint32_t* pack = nullptr;
+    const uint32_t* s1 = nullptr;
+    const uint64_t* s2 = nullptr;
+    const uint64_t* rec = nullptr;
+};
+__host__ __device__ inline PackView pack_view(const uint64_t* words, uint64_t E, uint64_t V)
+{
+    PackView k;
+    if (!words) return k;
+    const PackLayout L = pack_layout(E, V);
+    k.pack = (const uint32_t*)words;
+    k.s1 = (const uint32_t*)(words + L.s1);
+    k.s2 = words + L.s2;
+    k.rec = words + L.rec;
+    return k;
+}
+// Whether the kind's biases fit the packed array: weights or degrees below
+// 2^26, so that a block's sums fit 32 bits.
+bool pack_fits(const csaw_graph* g, int kind);
+// Enqueues its build into pack_layout(E, V).words words on s.  Defined in
+// csaw_pack.cu.
+csaw_status enqueue_pack_build(const csaw_graph* g, int kind, uint64_t* words, cudaStream_t s);
+
+// Walks that search an array of a static bias (or, for uniform bias, none):
+// one thread per walker.  Defined in csaw_walk_cdf.cu.
+// How a step finds its pick: uniform (x itself), the cumulative array's leaf
+// level, its summaries and the weights (w_search, no leaf level), or the
+// packed array.
+enum : int { WC_UNIFORM = 0, WC_LEAF = 1, WC_WEIGHTS = 2, WC_PACK = 3 };
+struct WalkArray {
+    int mode = WC_UNIFORM;
+    CdfView c;                 // WC_LEAF, WC_WEIGHTS
+    PackView k;                // WC_PACK
+    uint32_t tele = 0;         // CSAW_TELEPORT_* (WC_UNIFORM and WC_PACK)
+    uint32_t tele_q32 = 0;
+};
+// Walkers w0 .. w0+n-1 of the call: starts and path point at walker w0's
+// entries, and walker w0 + i draws as walker w0 + i.
+csaw_status launch_walk_cached(const csaw_graph* g, const WalkArray& arr, const uint32_t* starts, uint64_t w0,
+                               uint64_t n, uint32_t length, uint64_t rng_seed, uint32_t* path, cudaStream_t s);
+// The same walks with the path matrix copied to host memory h_path: the
+// walkers run in a few chunks on s, and each chunk's rows are copied out on
+// a second stream while the next chunk walks.  Returns after the copies.
+// The host starts h_starts (the source of d_starts) are checked while the
+// walks run: CSAW_ERR_INVALID for a start that is not a vertex.
+// walked (or null) is recorded on s after the last walk kernel.
+csaw_status walk_cached_to_host(const csaw_graph* g, const WalkArray& arr, const uint32_t* h_starts,
+                                const uint32_t* d_starts, uint64_t n, uint32_t length, uint64_t rng_seed,
+                                uint32_t* d_path, uint32_t* h_path, cudaStream_t s, cudaEvent_t walked);
 uint64_t cdf_words(uint64_t E, uint64_t V);
 
 // Summaries and records alone (edge weights, no leaf level), in one
@@ -375,6 +428,29 @@ __device__ __forceinline__ uint64_t philox_draw(const PhiloxKeys& K, uint32_t at
         c3 = (uint32_t)p0;
     }
     return ((uint64_t)c1 << 32) | (uint64_t)c0;
+}
+
+// 32-byte loads and stores: one instruction (and one tag look-up) per sector
+// where a lane's neighbours are elsewhere.  _stream: lines that are not read
+// again soon.
+__device__ __forceinline__ void ld256(const uint64_t* p, uint64_t (&v)[4])
+{
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
+}
+__device__ __forceinline__ void ld256(const uint32_t* p, uint32_t (&v)[8])
+{
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p));
+}
+__device__ __forceinline__ void ld256_stream(const uint32_t* p, uint32_t (&v)[8])
+{
+    asm("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p));
+}
+__device__ __forceinline__ void st256_stream(uint32_t* p, const uint32_t (&v)[8])
+{
+    asm volatile("st.global.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
 }
 
 // x = floor(r * T / 2^64), the draw placed in [0, T).
@@ -532,6 +608,81 @@ __device__ __forceinline__ uint64_t w_search(const CdfView& c, const uint32_t* _
         }
     }
     return hit;
+}
+
+// The column of the smallest e in [beg, end) with P[e] > y in a packed array,
+// for y in [P[beg - 1], P[end - 1]).  P does not decrease over all edges, so
+// the search is over all blocks, started where the draw r would fall if the
+// row's biases were equal: four block ends are read at once (one sector, and
+// the end before them), which holds the answer for most rows; otherwise a
+// galloping search goes on from there.  Then one sector of the block's group
+// sums and the group's biases and columns: four dependent loads a step, with
+// the record, against ten or so for the bisected summaries (cdf_group), and
+// one 64-byte line per pick where weights and column were two.
+__device__ __forceinline__ uint32_t pack_pick(const PackView& k, uint64_t beg, uint64_t end, uint64_t r, uint64_t y)
+{
+    uint64_t at = (beg + __umul64hi(r, end - beg)) >> 8;   // 256-edge window
+    uint64_t v[4];
+    ld256(k.s2 + 4 * at, v);
+    uint64_t before = at ? __ldg(k.s2 + 4 * at - 1) : 0ull;
+    if (before > y || v[3] <= y) {
+        // first window whose end exceeds y, in [lo, hi]
+        uint64_t lo = beg >> 8, hi = (end - 1) >> 8;
+        if (v[3] <= y) {
+            lo = at + 1;
+            for (uint64_t step = 1; lo + step - 1 < hi; step <<= 1) {
+                const uint64_t q = lo + step - 1;
+                if (__ldg(k.s2 + 4 * q + 3) > y) {
+                    hi = q;
+                    break;
+                }
+                lo = q + 1;
+            }
+        } else {
+            hi = at - 1;
+            for (uint64_t step = 1; lo < hi; step <<= 1) {
+                const uint64_t q = hi - (step < hi - lo ? step : hi - lo);
+                if (__ldg(k.s2 + 4 * q + 3) <= y) {
+                    lo = q + 1;
+                    break;
+                }
+                hi = q;
+            }
+        }
+        while (lo < hi) {
+            const uint64_t mid = lo + ((hi - lo) >> 1);
+            if (__ldg(k.s2 + 4 * mid + 3) > y) hi = mid; else lo = mid + 1;
+        }
+        at = lo;
+        ld256(k.s2 + 4 * at, v);
+        before = at ? __ldg(k.s2 + 4 * at - 1) : 0ull;
+    }
+    uint64_t h = 4 * at;
+    if (v[0] <= y) { before = v[0]; ++h; }
+    if (v[1] <= y) { before = v[1]; ++h; }
+    if (v[2] <= y) { before = v[2]; ++h; }
+    uint32_t x = (uint32_t)(y - before);
+    uint32_t s[8];
+    ld256(k.s1 + 8 * h, s);
+    uint64_t g = 8 * h;
+    uint32_t sub = 0;
+#pragma unroll
+    for (int j = 0; j < 7; ++j)
+        if (s[j] <= x) {
+            sub = s[j];
+            ++g;
+        }
+    x -= sub;
+    uint32_t b[8], c[8];
+    ld256_stream(k.pack + 16 * g, b);
+    ld256_stream(k.pack + 16 * g + 8, c);
+    uint32_t sum = 0, pick = c[0];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+        sum += b[j];
+        if (sum <= x) pick = c[j + 1];
+    }
+    return pick;
 }
 
 }  // namespace csaw

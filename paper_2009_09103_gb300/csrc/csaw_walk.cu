@@ -19,6 +19,7 @@
 // 32-entry block per warp (lane j holds entry 32*blk + j) and written with
 // one coalesced store per block.
 #include <atomic>
+#include <cmath>
 
 #include "csaw_internal.cuh"
 
@@ -923,6 +924,20 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
     return st;
 }
 
+// Whether building the packed array for one call pays.  In ps, with the chip
+// full: streaming a step costs about 250 + 0.3 per neighbour of the row (RMAT
+// s18 and s20; degrees are gathered, about three times that), the array 4 per
+// edge (degrees 8) and its launches 25 us.  The mean visited degree is taken
+// as sqrt(mean degree * largest degree), which RMAT graphs meet (950 at s18)
+// and which is the degree itself on a regular graph.
+static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length)
+{
+    const double gather = kind == CSAW_BIAS_NEIGHBOR_DEGREE ? 3.0 : 1.0;
+    const double visited = std::sqrt((double)g->E / (double)g->V * (double)g->max_degree);
+    return (double)n * (double)length * (250.0 + 0.3 * gather * visited) >=
+           (gather > 1.0 ? 8.0 : 4.0) * (double)g->E + 25e6;
+}
+
 // CUDA events around a call's phases, when the caller asks for their times:
 // [0] before the array's construction, [1] before the walk, [2] after it.
 struct PhaseTimer {
@@ -982,11 +997,48 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
 
     const uint32_t* d_starts = starts;
     uint32_t* d_path = path;
-    // static bias with a positive cumulative array: the graph's cached one,
-    // or (build_cdf) one built for this call into a stream-ordered temporary
-    const bool cached = cached_cdf_usable(g, kind);
-    const bool build = !cached && opts && opts->build_cdf && cdf_kind_positive(g, kind);
-    const bool over_array = tele == CSAW_TELEPORT_NONE && kind != CSAW_BIAS_NODE2VEC && (cached || build);
+    // a static bias: over the graph's kept array, or one built for this call
+    // into a stream-ordered temporary (build_cdf, or because the call is large
+    // enough that it pays); otherwise the rows are streamed
+    const bool kept = cached_cdf_usable(g, kind);
+    const bool build = !kept && tele == CSAW_TELEPORT_NONE && opts && opts->build_cdf && cdf_kind_positive(g, kind);
+    const bool pays = !kept && !build && kind != CSAW_BIAS_NODE2VEC && pack_fits(g, kind) &&
+                      walk_array_pays(g, kind, n_walkers, length);
+    WalkArray arr;
+    arr.tele = tele;
+    arr.tele_q32 = tele != CSAW_TELEPORT_NONE ? opts->teleport_q32 : 0u;
+    void* tmp = nullptr;
+    bool over_array = kind != CSAW_BIAS_NODE2VEC && (kept || build || pays);
+    if (over_array && kept && kind != CSAW_BIAS_UNIFORM) {
+        if (g->pack[kind]) {
+            arr.mode = WC_PACK;
+            arr.k = pack_view(g->pack[kind], g->E, g->V);
+        } else if (tele == CSAW_TELEPORT_NONE) {
+            arr.mode = WC_LEAF;
+            arr.c = cdf_view(g->cdf[kind], g->E, g->V);
+        } else {
+            over_array = false;
+        }
+    } else if (over_array && kind != CSAW_BIAS_UNIFORM) {
+        if (pack_fits(g, kind)) {
+            csaw_status st = dalloc(&tmp, sizeof(uint64_t) * pack_layout(g->E, g->V).words, s);
+            if (st != CSAW_OK && st != CSAW_ERR_NOMEM) return st;
+            if (st == CSAW_OK) {
+                arr.mode = WC_PACK;
+                arr.k = pack_view((const uint64_t*)tmp, g->E, g->V);
+            }
+            clear_error();
+        }
+        if (!tmp && build) {
+            // edge weights keep only the summaries and records (the leaf level
+            // is formed from the weights); neighbour degree the whole array
+            const bool leaf = kind != CSAW_BIAS_EDGE_WEIGHT;
+            CSAW_TRY(dalloc(&tmp, sizeof(uint64_t) * (leaf ? cdf_words(g->E, g->V) : wsum_layout(g->E, g->V).words), s));
+            arr.mode = leaf ? WC_LEAF : WC_WEIGHTS;
+            arr.c = leaf ? cdf_view((const uint64_t*)tmp, g->E, g->V) : wsum_view((const uint64_t*)tmp, g->E, g->V);
+        }
+        if (!tmp) over_array = false;   // no room: the rows are streamed
+    }
     if (mem_kind == CSAW_MEM_HOST) {
         // (over the array, the host starts are checked while the walk runs:
         // the kernels stop a walker whose start is not a vertex)
@@ -996,44 +1048,50 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
                             (unsigned long long)starts[i], (unsigned long long)i);
         void* a = nullptr;
         void* b = nullptr;
-        CSAW_TRY(dalloc(&a, sizeof(uint32_t) * n_walkers, s));
-        csaw_status st = dalloc(&b, path_bytes, s);
-        if (st != CSAW_OK) { dfree(a, s); return st; }
+        csaw_status st = dalloc(&a, sizeof(uint32_t) * n_walkers, s);
+        if (st == CSAW_OK) st = dalloc(&b, path_bytes, s);
+        if (st == CSAW_ERR_NOMEM && tmp && !build) {
+            // the buffers do not fit beside an array that was not asked for
+            dfree(tmp, s);
+            tmp = nullptr;
+            over_array = false;
+            for (uint64_t i = 0; i < n_walkers; ++i)
+                if (starts[i] >= g->V) {
+                    dfree(a, s);
+                    return fail(CSAW_ERR_INVALID, "start %llu of walker %llu out of range",
+                                (unsigned long long)starts[i], (unsigned long long)i);
+                }
+            st = a ? CSAW_OK : dalloc(&a, sizeof(uint32_t) * n_walkers, s);
+            if (st == CSAW_OK) st = dalloc(&b, path_bytes, s);
+        }
+        if (st != CSAW_OK) { dfree(a, s); dfree(tmp, s); return st; }
         d_starts = (const uint32_t*)a;
         d_path = (uint32_t*)b;
         cudaError_t e = cudaMemcpyAsync(a, starts, sizeof(uint32_t) * n_walkers,
                                         cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) { dfree(a, s); dfree(b, s); return cuda_fail(e, "copy starts"); }
+        if (e != cudaSuccess) { dfree(a, s); dfree(b, s); dfree(tmp, s); return cuda_fail(e, "copy starts"); }
     }
     PhaseTimer timer(opts ? opts->phase_ms : nullptr, s);
     if (over_array) {
-        const uint64_t* cdf = kind == CSAW_BIAS_UNIFORM ? nullptr : g->cdf[kind];
-        void* tmp = nullptr;
         csaw_status st = CSAW_OK;
-        // built for the call: edge weights keep only the summaries and
-        // records (the leaf level is formed from the weights); neighbour
-        // degree keeps the whole array (its biases are gathers)
-        const bool leaf = !(build && kind == CSAW_BIAS_EDGE_WEIGHT);
-        if (build) {
-            const uint64_t words = leaf ? cdf_words(g->E, g->V) : wsum_layout(g->E, g->V).words;
-            st = dalloc(&tmp, sizeof(uint64_t) * words, s);
-            if (st == CSAW_OK && leaf) st = enqueue_cdf_build(g, kind, (uint64_t*)tmp, s);
-            if (st == CSAW_OK && !leaf) {
-                const CdfView c = wsum_view((const uint64_t*)tmp, g->E, g->V);
-                st = enqueue_cdf_build_raw(g->off, g->col, g->w, g->deg, g->V, g->E, g->sm_count, kind, nullptr,
-                                           (uint64_t*)c.s1, (uint64_t*)c.s2, (uint64_t*)c.rec, s);
-            }
-            cdf = (const uint64_t*)tmp;
+        // (an array that was not asked for counts with the walk)
+        if (!build) timer.mark(1, s);
+        if (tmp && arr.mode == WC_PACK) {
+            st = enqueue_pack_build(g, kind, (uint64_t*)tmp, s);
+        } else if (tmp) {
+            const CdfView& c = arr.c;
+            st = enqueue_cdf_build_raw(g->off, g->col, g->w, g->deg, g->V, g->E, g->sm_count, kind, (uint64_t*)c.cdf,
+                                       (uint64_t*)c.s1, (uint64_t*)c.s2, (uint64_t*)c.rec, s);
         }
-        timer.mark(1, s);
+        if (build) timer.mark(1, s);
         // thread per walker; host paths come back chunk by chunk while the
         // next chunk walks
         if (st == CSAW_OK) {
             if (mem_kind == CSAW_MEM_HOST) {
-                st = walk_cached_to_host(g, kind, cdf, leaf, starts, d_starts, n_walkers, length, rng_seed, d_path,
-                                         path, s, timer.out && timer.ok ? timer.ev[2] : nullptr);
+                st = walk_cached_to_host(g, arr, starts, d_starts, n_walkers, length, rng_seed, d_path, path, s,
+                                         timer.out && timer.ok ? timer.ev[2] : nullptr);
             } else {
-                st = launch_walk_cached(g, kind, cdf, leaf, d_starts, 0, n_walkers, length, rng_seed, d_path, s);
+                st = launch_walk_cached(g, arr, d_starts, 0, n_walkers, length, rng_seed, d_path, s);
                 timer.mark(2, s);
             }
         }

@@ -28,20 +28,26 @@ namespace csaw {
 // sectors, the picked columns and the path rows are touched once.  Those are
 // read and written evict-first (ld/st .cs) so that they pass through L2
 // without pushing the summaries out.
+//
+// Over the packed array (WC_PACK) the walk of RMAT s20 (1 M walkers x 80
+// steps) takes 1.46 ms and its construction 0.11, against 2.88 and 0.15 over
+// summaries and weights: 133 DRAM bytes a step instead of 276 (a missing
+// sector is fetched as 64 bytes, so what one pick needs lies in one such
+// line), four dependent loads instead of ten.  Bound by their latency (DRAM
+// 4.5 TB/s, L2 65 % busy) at six blocks per SM; seven spill (1.90 ms), five
+// are even.
 constexpr int WC_THREADS = 256;
 constexpr int WC_WARPS = WC_THREADS / 32;
 constexpr int WC_TILE = 16;                  // path entries staged per walker
-
-// How a step finds its pick: uniform (x itself), the array's leaf level, or
-// the summaries and the weights (w_search, no leaf level).
-constexpr int WC_UNIFORM = 0, WC_LEAF = 1, WC_WEIGHTS = 2;
 
 struct WalkCdfParams {
     const uint64_t* __restrict__ off;
     const uint32_t* __restrict__ col;
     const uint32_t* __restrict__ w;      // weights (WC_WEIGHTS)
     uint64_t E;
-    CdfView c;                           // the cumulative array (cdf null for uniform bias)
+    CdfView c;                           // the cumulative array (WC_LEAF, WC_WEIGHTS)
+    PackView k;                          // the packed array (WC_PACK)
+    uint32_t tele, tele_q32;             // teleporting kernels
     uint32_t V;
     const uint32_t* __restrict__ starts;
     uint64_t n;
@@ -102,9 +108,11 @@ __device__ __forceinline__ T ld_graph(const T* p)
 }
 
 // HOST: off, col and w are host arrays (unpadded), read in place.
-template <int MODE, bool BATCH = false, bool HOST = false>
+// TELE: restart or jump, as in walk_kernel.
+template <int MODE, bool BATCH = false, bool HOST = false, bool TELE = false>
 __global__ void __launch_bounds__(WC_THREADS, 6) walk_cached_kernel(WalkCdfParams p)
 {
+    static_assert(!TELE || (!BATCH && !HOST), "teleporting walks are not batched");
     __shared__ uint32_t s_tile[WC_WARPS][32][WC_TILE + 1];   // +1: conflict-free column writes
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t (*tile)[WC_TILE + 1] = s_tile[wid];
@@ -133,38 +141,56 @@ __global__ void __launch_bounds__(WC_THREADS, 6) walk_cached_kernel(WalkCdfParam
         for (uint32_t s = 0; s < L; ++s) {
             if constexpr (BATCH) alive = alive && s < ws.L;
             if (alive) {
-                // the row: offsets (uniform) or the vertex's record {start, end, total}
-                uint64_t beg, end, T = 0;
-                if constexpr (MODE == WC_UNIFORM) {
-                    beg = ld_graph<HOST>(p.off + cur);
-                    end = ld_graph<HOST>(p.off + cur + 1);
-                } else {
-                    const ulonglong2* rc = reinterpret_cast<const ulonglong2*>(p.c.rec + 4ull * cur);
-                    const ulonglong2 r0 = __ldg(rc), r1 = __ldg(rc + 1);
-                    beg = r0.x;
-                    end = r0.y;
-                    T = r1.x;
-                }
-                bool stop = beg == end;
-                uint64_t i = 0;
-                if (!stop) {
+                const uint32_t id = p.w0 + (uint32_t)wk;
+                bool jump = false;
+                if constexpr (TELE) jump = (uint32_t)(philox_draw(p.keys, 1u, cur, s, id) >> 32) < p.tele_q32;
+                bool stop = false;
+                uint32_t nxt = CSAW_NONE;
+                if (!jump) {
                     uint64_t r;
                     if constexpr (BATCH) r = philox_draw(ws.k0, ws.k1, 0u, cur, s, ws.id);
-                    else r = philox_draw(p.keys, 0u, cur, s, p.w0 + (uint32_t)wk);
-                    if constexpr (MODE == WC_UNIFORM) {
-                        i = scale_draw(r, end - beg);
-                    } else {
+                    else r = philox_draw(p.keys, 0u, cur, s, id);
+                    if constexpr (MODE == WC_PACK) {
+                        const ulonglong2* rc = reinterpret_cast<const ulonglong2*>(p.k.rec) + cur;
+                        const ulonglong2 r0 = __ldg(rc), r1 = __ldg(rc + 1);
+                        const uint64_t T = r1.y - r0.y;
                         stop = T == 0;
+                        if (!stop) nxt = pack_pick(p.k, r0.x, r1.x, r, r0.y + scale_draw(r, T));
+                    } else {
+                        // the row: offsets (uniform) or the vertex's record {start, end, total}
+                        uint64_t beg, end, T = 0;
+                        if constexpr (MODE == WC_UNIFORM) {
+                            beg = ld_graph<HOST>(p.off + cur);
+                            end = ld_graph<HOST>(p.off + cur + 1);
+                            T = end - beg;
+                        } else {
+                            const ulonglong2* rc = reinterpret_cast<const ulonglong2*>(p.c.rec + 4ull * cur);
+                            const ulonglong2 r0 = __ldg(rc), r1 = __ldg(rc + 1);
+                            beg = r0.x;
+                            end = r0.y;
+                            T = r1.x;
+                        }
+                        stop = beg == end || T == 0;
                         if (!stop) {
                             const uint64_t x = scale_draw(r, T);
-                            if constexpr (MODE == WC_LEAF) i = cdf_search<true>(p.c, beg, end, x) - beg;
+                            uint64_t i;
+                            if constexpr (MODE == WC_UNIFORM) i = x;
+                            else if constexpr (MODE == WC_LEAF) i = cdf_search<true>(p.c, beg, end, x) - beg;
                             else i = w_search<!HOST>(p.c, p.w, p.E, beg, end, x) - beg;
+                            if constexpr (HOST) nxt = p.col[beg + i];
+                            else nxt = __ldcs(p.col + beg + i);
                         }
                     }
                 }
-                if (stop) { alive = false; cur = CSAW_NONE; }
-                else if constexpr (HOST) cur = p.col[beg + i];
-                else cur = __ldcs(p.col + beg + i);
+                if constexpr (TELE) {
+                    if (jump || stop)
+                        nxt = p.tele == CSAW_TELEPORT_RESTART
+                                  ? __ldg(p.starts + wk)
+                                  : (uint32_t)scale_draw(philox_draw(p.keys, 2u, cur, s, id), p.V);
+                } else if (stop) {
+                    alive = false;
+                }
+                cur = nxt;
             }
             const uint64_t t = (uint64_t)s + 1;      // path position of this step's vertex
             tile[lane][t - t0] = cur;
@@ -182,13 +208,13 @@ __global__ void __launch_bounds__(WC_THREADS, 6) walk_cached_kernel(WalkCdfParam
 }
 
 // Resident blocks per SM of one instantiation (queried once).
-template <int MODE, bool BATCH, bool HOST>
+template <int MODE, bool BATCH, bool HOST, bool TELE>
 static csaw_status walk_cached_occupancy(int* per_sm_out)
 {
     static std::atomic<int> cached{0};
     int per_sm = cached.load(std::memory_order_acquire);
     if (per_sm == 0) {
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_cached_kernel<MODE, BATCH, HOST>,
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_cached_kernel<MODE, BATCH, HOST, TELE>,
                                                                       WC_THREADS, 0);
         if (e != cudaSuccess) return cuda_fail(e, "occupancy(walk_cached)");
         if (per_sm < 1) per_sm = 1;
@@ -198,11 +224,11 @@ static csaw_status walk_cached_occupancy(int* per_sm_out)
     return CSAW_OK;
 }
 
-template <int MODE, bool BATCH, bool HOST = false>
+template <int MODE, bool BATCH, bool HOST = false, bool TELE = false>
 static csaw_status launch_walk_cached_k(const WalkCdfParams& p, int sm_count, cudaStream_t s)
 {
     int per_sm = 0;
-    CSAW_TRY((walk_cached_occupancy<MODE, BATCH, HOST>(&per_sm)));
+    CSAW_TRY((walk_cached_occupancy<MODE, BATCH, HOST, TELE>(&per_sm)));
     uint64_t blocks = (p.n + WC_THREADS - 1) / WC_THREADS;
     uint64_t cap = (uint64_t)sm_count * per_sm;
     if (BATCH && p.seg.warp_budget) {
@@ -212,27 +238,33 @@ static csaw_status launch_walk_cached_k(const WalkCdfParams& p, int sm_count, cu
     }
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    walk_cached_kernel<MODE, BATCH, HOST><<<(unsigned)blocks, WC_THREADS, 0, s>>>(p);
+    walk_cached_kernel<MODE, BATCH, HOST, TELE><<<(unsigned)blocks, WC_THREADS, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "walk_cached_kernel launch");
     return CSAW_OK;
 }
 
-csaw_status launch_walk_cached(const csaw_graph* g, int kind, const uint64_t* cdf, bool leaf,
-                               const uint32_t* starts, uint64_t w0, uint64_t n, uint32_t length, uint64_t rng_seed,
-                               uint32_t* path, cudaStream_t s)
+csaw_status launch_walk_cached(const csaw_graph* g, const WalkArray& arr, const uint32_t* starts, uint64_t w0,
+                               uint64_t n, uint32_t length, uint64_t rng_seed, uint32_t* path, cudaStream_t s)
 {
     WalkCdfParams p;
     p.off = g->off; p.col = g->col; p.w = g->w; p.E = g->E;
-    const uint64_t* base = kind == CSAW_BIAS_UNIFORM ? nullptr : cdf;
-    p.c = leaf ? cdf_view(base, g->E, g->V) : wsum_view(base, g->E, g->V);
+    p.c = arr.c; p.k = arr.k;
+    p.tele = arr.tele; p.tele_q32 = arr.tele_q32;
     p.V = g->V; p.starts = starts; p.n = n; p.L = length; p.path = path;
     p.w0 = (uint32_t)w0;
     p.keys = philox_round_keys(rng_seed);
     p.seg = WalkSegments{};
-    if (kind == CSAW_BIAS_UNIFORM) return launch_walk_cached_k<WC_UNIFORM, false>(p, g->sm_count, s);
-    if (!leaf) return launch_walk_cached_k<WC_WEIGHTS, false>(p, g->sm_count, s);
-    return launch_walk_cached_k<WC_LEAF, false>(p, g->sm_count, s);
+    switch (arr.mode) {
+    case WC_UNIFORM:
+        return arr.tele ? launch_walk_cached_k<WC_UNIFORM, false, false, true>(p, g->sm_count, s)
+                        : launch_walk_cached_k<WC_UNIFORM, false>(p, g->sm_count, s);
+    case WC_PACK:
+        return arr.tele ? launch_walk_cached_k<WC_PACK, false, false, true>(p, g->sm_count, s)
+                        : launch_walk_cached_k<WC_PACK, false>(p, g->sm_count, s);
+    case WC_WEIGHTS: return launch_walk_cached_k<WC_WEIGHTS, false>(p, g->sm_count, s);
+    default: return launch_walk_cached_k<WC_LEAF, false>(p, g->sm_count, s);
+    }
 }
 
 csaw_status launch_walk_host(const CdfView& c, const uint64_t* off, const uint32_t* col, const uint32_t* w,
@@ -241,7 +273,8 @@ csaw_status launch_walk_host(const CdfView& c, const uint64_t* off, const uint32
 {
     WalkCdfParams p;
     p.off = off; p.col = col; p.w = w; p.E = E;
-    p.c = c;
+    p.c = c; p.k = PackView{};
+    p.tele = p.tele_q32 = 0;
     p.V = V; p.starts = starts; p.n = n; p.L = length; p.path = path;
     p.w0 = 0;
     p.keys = philox_round_keys(rng_seed);
@@ -258,16 +291,18 @@ csaw_status launch_walk_host(const CdfView& c, const uint64_t* off, const uint32
 // copy is left after the walk.
 constexpr uint64_t WC_MAX_CHUNKS = 64;
 
-csaw_status walk_cached_to_host(const csaw_graph* g, int kind, const uint64_t* cdf, bool leaf,
-                                const uint32_t* h_starts, const uint32_t* d_starts, uint64_t n, uint32_t length,
-                                uint64_t rng_seed, uint32_t* d_path, uint32_t* h_path, cudaStream_t s,
-                                cudaEvent_t walked)
+csaw_status walk_cached_to_host(const csaw_graph* g, const WalkArray& arr, const uint32_t* h_starts,
+                                const uint32_t* d_starts, uint64_t n, uint32_t length, uint64_t rng_seed,
+                                uint32_t* d_path, uint32_t* h_path, cudaStream_t s, cudaEvent_t walked)
 {
     const uint64_t row_len = (uint64_t)length + 1;
     int per_sm = 0;
-    if (kind == CSAW_BIAS_UNIFORM) CSAW_TRY((walk_cached_occupancy<WC_UNIFORM, false, false>(&per_sm)));
-    else if (!leaf) CSAW_TRY((walk_cached_occupancy<WC_WEIGHTS, false, false>(&per_sm)));
-    else CSAW_TRY((walk_cached_occupancy<WC_LEAF, false, false>(&per_sm)));
+    if (arr.mode == WC_UNIFORM && arr.tele) CSAW_TRY((walk_cached_occupancy<WC_UNIFORM, false, false, true>(&per_sm)));
+    else if (arr.mode == WC_UNIFORM) CSAW_TRY((walk_cached_occupancy<WC_UNIFORM, false, false, false>(&per_sm)));
+    else if (arr.mode == WC_PACK && arr.tele) CSAW_TRY((walk_cached_occupancy<WC_PACK, false, false, true>(&per_sm)));
+    else if (arr.mode == WC_PACK) CSAW_TRY((walk_cached_occupancy<WC_PACK, false, false, false>(&per_sm)));
+    else if (arr.mode == WC_WEIGHTS) CSAW_TRY((walk_cached_occupancy<WC_WEIGHTS, false, false, false>(&per_sm)));
+    else CSAW_TRY((walk_cached_occupancy<WC_LEAF, false, false, false>(&per_sm)));
     const uint64_t wave = (uint64_t)g->sm_count * (uint64_t)per_sm * WC_THREADS;
     const uint64_t waves = (n + wave - 1) / wave;
     const uint64_t per_chunk = (waves + WC_MAX_CHUNKS - 1) / WC_MAX_CHUNKS;
@@ -283,7 +318,7 @@ csaw_status walk_cached_to_host(const csaw_graph* g, int kind, const uint64_t* c
     // every chunk's walk first (the copies of pageable memory block the host)
     for (uint64_t c = 0, w0 = 0; st == CSAW_OK && w0 < n; w0 += chunk, ++c) {
         const uint64_t m = n - w0 < chunk ? n - w0 : chunk;
-        st = launch_walk_cached(g, kind, cdf, leaf, d_starts + w0, w0, m, length, rng_seed, d_path + w0 * row_len, s);
+        st = launch_walk_cached(g, arr, d_starts + w0, w0, m, length, rng_seed, d_path + w0 * row_len, s);
         if (st == CSAW_OK && k > 1) {
             e = cudaEventRecord(ev[c], s);
             if (e != cudaSuccess) st = cuda_fail(e, "chunk event");
@@ -325,13 +360,17 @@ csaw_status walk_batch_cached(const csaw_graph* g, int kind, const uint32_t* d_s
 {
     WalkCdfParams p;
     p.off = g->off; p.col = g->col; p.w = g->w; p.E = g->E;
-    p.c = cdf_view(kind == CSAW_BIAS_UNIFORM ? nullptr : g->cdf[kind], g->E, g->V);
+    const bool uniform = kind == CSAW_BIAS_UNIFORM;
+    p.c = cdf_view(uniform ? nullptr : g->cdf[kind], g->E, g->V);
+    p.k = pack_view(uniform ? nullptr : g->pack[kind], g->E, g->V);
+    p.tele = p.tele_q32 = 0;
     p.V = g->V; p.starts = d_starts; p.n = n; p.L = max_len; p.path = d_path;
     p.w0 = 0;
     p.keys = philox_round_keys(0);
     p.seg = seg;
-    return kind == CSAW_BIAS_UNIFORM ? launch_walk_cached_k<WC_UNIFORM, true>(p, g->sm_count, s)
-                                     : launch_walk_cached_k<WC_LEAF, true>(p, g->sm_count, s);
+    if (uniform) return launch_walk_cached_k<WC_UNIFORM, true>(p, g->sm_count, s);
+    return p.k.pack ? launch_walk_cached_k<WC_PACK, true>(p, g->sm_count, s)
+                    : launch_walk_cached_k<WC_LEAF, true>(p, g->sm_count, s);
 }
 
 }  // namespace csaw
