@@ -610,18 +610,23 @@ __device__ __forceinline__ uint64_t w_search(const CdfView& c, const uint32_t* _
     return hit;
 }
 
-// The column of the smallest e in [beg, end) with P[e] > y in a packed array,
-// for y in [P[beg - 1], P[end - 1]).  P does not decrease over all edges, so
-// the search is over all blocks, started where the draw r would fall if the
-// row's biases were equal: four block ends are read at once (one sector, and
+// The smallest e in [beg, end) with P[e] > y in a packed array, for y in
+// [P[beg - 1], P[end - 1]): its column, its number, P before it and its bias.
+// P does not decrease over all edges, so the search is over all blocks,
+// started at edge `guess` (of the row), where the draw would fall if the row's
+// biases were equal: four block ends are read at once (one sector, and
 // the end before them), which holds the answer for most rows; otherwise a
 // galloping search goes on from there.  Then one sector of the block's group
 // sums and the group's biases and columns: four dependent loads a step, with
 // the record, against ten or so for the bisected summaries (cdf_group), and
 // one 64-byte line per pick where weights and column were two.
-__device__ __forceinline__ uint32_t pack_pick(const PackView& k, uint64_t beg, uint64_t end, uint64_t r, uint64_t y)
+struct PackHit {
+    uint32_t col, bias;
+    uint64_t e, low;
+};
+__device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, uint64_t end, uint64_t guess, uint64_t y)
 {
-    uint64_t at = (beg + __umul64hi(r, end - beg)) >> 8;   // 256-edge window
+    uint64_t at = guess >> 8;   // 256-edge window
     uint64_t v[4];
     ld256(k.s2 + 4 * at, v);
     uint64_t before = at ? __ldg(k.s2 + 4 * at - 1) : 0ull;
@@ -676,13 +681,20 @@ __device__ __forceinline__ uint32_t pack_pick(const PackView& k, uint64_t beg, u
     uint32_t b[8], c[8];
     ld256_stream(k.pack + 16 * g, b);
     ld256_stream(k.pack + 16 * g + 8, c);
-    uint32_t sum = 0, pick = c[0];
+    uint32_t sum = 0, low = 0;
+    PackHit hit{c[0], b[0], 8 * g, 0};
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
         sum += b[j];
-        if (sum <= x) pick = c[j + 1];
+        if (sum <= x) {
+            hit.col = c[j + 1];
+            hit.bias = b[j + 1];
+            hit.e = 8 * g + j + 1;
+            low = sum;
+        }
     }
-    return pick;
+    hit.low = before + sub + low;
+    return hit;
 }
 
 }  // namespace csaw

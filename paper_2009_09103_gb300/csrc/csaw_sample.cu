@@ -30,6 +30,7 @@
 // the same choice as searching a recomputed prefix sum.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -1210,8 +1211,11 @@ struct LayerSelParams {
     uint64_t* p_eid;                     // select: [edges] edge index of each pick
     uint64_t* p_start;                   // select: [edges] pool prefix before each pick
     uint32_t* p_bias;                    // select: [edges] bias of each pick
-    uint64_t* ctb;                       // select: [frontier] chunk table base of each entry (~0: none)
+    uint64_t* ctb;                       // select: [frontier] chunk table base of each entry (~0: none);
+                                         // layer_draw_kernel: prefix of the entries' degrees
     uint64_t* ct;                        // select: [warps][LAYER_CT_CAP] chunk prefix tables
+    PackView pk;                         // layer_draw_kernel: the packed array (null: uniform)
+    uint32_t table;                      // layer_draw_kernel: slots of its hash table (a power of two)
 };
 
 // Rows longer than LAYER_CHUNK keep the running sum at the end of every
@@ -1256,18 +1260,21 @@ __global__ void __launch_bounds__(SEL_THREADS) layer_count_kernel(LayerSelParams
     for (uint64_t i = gw; i < P.n_inst; i += nw) {
         const uint64_t a = P.FO[i], b = P.FO[i + 1];
         uint64_t npos = 0;
-        for (uint64_t e = a; e < b; ++e) {
+        if (!p.zero_bias) {
+            for (uint64_t e = a + lane; e < b; e += 32) {
+                const uint32_t v = (uint32_t)(p.fkeys[e] & p.vmask);
+                npos += __ldg(p.off + v + 1) - __ldg(p.off + v);
+            }
+            npos = warp_sum_u64(npos);
+        }
+        for (uint64_t e = a; p.zero_bias && e < b; ++e) {
             const uint32_t v = (uint32_t)(p.fkeys[e] & p.vmask);
             const uint64_t beg = __ldg(p.off + v);
             const uint32_t d = (uint32_t)(__ldg(p.off + v + 1) - beg);
-            if (!p.zero_bias) {
-                npos += d;
-            } else {
-                uint64_t t;
-                uint32_t c;
-                layer_row_total<KIND>(p, beg, d, lane, &t, &c);
-                npos += c;
-            }
+            uint64_t t;
+            uint32_t c;
+            layer_row_total<KIND>(p, beg, d, lane, &t, &c);
+            npos += c;
         }
         for (uint64_t e = a + lane; e < b; e += 32)
             P.cnt[e] = e == a ? (uint32_t)(npos < p.k ? npos : p.k) : 0u;
@@ -1447,6 +1454,302 @@ __global__ void __launch_bounds__(SEL_THREADS) layer_select_kernel(LayerSelParam
                 __syncwarp();
             }
         }
+    }
+}
+
+// The same selection over the packed array (or uniform biases), every bias
+// positive: one block per instance.  Row totals are two records apart instead
+// of a pass over each row, and a round takes LD_THREADS attempts at once, a
+// thread each: the entry by bisection of the totals' prefix, the edge by
+// pack_pick.  Attempts of one edge meet in a shared hash table that keeps the
+// lowest attempt, so that an attempt is a new pick when it is still its
+// edge's lowest after the round; new picks are taken in attempt order.  What
+// attempt_cap leaves is drawn by updated sampling.
+// RMAT s20, 2000 instances, 512 picks of frontiers of 64 and about 500
+// vertices: 0.089 + 0.071 ms for the two layers (latency of the searches, a
+// few rounds a block) and 0.11 for the array, against 10.8 ms a warp per
+// instance, which streams 2.2 G pool edges; with updated sampling left to one
+// warp's passes over its picks the first layer, whose pools are often little
+// more than the picks, took 2.36 ms.
+constexpr int LD_THREADS = 256;
+constexpr uint32_t LD_MAX_K = 2048;     // picks per instance and layer the table is sized for
+constexpr uint32_t LD_MIN_CAP = 64;     // attempt caps below this leave most picks to updated sampling
+constexpr uint32_t LD_VP = 1024;        // prefix entries kept in shared memory
+
+static uint32_t layer_table_slots(uint32_t k)
+{
+    uint32_t t = 1024;
+    while (t < 2 * (k + LD_THREADS)) t *= 2;
+    return t;
+}
+
+template <bool UNIFORM>
+__global__ void __launch_bounds__(LD_THREADS) layer_draw_kernel(LayerSelParams P)
+{
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    unsigned long long* t_key = (unsigned long long*)s_dyn;   // edge + 1 (0: free)
+    uint32_t* t_att = (uint32_t*)(t_key + P.table);           // its lowest attempt
+    __shared__ uint64_t s_vp[LD_VP];
+    __shared__ uint64_t s_warp[LD_THREADS / 32];
+    __shared__ uint32_t s_cnt[LD_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    SelParams p = P.s;
+    if (p.key_dev) {
+        p.k0 = p.key_dev[0];
+        p.k1 = p.key_dev[1];
+    }
+    const uint32_t inst = blockIdx.x;
+    const uint64_t a = P.FO[inst], b = P.FO[inst + 1];
+    if (a == b) return;
+    const uint64_t q0 = p.pos[a];
+    const uint32_t k = (uint32_t)(p.pos[a + 1] - q0);
+    if (k == 0) return;
+    const ulonglong2* rec = reinterpret_cast<const ulonglong2*>(P.pk.rec);
+    // row start, end and total of vertex v; *low: P before the row
+    const auto row = [&](uint32_t v, uint64_t* beg, uint64_t* end, uint64_t* low) -> uint64_t {
+        if constexpr (UNIFORM) {
+            *beg = __ldg(p.off + v);
+            *end = __ldg(p.off + v + 1);
+            *low = 0;
+            return *end - *beg;
+        } else {
+            const ulonglong2 r0 = __ldg(rec + v), r1 = __ldg(rec + v + 1);
+            *beg = r0.x;
+            *end = r1.x;
+            *low = r0.y;
+            return r1.y - r0.y;
+        }
+    };
+    // inclusive prefix of the entries' totals; edges of the pool
+    const bool near = b - a <= LD_VP;
+    uint64_t* vp = near ? s_vp : P.VP + a;
+    uint64_t T = 0, pool = 0;
+    for (uint64_t e0 = a; e0 < b; e0 += LD_THREADS) {
+        const uint64_t e = e0 + tid;
+        uint64_t t = 0, d = 0;
+        if (e < b) {
+            uint64_t beg, end, low;
+            t = row((uint32_t)(p.fkeys[e] & p.vmask), &beg, &end, &low);
+            d = end - beg;
+        }
+        pool += d;
+        const uint64_t incl = warp_inclusive_scan_u64(t, lane);
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        uint64_t before = T;
+        for (int w = 0; w < LD_THREADS / 32; ++w) {
+            if (w < wid) before += s_warp[w];
+            T += s_warp[w];
+        }
+        if (e < b) vp[e - a] = before + incl;
+        __syncthreads();
+    }
+    pool = warp_sum_u64(pool);
+    if (lane == 0) s_warp[wid] = pool;
+    for (uint32_t i = tid; i < P.table; i += LD_THREADS) {
+        t_key[i] = 0ull;
+        t_att[i] = 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    pool = 0;
+    for (int w = 0; w < LD_THREADS / 32; ++w) pool += s_warp[w];
+    if (pool <= p.k) {
+        // every entry, pool order
+        uint64_t q = q0;
+        for (uint64_t e = a; e < b; ++e) {
+            const uint32_t v = (uint32_t)(p.fkeys[e] & p.vmask);
+            const uint64_t beg = __ldg(p.off + v);
+            const uint32_t d = (uint32_t)(__ldg(p.off + v + 1) - beg);
+            for (uint32_t j = tid; j < d; j += LD_THREADS) emit(p, q + j, v, inst, __ldg(p.col + beg + j));
+            q += d;
+        }
+        return;
+    }
+    // the pool entry that holds x: first with vp > x
+    const auto entry = [&](uint64_t x) -> uint64_t {
+        uint64_t lo = 0, hi = b - a;
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if (vp[mid] > x) hi = mid; else lo = mid + 1;
+        }
+        return lo;
+    };
+    const auto pick = [&](uint64_t x, uint32_t* v) -> PackHit {
+        const uint64_t i = entry(x);
+        const uint64_t before = i ? vp[i - 1] : 0ull;
+        *v = (uint32_t)(p.fkeys[a + i] & p.vmask);
+        uint64_t beg, end, low;
+        const uint64_t t = row(*v, &beg, &end, &low);
+        const uint64_t xr = x - before;
+        PackHit h;
+        if constexpr (UNIFORM) {
+            h = PackHit{__ldg(p.col + beg + xr), 1u, beg + xr, x};
+        } else {
+            const uint64_t d = end - beg;
+            const uint64_t at = (uint64_t)((float)d * __fdividef((float)xr, (float)t));
+            h = pack_pick(P.pk, beg, end, beg + (at < d ? at : d - 1), low + xr);
+            h.low = h.low - low + before;   // in the pool's prefix sums
+        }
+        return h;
+    };
+    uint32_t have = 0;
+    for (uint32_t a0 = 0; have < k && a0 < p.attempt_cap; a0 += LD_THREADS) {
+        const uint32_t at = a0 + tid;
+        const bool live = at < p.attempt_cap;
+        uint32_t v = 0, slot = 0;
+        PackHit h{};
+        if (live) {
+            h = pick(scale_draw(philox_draw(p.k0, p.k1, at, CSAW_NONE, p.layer, inst), T), &v);
+            const unsigned long long key = h.e + 1;
+            slot = (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 32) & (P.table - 1);
+            while (true) {
+                const unsigned long long was = atomicCAS(t_key + slot, 0ull, key);
+                if (was == 0ull || was == key) break;
+                slot = (slot + 1) & (P.table - 1);
+            }
+            atomicMin(t_att + slot, at);
+        }
+        __syncthreads();
+        const bool fresh = live && t_att[slot] == at;
+        const uint32_t bal = __ballot_sync(CSAW_FULL_MASK, fresh);
+        if (lane == 0) s_cnt[wid] = __popc(bal);
+        __syncthreads();
+        uint32_t rank = have + __popc(bal & lanemask_lt()), total = 0;
+        for (int w = 0; w < LD_THREADS / 32; ++w) {
+            if (w < wid) rank += s_cnt[w];
+            total += s_cnt[w];
+        }
+        if (fresh && rank < k) {
+            P.p_eid[q0 + rank] = h.e;
+            P.p_start[q0 + rank] = h.low;
+            P.p_bias[q0 + rank] = h.bias;
+            emit(p, q0 + rank, v, inst, h.col);
+        }
+        have = min(have + total, k);
+        __syncthreads();   // the counts are read before the next round's
+    }
+    if (have == k) return;
+    // Updated sampling for the rest.  A pool that fits the table's memory is
+    // laid out there as prefix sums of the unpicked biases: each thread holds
+    // a run of entries, relative to its start, so that taking a pick out
+    // changes one run and the later runs' starts, which are registers; a pick
+    // is then two barriers' worth of time instead of a chain of loads.
+    const uint32_t n = (uint32_t)min(pool, (uint64_t)0xFFFFFFFFu);
+    if (n <= 3 * P.table && T < (1ull << 32)) {
+        uint32_t* S = (uint32_t*)s_dyn;
+        uint64_t* dp = P.ctb + a;   // pool entries up to each frontier vertex
+        __shared__ uint32_t s_hit[2][3];
+        // degrees' prefix, then the biases at their places
+        uint64_t run = 0;
+        for (uint64_t e0 = a; e0 < b; e0 += LD_THREADS) {
+            const uint64_t e = e0 + tid;
+            uint64_t beg = 0, end = 0, low;
+            if (e < b) row((uint32_t)(p.fkeys[e] & p.vmask), &beg, &end, &low);
+            const uint64_t incl = warp_inclusive_scan_u64(end - beg, lane);
+            if (lane == 31) s_warp[wid] = incl;
+            __syncthreads();
+            uint64_t before = run;
+            for (int w = 0; w < LD_THREADS / 32; ++w) {
+                if (w < wid) before += s_warp[w];
+                run += s_warp[w];
+            }
+            if (e < b) dp[e - a] = before + incl;
+            __syncthreads();
+        }
+        for (uint64_t e = a + wid; e < b; e += LD_THREADS / 32) {
+            uint64_t beg, end, low;
+            row((uint32_t)(p.fkeys[e] & p.vmask), &beg, &end, &low);
+            const uint32_t first = (uint32_t)(e > a ? dp[e - a - 1] : 0ull);
+            for (uint64_t q = beg + lane; q < end; q += 32)
+                S[first + (uint32_t)(q - beg)] = UNIFORM ? 1u : P.pk.pack[16 * (q >> 3) + (q & 7)];
+        }
+        __syncthreads();
+        // the picked entries' biases to zero: an edge's place in the pool from
+        // its vertex's, found by its pool prefix
+        for (uint32_t t = tid; t < have; t += LD_THREADS) {
+            const uint64_t e = entry(P.p_start[q0 + t]);
+            uint64_t beg, end, low;
+            row((uint32_t)(p.fkeys[a + e] & p.vmask), &beg, &end, &low);
+            S[(uint32_t)(e ? dp[e - 1] : 0ull) + (uint32_t)(P.p_eid[q0 + t] - beg)] = 0u;
+        }
+        __syncthreads();
+        const uint32_t per = (n + LD_THREADS - 1) / LD_THREADS;
+        const uint32_t i0 = min(per * tid, n), i1 = min(i0 + per, n);
+        uint32_t len = 0;
+        for (uint32_t i = i0; i < i1; ++i) {
+            len += S[i];
+            S[i] = len;
+        }
+        const uint64_t incl = warp_inclusive_scan_u64(len, lane);
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        uint64_t start = incl - len, left = 0;   // the run's start; the unpicked total
+        for (int w = 0; w < LD_THREADS / 32; ++w) {
+            if (w < wid) start += s_warp[w];
+            left += s_warp[w];
+        }
+        const uint32_t have0 = have;
+        for (uint32_t at = p.attempt_cap; have < k; ++at, ++have) {
+            const uint64_t x = scale_draw(philox_draw(p.k0, p.k1, at, CSAW_NONE, p.layer, inst), left);
+            uint32_t* hit = s_hit[have & 1];
+            if (x >= start && x < start + len) {
+                const uint32_t y = (uint32_t)(x - start);
+                uint32_t lo = i0, hi = i1 - 1;   // first with S > y
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (S[mid] > y) hi = mid; else lo = mid + 1;
+                }
+                const uint32_t bias = S[lo] - (lo > i0 ? S[lo - 1] : 0u);
+                for (uint32_t i = lo; i < i1; ++i) S[i] -= bias;
+                len -= bias;
+                hit[0] = lo;
+                hit[1] = bias;
+                hit[2] = (uint32_t)tid;
+            }
+            __syncthreads();
+            left -= hit[1];
+            if ((uint32_t)tid > hit[2]) start -= hit[1];
+            if (tid == 0) P.p_eid[q0 + have] = hit[0];   // place in the pool
+        }
+        __syncthreads();
+        for (uint32_t t = have0 + tid; t < k; t += LD_THREADS) {
+            const uint64_t i = P.p_eid[q0 + t];
+            uint64_t lo = 0, hi = b - a;   // first vertex with dp > i
+            while (lo < hi) {
+                const uint64_t mid = (lo + hi) >> 1;
+                if (dp[mid] > i) hi = mid; else lo = mid + 1;
+            }
+            const uint32_t v = (uint32_t)(p.fkeys[a + lo] & p.vmask);
+            emit(p, q0 + t, v, inst, __ldg(p.col + __ldg(p.off + v) + (i - (lo ? dp[lo - 1] : 0ull))));
+        }
+        return;
+    }
+    if (wid != 0) return;
+    // a larger pool: the draw over the unpicked total, mapped past the picked
+    // intervals (fixpoint of y = x + picked biases starting at or below y)
+    uint64_t R = 0;
+    for (uint32_t t = lane; t < have; t += 32) R += P.p_bias[q0 + t];
+    R = warp_sum_u64(R);
+    for (uint32_t at = p.attempt_cap; have < k; ++at, ++have) {
+        const uint64_t x = scale_draw(philox_draw(p.k0, p.k1, at, CSAW_NONE, p.layer, inst), T - R);
+        uint64_t y = x;
+        while (true) {
+            uint64_t add = 0;
+            for (uint32_t t = lane; t < have; t += 32)
+                if (P.p_start[q0 + t] <= y) add += P.p_bias[q0 + t];
+            const uint64_t ny = x + warp_sum_u64(add);
+            if (ny == y) break;
+            y = ny;
+        }
+        uint32_t v;
+        const PackHit h = pick(y, &v);
+        if (lane == 0) {
+            P.p_start[q0 + have] = h.low;
+            P.p_bias[q0 + have] = h.bias;
+            emit(p, q0 + have, v, inst, h.col);
+        }
+        R += h.bias;
+        __syncwarp();
     }
 }
 
@@ -1908,10 +2211,39 @@ static csaw_status enqueue_layer_count(Pipeline& P, uint32_t l, cudaStream_t s)
     return scan_u32(B.cnt, B.pos, P.lc(l, L_N), B.f_cap, P.scan_scr, P.lc(l, L_TOTAL), s);
 }
 
+// Whether layer l is drawn by layer_draw_kernel: every bias positive, the
+// packed array (or uniform biases), picks that fit its table, and attempts
+// enough that few are left to updated sampling, which it does one warp per
+// block where layer_select_kernel runs a warp per instance.
+static bool layer_draws(const Pipeline& P, uint32_t l, const uint64_t* pack)
+{
+    return !P.zero_bias && P.fanout[l] <= LD_MAX_K && P.attempt_cap >= LD_MIN_CAP &&
+           (pack || P.kind == CSAW_BIAS_UNIFORM);
+}
+
+// Whether building the packed array for one layer-sampling call pays.  In ps:
+// layer_select_kernel's pass over the pool takes about 5 per edge with the
+// chip full and its picks about 2 us each in turn (512 picks from 500 rows);
+// the array takes 4 per edge of the graph (8 where degrees are gathered) and
+// 25 us.  Rows of later layers are reached by degree (see walk_array_pays).
+static bool layer_array_pays(const Pipeline& P, uint64_t n_seeds)
+{
+    const csaw_graph* g = P.g;
+    const double avg = (double)g->E / (double)g->V, visited = std::sqrt(avg * (double)g->max_degree);
+    double cost = 0, f = (double)n_seeds;
+    bool any = false;
+    for (uint32_t l = 0; l < P.depth; ++l) {
+        cost += 5.0 * f * (l ? visited : avg) + 2e6 * P.fanout[l];
+        f = (double)P.n_inst * P.fanout[l];
+        any |= P.fanout[l] <= LD_MAX_K;
+    }
+    return any && cost >= (P.kind == CSAW_BIAS_NEIGHBOR_DEGREE ? 8.0 : 4.0) * (double)g->E + 25e6;
+}
+
 // Layer l of layer sampling: the picks of every instance, then the offsets.
 static csaw_status enqueue_layer_select(Pipeline& P, uint32_t l, uint64_t* VP, uint64_t* p_eid,
                                         uint64_t* p_start, uint32_t* p_bias, uint64_t* ctb, uint64_t* ct,
-                                        cudaStream_t s)
+                                        const uint64_t* pack, cudaStream_t s)
 {
     csaw_graph* g = P.g;
     LayerBufs& B = P.L[l];
@@ -1919,7 +2251,18 @@ static csaw_status enqueue_layer_select(Pipeline& P, uint32_t l, uint64_t* VP, u
         LayerSelParams lp = layer_params(P, l);
         lp.VP = VP; lp.p_eid = p_eid; lp.p_start = p_start; lp.p_bias = p_bias;
         lp.ctb = ctb; lp.ct = ct;
-        switch (P.kind) {
+        if (layer_draws(P, l, pack)) {
+            const bool uniform = P.kind == CSAW_BIAS_UNIFORM;
+            lp.pk = pack_view(pack, g->E, g->V);
+            lp.table = layer_table_slots(P.fanout[l]);
+            const size_t smem = (size_t)lp.table * 12;
+            const void* fn = uniform ? (const void*)layer_draw_kernel<true> : (const void*)layer_draw_kernel<false>;
+            if (smem > 32768)   // beside the static arrays, past what a launch may take unasked
+                CSAW_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)layer_table_slots(LD_MAX_K) * 12));
+            if (uniform) layer_draw_kernel<true><<<P.n_inst, LD_THREADS, smem, s>>>(lp);
+            else layer_draw_kernel<false><<<P.n_inst, LD_THREADS, smem, s>>>(lp);
+        } else switch (P.kind) {
         case CSAW_BIAS_UNIFORM: layer_select_kernel<CSAW_BIAS_UNIFORM><<<layer_grid(P), SEL_THREADS, 0, s>>>(lp); break;
         case CSAW_BIAS_EDGE_WEIGHT: layer_select_kernel<CSAW_BIAS_EDGE_WEIGHT><<<layer_grid(P), SEL_THREADS, 0, s>>>(lp); break;
         default: layer_select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE><<<layer_grid(P), SEL_THREADS, 0, s>>>(lp); break;
@@ -1965,6 +2308,23 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
     R->dst.assign(depth, nullptr);
     R->layer_edges.assign(depth, 0);
     const bool hubs = (P.hub_path || P.hub_order) && !layer_mode;
+    // layer sampling: the graph's packed array, or one built for the call
+    const uint64_t* pack = nullptr;
+    if (layer_mode && P.kind != CSAW_BIAS_UNIFORM && !P.zero_bias && attempt_cap >= LD_MIN_CAP) {
+        pack = g->pack[P.kind];
+        if (!pack && pack_fits(g, P.kind) && layer_array_pays(P, n_seeds)) {
+            uint64_t* words = nullptr;
+            const csaw_status st = get((void**)&words, sizeof(uint64_t) * pack_layout(g->E, g->V).words);
+            if (st == CSAW_OK) {
+                CSAW_TRY(enqueue_pack_build(g, P.kind, words, s));
+                pack = words;
+            } else if (st != CSAW_ERR_NOMEM) {
+                return st;
+            } else {
+                clear_error();   // the rows are streamed
+            }
+        }
+    }
     for (uint32_t l = 0; l < depth; ++l) {
         // the layer's hub grouping buffers and shared hub prefix sums live
         // until its selection is done
@@ -2002,8 +2362,10 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
             CSAW_TRY(get((void**)&p_bias, sizeof(uint32_t) * e));
             uint64_t *ctb = nullptr, *ct = nullptr;
             CSAW_TRY(get((void**)&ctb, sizeof(uint64_t) * f));
-            CSAW_TRY(get((void**)&ct, sizeof(uint64_t) * LAYER_CT_CAP * (uint64_t)layer_grid(P) * SEL_WARPS));
-            CSAW_TRY(enqueue_layer_select(P, l, VP, p_eid, p_start, p_bias, ctb, ct, s));
+            if (!layer_draws(P, l, pack)) {
+                CSAW_TRY(get((void**)&ct, sizeof(uint64_t) * LAYER_CT_CAP * (uint64_t)layer_grid(P) * SEL_WARPS));
+            }
+            CSAW_TRY(enqueue_layer_select(P, l, VP, p_eid, p_start, p_bias, ctb, ct, pack, s));
         } else {
             CSAW_TRY(enqueue_select(P, l, s));
         }

@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(WC_THREADS, 6) walk_cached_kernel(WalkCdfParam
                         const ulonglong2 r0 = __ldg(rc), r1 = __ldg(rc + 1);
                         const uint64_t T = r1.y - r0.y;
                         stop = T == 0;
-                        if (!stop) nxt = pack_pick(p.k, r0.x, r1.x, r, r0.y + scale_draw(r, T));
+                        if (!stop)
+                            nxt = pack_pick(p.k, r0.x, r1.x, r0.x + __umul64hi(r, r1.x - r0.x), r0.y + scale_draw(r, T)).col;
                     } else {
                         // the row: offsets (uniform) or the vertex's record {start, end, total}
                         uint64_t beg, end, T = 0;
