@@ -238,10 +238,11 @@ __host__ __device__ inline CdfView cdf_view(const uint64_t* base, uint64_t E, ui
 //   s1[g]        P at the group's end less P at its 64-edge block's start, 32 bits
 //   s2[h]        P at the end of block h
 //   rec[v]       {off[v], P before off[v]}, v <= V
+//   sums[c]      scratch of the build, one word per chunk
 // Edges are padded with zero biases to whole chunks.
 constexpr uint64_t PACK_CHUNK = 8192;
 struct PackLayout {
-    uint64_t chunks, s1, s2, rec, words;   // word (8-byte) offsets and the total; pack at word 0
+    uint64_t chunks, s1, s2, rec, sums, words;   // word (8-byte) offsets and the total; pack at word 0
 };
 __host__ __device__ inline PackLayout pack_layout(uint64_t E, uint64_t V)
 {
@@ -250,7 +251,8 @@ __host__ __device__ inline PackLayout pack_layout(uint64_t E, uint64_t V)
     L.s1 = L.chunks * PACK_CHUNK;
     L.s2 = L.s1 + L.chunks * (PACK_CHUNK / 16);
     L.rec = L.s2 + L.chunks * (PACK_CHUNK / 64);
-    L.words = L.rec + 2 * (V + 1);
+    L.sums = L.rec + 2 * (V + 1);
+    L.words = L.sums + L.chunks;
     return L;
 }
 struct PackView {
@@ -273,8 +275,8 @@ __host__ __device__ inline PackView pack_view(const uint64_t* words, uint64_t E,
 // Whether the kind's biases fit the packed array: weights or degrees below
 // 2^26, so that a block's sums fit 32 bits.
 bool pack_fits(const csaw_graph* g, int kind);
-// Enqueues its build into pack_layout(E, V).words words on s.  Defined in
-// csaw_pack.cu.
+// Enqueues its build into pack_layout(E, V).words words on s (kernels alone,
+// so it can be captured).  Defined in csaw_pack.cu.
 csaw_status enqueue_pack_build(const csaw_graph* g, int kind, uint64_t* words, cudaStream_t s);
 
 // Walks that search an array of a static bias (or, for uniform bias, none):
@@ -695,6 +697,16 @@ __device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, ui
     }
     hit.low = before + sub + low;
     return hit;
+}
+
+// The sum of all biases before edge e in a packed array.
+__device__ __forceinline__ uint64_t pack_prefix(const PackView& k, uint64_t e)
+{
+    const uint64_t g = e >> 3;
+    uint64_t sum = g >= 8 ? __ldg(k.s2 + (g >> 3) - 1) : 0ull;
+    if (g & 7) sum += __ldg(k.s1 + g - 1);
+    for (uint32_t j = 0; j < (uint32_t)(e & 7); ++j) sum += __ldg(k.pack + 16 * g + j);
+    return sum;
 }
 
 }  // namespace csaw

@@ -135,9 +135,7 @@ csaw_status enqueue_pack_build(const csaw_graph* g, int kind, uint64_t* words, c
     uint32_t* s1 = (uint32_t*)(words + L.s1);
     uint64_t* s2 = words + L.s2;
     uint64_t* rec = words + L.rec;
-    void* sums = nullptr;
-    CSAW_TRY(dalloc(&sums, sizeof(uint64_t) * L.chunks, s));
-    uint64_t* cs = (uint64_t*)sums;
+    uint64_t* cs = words + L.sums;
     if (kind == CSAW_BIAS_EDGE_WEIGHT)
         pack_groups_kernel<CSAW_BIAS_EDGE_WEIGHT><<<(unsigned)L.chunks, PK_THREADS, 0, s>>>(g->col, g->w, g->deg, g->E,
                                                                                             pack, s1, s2, cs);
@@ -153,7 +151,6 @@ csaw_status enqueue_pack_build(const csaw_graph* g, int kind, uint64_t* words, c
     pack_ends_kernel<<<grid(blocks), 256, 0, s>>>(cs, blocks, s2);
     pack_rows_kernel<<<grid((uint64_t)g->V + 1), 256, 0, s>>>(g->off, g->V, pack, s1, s2, rec);
     const cudaError_t e = cudaGetLastError();
-    dfree(sums, s);
     return e == cudaSuccess ? CSAW_OK : cuda_fail(e, "packed array launch");
 }
 

@@ -35,6 +35,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "csaw_internal.cuh"
@@ -45,11 +46,16 @@ constexpr int SEL_THREADS = 256;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr uint32_t WARP_MAX_DEG = 256;     // warp items: degree <= this
 constexpr uint32_t CTA_SMEM_DEG = 8192;    // CTA items keep S in shared memory up to this
-constexpr uint32_t WARP_SLOT = WARP_MAX_DEG * 8 + (WARP_MAX_DEG / 32) * 4;   // bytes per warp
+// A warp item's prefix sums start at its row's 32-byte sector, so up to seven
+// places more than its neighbours; 32 bits each where they fit (NARROW).
+constexpr uint32_t WARP_SPAN = WARP_MAX_DEG + 8;
+constexpr uint32_t WARP_BITS = (WARP_SPAN + 31) / 32;
+constexpr uint32_t WARP_SLOT = (WARP_SPAN * 8 + WARP_BITS * 4 + 15) & ~15u;          // bytes per warp
+constexpr uint32_t WARP_SLOT_NARROW = (WARP_SPAN * 4 + WARP_BITS * 4 + 15) & ~15u;
 constexpr size_t SEL_DYN_SMEM = (size_t)CTA_SMEM_DEG * 8 + (CTA_SMEM_DEG / 32) * 4;
 // Warp items alone use only the warps' slots: a launch that can hold no CTA
 // item takes this much, and more blocks fit an SM.
-constexpr size_t SEL_WARP_SMEM = (size_t)(SEL_THREADS / 32) * WARP_SLOT;
+constexpr size_t sel_warp_smem(bool wide) { return (size_t)(SEL_THREADS / 32) * (wide ? WARP_SLOT : WARP_SLOT_NARROW); }
 constexpr uint32_t PICK_MAX = 256;         // picks a cached-array warp item may hold
 
 static_assert(SEL_WARPS * WARP_SLOT <= SEL_DYN_SMEM, "warp slots reuse the CTA region");
@@ -110,6 +116,7 @@ struct SelParams {
     const uint64_t* __restrict__ hubS = nullptr;
     uint64_t hubS_cap = 0;                // entries of hubS
     CdfView cv;                           // the cached array and its search aids (cv.cdf == cdf)
+    PackView pk;                          // the packed array, or none
     uint32_t* err = nullptr;              // error flags (8: a hub range beyond hubS_cap)
     // instances of several requests in one run (null: one request): per
     // instance its Philox key, its index within its request (the draw
@@ -141,7 +148,8 @@ __device__ __forceinline__ uint32_t sel_bias(const SelParams& p, uint64_t e)
 {
     if constexpr (KIND == CSAW_BIAS_UNIFORM) return 1u;
     else if constexpr (KIND == CSAW_BIAS_EDGE_WEIGHT) return __ldg(p.w + e);
-    else return __ldg(p.deg + __ldg(p.col + e));
+    // the packed array holds the degrees in edge order: no gather
+    else return p.pk.pack ? __ldg(p.pk.pack + 16 * (e >> 3) + (e & 7)) : __ldg(p.deg + __ldg(p.col + e));
 }
 
 __device__ __forceinline__ void emit(const SelParams& p, uint64_t q, uint32_t v, uint32_t inst, uint32_t u)
@@ -152,7 +160,8 @@ __device__ __forceinline__ void emit(const SelParams& p, uint64_t q, uint32_t v,
 }
 
 // Smallest i in [0, d) with S[i] > x (S inclusive prefix sums, x < S[d-1]).
-__device__ __forceinline__ uint32_t upper_bound_S(const uint64_t* S, uint32_t d, uint64_t x)
+template <class A>
+__device__ __forceinline__ uint32_t upper_bound_S(const A* S, uint32_t d, A x)
 {
     uint32_t lo = 0, hi = d;
     while (lo < hi) {
@@ -162,11 +171,18 @@ __device__ __forceinline__ uint32_t upper_bound_S(const uint64_t* S, uint32_t d,
     return lo;
 }
 
+// floor(r * T / 2^64) for a total of either width.
+__device__ __forceinline__ uint64_t scale_to(uint64_t r, uint64_t T) { return __umul64hi(r, T); }
+__device__ __forceinline__ uint32_t scale_to(uint64_t r, uint32_t T)
+{
+    return (uint32_t)(((r >> 32) * T + (((r & 0xFFFFFFFFull) * T) >> 32)) >> 32);
+}
+
 // Attempt rounds of one warp over a built prefix array S[0..d) with total T.
 // bits: d-bit chosen set, already cleared.  Emits picks at q0 + have.
-__device__ void draw_picks(const SelParams& p, const uint64_t* S, uint32_t* bits, uint32_t d,
-                           uint64_t T, uint32_t cnt, uint64_t q0, uint32_t v, uint32_t inst,
-                           uint64_t beg, int lane)
+template <class A>
+__device__ void draw_picks(const SelParams& p, const A* S, uint32_t* bits, uint32_t d, A T, uint32_t cnt,
+                           uint64_t q0, uint32_t v, uint32_t inst, uint64_t beg, int lane)
 {
     const DrawKey dk = draw_key(p, inst);
     const uint32_t lt = lanemask_lt();
@@ -178,7 +194,7 @@ __device__ void draw_picks(const SelParams& p, const uint64_t* S, uint32_t* bits
     while (have < cnt && a0 < p.attempt_cap) {
         const bool live = a0 + lane < p.attempt_cap;   // the last round may be partial
         const uint64_t r = philox_draw(dk.k0, dk.k1, a0 + lane, v, p.layer, dk.id);
-        const uint32_t i = live ? upper_bound_S(S, d, scale_draw(r, T)) : 0xFFFFFFFFu;
+        const uint32_t i = live ? upper_bound_S<A>(S, d, scale_to(r, T)) : 0xFFFFFFFFu;
         const bool chosen = live && ((bits[i >> 5] >> (i & 31)) & 1u);
         const uint32_t peers = __match_any_sync(CSAW_FULL_MASK, i);
         const bool fresh = live && !chosen && lane == __ffs(peers) - 1;
@@ -209,20 +225,20 @@ __device__ void draw_picks(const SelParams& p, const uint64_t* S, uint32_t* bits
     (void)have0;
     // Updated sampling for the remaining picks (attempts attempt_cap, ...).
     const uint32_t nwords = (d + 31) >> 5;
-    uint64_t R = 0;
+    A R = 0;
     for (uint32_t wi = lane; wi < nwords; wi += 32) {
         uint32_t m = bits[wi];
         while (m) {
             const uint32_t i = (wi << 5) + __ffs(m) - 1;
             m &= m - 1;
-            R += S[i] - (i ? S[i - 1] : 0);
+            R += S[i] - (i ? S[i - 1] : (A)0);
         }
     }
-    R = warp_sum_u64(R);
+    R = (A)warp_sum_u64(R);
     if (lane == 0) {
         for (uint32_t a = p.attempt_cap; have < cnt; ++a) {
             const uint64_t r = philox_draw(dk.k0, dk.k1, a, v, p.layer, dk.id);
-            uint64_t x = scale_draw(r, T - R);
+            A x = scale_to(r, (A)(T - R));
             // Walk the picked intervals in ascending order, skipping each one
             // that starts at or below the running position.
             bool done = false;
@@ -231,14 +247,14 @@ __device__ void draw_picks(const SelParams& p, const uint64_t* S, uint32_t* bits
                 while (m) {
                     const uint32_t i = (wi << 5) + __ffs(m) - 1;
                     m &= m - 1;
-                    const uint64_t start = i ? S[i - 1] : 0;
+                    const A start = i ? S[i - 1] : (A)0;
                     if (x >= start) x += S[i] - start;
                     else { done = true; break; }
                 }
             }
-            const uint32_t i = min(upper_bound_S(S, d, x), d - 1);   // x < T: always inside
+            const uint32_t i = min(upper_bound_S<A>(S, d, x), d - 1);   // x < T: always inside
             bits[i >> 5] |= 1u << (i & 31);
-            R += S[i] - (i ? S[i - 1] : 0);
+            R += S[i] - (i ? S[i - 1] : (A)0);
             emit(p, q0 + have, v, inst, __ldg(p.col + beg + i));
             ++have;
         }
@@ -251,10 +267,63 @@ __device__ void draw_picks(const SelParams& p, const uint64_t* S, uint32_t* bits
     __syncwarp();
 }
 
-// One warp item: all positive neighbours (any degree), or a draw over at most
-// WARP_MAX_DEG neighbours with S in this warp's shared slot.
+// Items that a worker claims from a queue at once: claims are atomics on one
+// address, which the L2 serves one at a time (about 1 ns each), so a layer of
+// millions of items is bound by them when each is claimed alone.  About eight
+// claims per worker still even the work out.
+__device__ __forceinline__ uint32_t claim_chunk(unsigned long long n, uint32_t workers)
+{
+    const unsigned long long c = n / (8ull * workers);
+    return c < 1 ? 1u : c > 32 ? 32u : (uint32_t)c;
+}
+
+// Biases of the eight edges of a lane's group of a row, from the row's first
+// 32-byte sector on (32 bytes per lane, one load): places before `lead` and
+// from `span` on are not the row's.  *skew: the row's place in that sector.
 template <int KIND>
-__device__ void warp_item(const SelParams& p, uint32_t e, uint64_t* sS, uint32_t* sBits, int lane)
+__device__ __forceinline__ uint32_t sector_lead(const SelParams& p, uint64_t beg)
+{
+    if constexpr (KIND == CSAW_BIAS_UNIFORM) return 0u;
+    // by address: a slot of a host graph's partition starts anywhere in its row numbering
+    else if constexpr (KIND == CSAW_BIAS_EDGE_WEIGHT) return (uint32_t)((uintptr_t)(p.w + beg) >> 2) & 7u;
+    else return p.pk.pack ? (uint32_t)(beg & 7) : (uint32_t)((uintptr_t)(p.col + beg) >> 2) & 7u;
+}
+
+template <int KIND>
+__device__ __forceinline__ void sector_biases(const SelParams& p, uint64_t beg, uint32_t lead, uint32_t q,
+                                              uint32_t span, uint32_t (&b)[8])
+{
+#pragma unroll
+    for (int j = 0; j < 8; ++j) b[j] = KIND == CSAW_BIAS_UNIFORM ? 1u : 0u;
+    if (q < span) {
+        if constexpr (KIND == CSAW_BIAS_EDGE_WEIGHT) {
+            ld256(p.w + beg - lead + q, b);
+        } else if constexpr (KIND == CSAW_BIAS_NEIGHBOR_DEGREE) {
+            if (p.pk.pack) {
+                ld256(p.pk.pack + 2 * (beg - lead + q), b);
+            } else {
+                uint32_t c[8];
+                ld256(p.col + beg - lead + q, c);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (q + j >= lead && q + j < span) b[j] = __ldg(p.deg + c[j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (q + j < lead || q + j >= span) b[j] = 0u;
+}
+
+// One warp item: all positive neighbours (any degree), or a draw over at most
+// WARP_MAX_DEG neighbours with S in this warp's shared slot.  A lane holds
+// eight consecutive neighbours (one 32-byte load), so that the row takes one
+// warp scan of lane totals, of 32-bit sums where they fit (A).  Bound by
+// instruction issue (70 %): RMAT s22, 2048 instances, neighbour degree, both
+// layers 4.5 ms, against 5.1 with eight 64-bit scans of strided tiles and 5.7
+// with the degrees gathered and whole rows among the items.
+template <int KIND, class A>
+__device__ void warp_item(const SelParams& p, uint32_t e, A* sS, uint32_t* sBits, int lane)
 {
     const uint64_t key = p.fkeys[e];
     const uint32_t v = (uint32_t)(key & p.vmask);
@@ -264,8 +333,50 @@ __device__ void warp_item(const SelParams& p, uint32_t e, uint64_t* sS, uint32_t
     const uint64_t q0 = p.pos[e];
     const uint32_t cnt = (uint32_t)(p.pos[e + 1] - q0);
     const uint32_t lt = lanemask_lt();
-    if (d > WARP_MAX_DEG) {
-        // Take-all over a long row: stream it, keeping positive biases in CSR order.
+    bool all = d > WARP_MAX_DEG || (!p.zero_bias && cnt >= d);
+    uint32_t lead = 0, span = d;
+    A total = 0;
+    if (!all) {
+        lead = sector_lead<KIND>(p, beg);
+        span = lead + d;
+        uint32_t npos = 0;
+        for (uint32_t base = 0; base < span; base += 256) {
+            const uint32_t q = base + 8 * lane;
+            uint32_t b[8];
+            sector_biases<KIND>(p, beg, lead, q, span, b);
+            A sum[8], run = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                run += b[j];
+                sum[j] = run;
+                npos += b[j] > 0;
+            }
+            A incl = run;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const A y = __shfl_up_sync(CSAW_FULL_MASK, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const A before = total + incl - run;
+            if (q < span) {   // at most to place WARP_SPAN
+                using V = typename std::conditional<sizeof(A) == 4, uint4, ulonglong2>::type;
+                constexpr int N = 16 / (int)sizeof(A);
+                V* out = reinterpret_cast<V*>(sS + q);
+#pragma unroll
+                for (int j = 0; j < 8; j += N) {
+                    V x;
+                    A* xs = reinterpret_cast<A*>(&x);
+#pragma unroll
+                    for (int i = 0; i < N; ++i) xs[i] = before + sum[j + i];
+                    out[j / N] = x;
+                }
+            }
+            total += __shfl_sync(CSAW_FULL_MASK, incl, 31);
+        }
+        if (p.zero_bias) all = __reduce_add_sync(CSAW_FULL_MASK, npos) <= picks_of(p, inst);
+    }
+    if (all) {
+        // stream the row, keeping positive biases in CSR order
         uint64_t q = q0;
         for (uint32_t base = 0; base < d; base += 32) {
             const uint32_t j = base + lane;
@@ -281,42 +392,9 @@ __device__ void warp_item(const SelParams& p, uint32_t e, uint64_t* sS, uint32_t
         }
         return;
     }
-    constexpr int TILES = WARP_MAX_DEG / 32;
-    const uint32_t ntiles = (d + 31) >> 5;
-    uint32_t b[TILES];
-#pragma unroll
-    for (int t = 0; t < TILES; ++t) {
-        const uint32_t j = 32u * t + lane;
-        b[t] = ((uint32_t)t < ntiles && j < d) ? sel_bias<KIND>(p, beg + j) : 0u;
-    }
-    uint64_t run = 0;
-    uint32_t npos = 0;
-#pragma unroll
-    for (int t = 0; t < TILES; ++t) {
-        if ((uint32_t)t < ntiles) {
-            const uint64_t incl = warp_inclusive_scan_u64(b[t], lane) + run;
-            const uint32_t j = 32u * t + lane;
-            if (j < d) sS[j] = incl;
-            run = __shfl_sync(CSAW_FULL_MASK, incl, 31);
-            npos += __popc(__ballot_sync(CSAW_FULL_MASK, b[t] > 0));
-        }
-    }
-    if (npos <= picks_of(p, inst)) {
-        uint64_t q = q0;
-#pragma unroll
-        for (int t = 0; t < TILES; ++t) {
-            if ((uint32_t)t < ntiles) {
-                const bool take = b[t] > 0;
-                const uint32_t bal = __ballot_sync(CSAW_FULL_MASK, take);
-                if (take) emit(p, q + __popc(bal & lt), v, inst, __ldg(p.col + beg + 32u * t + lane));
-                q += __popc(bal);
-            }
-        }
-        return;
-    }
-    if (lane < (int)(WARP_MAX_DEG / 32)) sBits[lane] = 0;
+    if (lane < (int)WARP_BITS) sBits[lane] = 0;
     __syncwarp();
-    draw_picks(p, sS, sBits, d, run, cnt, q0, v, inst, beg, lane);
+    draw_picks<A>(p, sS, sBits, span, total, cnt, q0, v, inst, beg - lead, lane);
     __syncwarp();
 }
 
@@ -370,11 +448,11 @@ __device__ void cta_item(const SelParams& p, uint32_t e, uint64_t* S, uint32_t* 
         carry += tile;
         __syncthreads();
     }
-    if (wid == 0) draw_picks(p, S, bits, d, carry, cnt, q0, v, inst, beg, lane);
+    if (wid == 0) draw_picks<uint64_t>(p, S, bits, d, carry, cnt, q0, v, inst, beg, lane);
     __syncthreads();
 }
 
-template <int KIND>
+template <int KIND, bool WIDE>
 __global__ void __launch_bounds__(SEL_THREADS, 6) select_kernel(SelParams p)
 {
     if (p.key_dev) {
@@ -408,15 +486,18 @@ __global__ void __launch_bounds__(SEL_THREADS, 6) select_kernel(SelParams p)
         cta_item<KIND>(p, e, S, bits, s_wsum);
     }
     // Warp items: each warp uses its own slice of the dynamic region.
-    uint64_t* sS = (uint64_t*)(s_dyn + (size_t)wid * WARP_SLOT);
-    uint32_t* sBits = (uint32_t*)(s_dyn + (size_t)wid * WARP_SLOT + WARP_MAX_DEG * 8);
+    using A = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+    A* sS = (A*)(s_dyn + (size_t)wid * (WIDE ? WARP_SLOT : WARP_SLOT_NARROW));
+    uint32_t* sBits = (uint32_t*)(sS + WARP_SPAN);
     const unsigned long long n_warp = p.skip_warp_items ? 0ull : p.n_items[0];
+    const uint32_t chunk = claim_chunk(n_warp, gridDim.x * SEL_WARPS);
     while (true) {
         unsigned long long it = 0;
-        if (lane == 0) it = atomicAdd(p.next, 1ull);
+        if (lane == 0) it = atomicAdd(p.next, (unsigned long long)chunk);
         it = __shfl_sync(CSAW_FULL_MASK, it, 0);
         if (it >= n_warp) break;
-        warp_item<KIND>(p, p.warp_list[it], sS, sBits, lane);
+        const unsigned long long end = min(it + chunk, n_warp);
+        for (; it < end; ++it) warp_item<KIND, A>(p, p.warp_list[it], sS, sBits, lane);
     }
 }
 
@@ -434,16 +515,20 @@ __device__ __forceinline__ uint64_t cdf_at(const uint64_t* __restrict__ row, boo
     return implicit ? (uint64_t)i + 1 : __ldg(row + i);
 }
 
-// CACHED: rows of the graph's cumulative array, searched through its
-// summaries (cdf_search); otherwise bisected directly (shared hub arrays).
+// SRC: where the prefix sums are -- implicit (uniform), the rows of the
+// graph's cumulative array, searched through its summaries (cdf_search), the
+// packed array (pack_pick), or the shared hub arrays, bisected directly.
 // G: lanes per item -- 32, or 16 (two items per warp, rounds of 16
 // attempts; for layers whose fanout is at most 16, where a hub row's first
 // round nearly always holds the picks).  Attempts are taken in the same
 // order either way, so the picks do not depend on G.
-template <bool IMPLICIT, bool CACHED = false, int G = 32>
-__global__ void __launch_bounds__(SEL_THREADS, CACHED ? 6 : 8) select_cdf_kernel(SelParams p)
+enum : int { SRC_IMPLICIT = 0, SRC_LEAF = 1, SRC_HUB = 2, SRC_PACK = 3 };
+
+template <int SRC, int G = 32>
+__global__ void __launch_bounds__(SEL_THREADS, SRC == SRC_PACK ? 5 : SRC == SRC_LEAF ? 6 : 8) select_cdf_kernel(SelParams p)
 {
     static_assert(G == 32 || G == 16, "16 or 32 lanes per item");
+    constexpr bool IMPLICIT = SRC == SRC_IMPLICIT;
     __shared__ uint32_t s_picks[SEL_WARPS][PICK_MAX];
     if (p.key_dev) {
         p.k0 = p.key_dev[0];
@@ -457,17 +542,31 @@ __global__ void __launch_bounds__(SEL_THREADS, CACHED ? 6 : 8) select_cdf_kernel
     const bool hub = p.item_e != nullptr;   // hub items (vertex order): shared array or cached one
     const unsigned long long n_warp = hub ? p.n_items[2] : p.n_items[0];
     unsigned long long* counter = hub ? p.next + 2 : p.next;
-    while (true) {
-        unsigned long long it = 0;
-        if (gl == 0) it = atomicAdd(counter, 1ull);
-        it = __shfl_sync(gmask, it, gb);
-        if (it >= n_warp) break;
+    const uint32_t chunk = claim_chunk(n_warp, gridDim.x * (SEL_THREADS / G));
+    for (unsigned long long it = 0, end = 0;; ++it) {
+        if (it == end) {
+            if (gl == 0) it = atomicAdd(counter, (unsigned long long)chunk);
+            it = __shfl_sync(gmask, it, gb);
+            if (it >= n_warp) break;
+            end = min(it + chunk, n_warp);
+        }
         const uint32_t e = hub ? p.item_e[it] : p.warp_list[it];
         const uint64_t key = p.fkeys[e];
         const uint32_t v = (uint32_t)(key & p.vmask);
         const uint32_t inst = (uint32_t)(key >> p.vbits);
-        const uint64_t beg = __ldg(p.off + v);
-        const uint32_t d = (uint32_t)(__ldg(p.off + v + 1) - beg);
+        uint64_t beg, low = 0, T = 0;   // low: the packed array's sum before the row
+        uint32_t d;
+        if constexpr (SRC == SRC_PACK) {
+            const ulonglong2* rc = reinterpret_cast<const ulonglong2*>(p.pk.rec) + v;
+            const ulonglong2 r0 = __ldg(rc), r1 = __ldg(rc + 1);
+            beg = r0.x;
+            d = (uint32_t)(r1.x - beg);
+            low = r0.y;
+            T = r1.y - low;
+        } else {
+            beg = __ldg(p.off + v);
+            d = (uint32_t)(__ldg(p.off + v + 1) - beg);
+        }
         const uint64_t q0 = p.pos[e];
         const uint32_t cnt = (uint32_t)(p.pos[e + 1] - q0);
         if (cnt >= d) {
@@ -475,25 +574,39 @@ __global__ void __launch_bounds__(SEL_THREADS, CACHED ? 6 : 8) select_cdf_kernel
             for (uint32_t j = gl; j < d; j += G) emit(p, q0 + j, v, inst, __ldg(p.col + beg + j));
             continue;
         }
-        if (hub && p.hubS && p.hub_off[p.item_h[it]] + d > p.hubS_cap) {
-            if (gl == 0) atomicOr(p.err, 8u);   // never happens when the scratch is sized right
-            continue;
+        const uint64_t* row = SRC == SRC_LEAF ? p.cdf + beg : nullptr;
+        if constexpr (SRC == SRC_HUB) {
+            const uint64_t at = p.hub_off[p.item_h[it]];
+            if (at + d > p.hubS_cap) {
+                if (gl == 0) atomicOr(p.err, 8u);   // never happens when the scratch is sized right
+                continue;
+            }
+            row = p.hubS + at;
         }
-        const uint64_t* row = hub && p.hubS ? p.hubS + p.hub_off[p.item_h[it]] : p.cdf ? p.cdf + beg : nullptr;
         const DrawKey dk = draw_key(p, inst);
-        const uint64_t T = cdf_at(row, IMPLICIT, d - 1);
+        // the row's prefix sum up to its i-th neighbour
+        const auto sum_to = [&](uint32_t i) -> uint64_t {
+            if constexpr (SRC == SRC_PACK) return pack_prefix(p.pk, beg + i + 1) - low;
+            else return cdf_at(row, IMPLICIT, i);
+        };
+        if constexpr (SRC != SRC_PACK) T = cdf_at(row, IMPLICIT, d - 1);
         uint32_t have = 0, a0 = 0;
         uint32_t used = 0, rounds = 0;   // counters (CSAW_STATS)
         (void)used;
         (void)rounds;
         while (have < cnt && a0 < p.attempt_cap) {
             const bool live = a0 + gl < p.attempt_cap;   // the last round may be partial
-            const uint64_t x = scale_draw(philox_draw(dk.k0, dk.k1, a0 + gl, v, p.layer, dk.id), T);
-            uint32_t i = 0xFFFFFFFFu;
+            const uint64_t r = philox_draw(dk.k0, dk.k1, a0 + gl, v, p.layer, dk.id);
+            const uint64_t x = scale_draw(r, T);
+            uint32_t i = 0xFFFFFFFFu, u = 0;
             if (!live) {
-            } else if (IMPLICIT) {
+            } else if constexpr (IMPLICIT) {
                 i = (uint32_t)x;
-            } else if (CACHED) {
+            } else if constexpr (SRC == SRC_PACK) {
+                const PackHit h = pack_pick(p.pk, beg, beg + d, beg + __umul64hi(r, d), low + x);
+                i = (uint32_t)(h.e - beg);
+                u = h.col;
+            } else if constexpr (SRC == SRC_LEAF) {
                 i = (uint32_t)(cdf_search(p.cv, beg, beg + d, x) - beg);   // the cached array
             } else {
                 uint32_t lo = 0, hi = d - 1;
@@ -512,7 +625,7 @@ __global__ void __launch_bounds__(SEL_THREADS, CACHED ? 6 : 8) select_cdf_kernel
             const uint32_t need = cnt - have;
             if (fresh && rank < need) {
                 picks[have + rank] = i;
-                emit(p, q0 + have + rank, v, inst, __ldg(p.col + beg + i));
+                emit(p, q0 + have + rank, v, inst, SRC == SRC_PACK ? u : __ldg(p.col + beg + i));
             }
 #ifdef CSAW_STATS
             used = (uint32_t)__popc(bal) >= need ? a0 + nth_set_bit(bal, need) + 1 : min(a0 + G, p.attempt_cap);
@@ -544,26 +657,26 @@ __global__ void __launch_bounds__(SEL_THREADS, CACHED ? 6 : 8) select_cdf_kernel
             uint64_t R = 0;
             for (uint32_t j = 0; j < have; ++j) {
                 const uint32_t q = picks[j];
-                R += cdf_at(row, IMPLICIT, q) - (q ? cdf_at(row, IMPLICIT, q - 1) : 0);
+                R += sum_to(q) - (q ? sum_to(q - 1) : 0);
             }
             for (uint32_t a = p.attempt_cap; have < cnt; ++a) {
                 uint64_t x = scale_draw(philox_draw(dk.k0, dk.k1, a, v, p.layer, dk.id), T - R);
                 for (uint32_t j = 0; j < have; ++j) {
                     const uint32_t q = picks[j];
-                    const uint64_t start = q ? cdf_at(row, IMPLICIT, q - 1) : 0;
-                    if (x >= start) x += cdf_at(row, IMPLICIT, q) - start;
+                    const uint64_t start = q ? sum_to(q - 1) : 0;
+                    if (x >= start) x += sum_to(q) - start;
                     else break;
                 }
                 uint32_t lo = 0, hi = d - 1;
                 while (lo < hi) {
                     const uint32_t mid = (lo + hi) >> 1;
-                    if (cdf_at(row, IMPLICIT, mid) > x) hi = mid; else lo = mid + 1;
+                    if (sum_to(mid) > x) hi = mid; else lo = mid + 1;
                 }
                 const uint32_t i = lo;
                 uint32_t b = have;
                 while (b > 0 && picks[b - 1] > i) { picks[b] = picks[b - 1]; --b; }
                 picks[b] = i;
-                R += cdf_at(row, IMPLICIT, i) - (i ? cdf_at(row, IMPLICIT, i - 1) : 0);
+                R += sum_to(i) - (i ? sum_to(i - 1) : 0);
                 emit(p, q0 + have, v, inst, __ldg(p.col + beg + i));
                 ++have;
             }
@@ -594,6 +707,11 @@ struct CountParams {
     // hub items (degree above theta_w, at most PICK_MAX picks) when the layer
     // shares one cumulative array per distinct hub; null: they are CTA items
     uint32_t* __restrict__ hub_list = nullptr;
+    // entries that take a whole row of at most TAKE_MAX_DEG neighbours, every
+    // bias positive, when take_all_kernel serves them: from the end of
+    // warp_list (which has room for every entry) backwards; 0: warp items
+    uint64_t take_end = 0;
+    unsigned long long* n_take = nullptr;
     // picks per vertex of each instance at this layer (null: k for all)
     const uint32_t* __restrict__ inst_k = nullptr;
     uint32_t vbits = 0;
@@ -618,17 +736,20 @@ __device__ uint32_t count_positive(const CountParams& p, uint64_t beg, uint32_t 
     return __reduce_add_sync(CSAW_FULL_MASK, c);
 }
 
+constexpr uint32_t TAKE_MAX_DEG = 1024;
+constexpr int COUNT_THREADS = 256, COUNT_WARPS = COUNT_THREADS / 32;
+
 template <int KIND>
-__global__ void count_kernel(CountParams p)
+__global__ void __launch_bounds__(COUNT_THREADS) count_kernel(CountParams p)
 {
+    __shared__ uint32_t s_n[4][COUNT_WARPS];
+    __shared__ unsigned long long s_base[4];
     const int lane = threadIdx.x & 31;
     const uint64_t n = *p.n_dev;
-    const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     // one warp handles 32 consecutive entries; the positive count (if needed)
     // is computed cooperatively entry by entry
-    for (uint64_t base = gw * 32; base < n; base += nw * 32) {
-        const uint64_t e = base + lane;
+    for (uint64_t base = (uint64_t)blockIdx.x * COUNT_THREADS; base < n; base += (uint64_t)gridDim.x * COUNT_THREADS) {
+        const uint64_t e = base + threadIdx.x;
         uint32_t v = 0, d = 0;
         uint64_t beg = 0;
         if (e < n) {
@@ -649,30 +770,88 @@ __global__ void count_kernel(CountParams p)
         const uint32_t c = min(k, npos);
         const bool take_all = npos <= k;
         const bool listed = e < n && c > 0 && v >= p.v_lo && v < p.v_hi;
-        const bool to_warp = listed && (take_all || (p.cached && !p.hub_list ? c <= PICK_MAX : d <= p.theta_w));
-        const bool to_hub = listed && !to_warp && p.hub_list != nullptr && c <= PICK_MAX;
-        const bool to_cta = listed && !to_warp && !to_hub;
+        const bool to_take = listed && take_all && p.take_end && !p.zero_bias && d <= TAKE_MAX_DEG;
+        const bool to_warp = listed && !to_take &&
+                             (take_all || (p.cached && !p.hub_list ? c <= PICK_MAX : d <= p.theta_w));
+        const bool to_hub = listed && !to_warp && !to_take && p.hub_list != nullptr && c <= PICK_MAX;
+        const bool to_cta = listed && !to_warp && !to_take && !to_hub;
         if (e < n && p.write_cnt) p.cnt[e] = c;
-        // warp-aggregated appends
+        // appends to the lists, one atomic per block and list
         const uint32_t bw = __ballot_sync(CSAW_FULL_MASK, to_warp);
         const uint32_t bc = __ballot_sync(CSAW_FULL_MASK, to_cta);
         const uint32_t bh = __ballot_sync(CSAW_FULL_MASK, to_hub);
-        unsigned long long basew = 0, basec = 0, baseh = 0;
-        if (lane == 0) {
-            if (bw) basew = atomicAdd(p.n_items, (unsigned long long)__popc(bw));
-            if (bc) basec = atomicAdd(p.n_items + 1, (unsigned long long)__popc(bc));
-            if (bh) baseh = atomicAdd(p.n_items + 2, (unsigned long long)__popc(bh));
-            CSAW_STAT_ADD(4, __popc(bw));
-            CSAW_STAT_ADD(5, __popc(bc));
-            CSAW_STAT_ADD(6, __popc(bh));
+        const uint32_t bt = __ballot_sync(CSAW_FULL_MASK, to_take);
+        const int wid = threadIdx.x >> 5;
+        if (lane < 4) s_n[lane][wid] = __popc(lane == 0 ? bw : lane == 1 ? bc : lane == 2 ? bh : bt);
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            uint32_t t = 0;
+            for (int k2 = 0; k2 < COUNT_WARPS; ++k2) {
+                const uint32_t c2 = s_n[threadIdx.x][k2];
+                s_n[threadIdx.x][k2] = t;
+                t += c2;
+            }
+            s_base[threadIdx.x] = t ? atomicAdd(threadIdx.x < 3 ? p.n_items + threadIdx.x : p.n_take,
+                                                (unsigned long long)t) : 0ull;
+            CSAW_STAT_ADD(threadIdx.x < 3 ? 4 + threadIdx.x : 4, t);   // a whole row is a warp item
         }
-        basew = __shfl_sync(CSAW_FULL_MASK, basew, 0);
-        basec = __shfl_sync(CSAW_FULL_MASK, basec, 0);
-        baseh = __shfl_sync(CSAW_FULL_MASK, baseh, 0);
+        __syncthreads();
+        const unsigned long long basew = s_base[0] + s_n[0][wid], basec = s_base[1] + s_n[1][wid],
+                                 baseh = s_base[2] + s_n[2][wid], baset = s_base[3] + s_n[3][wid];
         const uint32_t lt = lanemask_lt();
         if (to_warp) p.warp_list[basew + __popc(bw & lt)] = (uint32_t)e;
         if (to_cta) p.cta_list[basec + __popc(bc & lt)] = (uint32_t)e;
         if (to_hub) p.hub_list[baseh + __popc(bh & lt)] = (uint32_t)e;
+        if (to_take) p.warp_list[p.take_end - 1 - (baset + __popc(bt & lt))] = (uint32_t)e;
+        __syncthreads();   // the offsets are read before the next round's
+    }
+}
+
+// Entries that take every neighbour of a short row: a warp takes 32 of them at
+// once, and its lanes their edges in turn (most rows of a power-law graph are
+// a few neighbours, so a warp per entry waited on the loads of one row at a
+// time with most lanes idle): 0.26 ms for both layers of the s22 plan, where
+// the warp items took 1.3 ms longer with them.
+__global__ void __launch_bounds__(SEL_THREADS) take_all_kernel(SelParams p, const uint32_t* __restrict__ list_end,
+                                                              const unsigned long long* __restrict__ n_dev)
+{
+    const int lane = threadIdx.x & 31;
+    const uint64_t n = *n_dev;
+    const uint64_t gw = ((uint64_t)blockIdx.x * SEL_THREADS + threadIdx.x) >> 5;
+    const uint64_t nw = ((uint64_t)gridDim.x * SEL_THREADS) >> 5;
+    for (uint64_t base = gw * 32; base < n; base += nw * 32) {
+        uint64_t key = 0, beg = 0, q0 = 0;
+        uint32_t d = 0;
+        if (base + lane < n) {
+            const uint32_t e = list_end[-1 - (int64_t)(base + lane)];
+            key = p.fkeys[e];
+            const uint32_t v = (uint32_t)(key & p.vmask);
+            beg = __ldg(p.off + v);
+            d = (uint32_t)(__ldg(p.off + v + 1) - beg);
+            q0 = p.pos[e];
+        }
+        uint32_t incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(CSAW_FULL_MASK, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(CSAW_FULL_MASK, incl, 31);
+        // row of edge t: column base and edge position less the edges before
+        const uint64_t from = beg - (incl - d), to = q0 - (incl - d);
+        for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+            const uint32_t t = t0 + lane;
+            int j = 0;   // the number of rows that end at or before t
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(CSAW_FULL_MASK, incl, j + o - 1) <= t) j += o;
+            j = min(j, 31);
+            const uint64_t kj = __shfl_sync(CSAW_FULL_MASK, key, j);
+            const uint64_t fj = __shfl_sync(CSAW_FULL_MASK, from, j);
+            const uint64_t tj = __shfl_sync(CSAW_FULL_MASK, to, j);
+            if (t < total)
+                emit(p, tj + t, (uint32_t)(kj & p.vmask), (uint32_t)(kj >> p.vbits), __ldg(p.col + fj + t));
+        }
     }
 }
 
@@ -1080,10 +1259,40 @@ struct Temps {
     }
 };
 
-template <int KIND>
-static csaw_status launch_select(const SelParams& p, int blocks, cudaStream_t s, size_t smem = SEL_DYN_SMEM)
+// Whether a warp item's sums of this kind may pass 32 bits.
+static bool select_wide(const csaw_graph* g, int kind)
 {
-    select_kernel<KIND><<<blocks, SEL_THREADS, smem, s>>>(p);
+    const uint64_t most = kind == CSAW_BIAS_UNIFORM ? 1 : kind == CSAW_BIAS_EDGE_WEIGHT ? g->max_weight : g->max_degree;
+    return most * WARP_SPAN >= (1ull << 32);
+}
+
+static const void* select_fn(int kind, bool wide)
+{
+    switch (kind) {
+    case CSAW_BIAS_UNIFORM: return (const void*)select_kernel<CSAW_BIAS_UNIFORM, false>;
+    case CSAW_BIAS_EDGE_WEIGHT:
+        return wide ? (const void*)select_kernel<CSAW_BIAS_EDGE_WEIGHT, true>
+                    : (const void*)select_kernel<CSAW_BIAS_EDGE_WEIGHT, false>;
+    default:
+        return wide ? (const void*)select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE, true>
+                    : (const void*)select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE, false>;
+    }
+}
+
+static csaw_status launch_select(int kind, bool wide, const SelParams& p, int blocks, cudaStream_t s,
+                                 size_t smem = SEL_DYN_SMEM)
+{
+    switch (kind) {
+    case CSAW_BIAS_UNIFORM: select_kernel<CSAW_BIAS_UNIFORM, false><<<blocks, SEL_THREADS, smem, s>>>(p); break;
+    case CSAW_BIAS_EDGE_WEIGHT:
+        if (wide) select_kernel<CSAW_BIAS_EDGE_WEIGHT, true><<<blocks, SEL_THREADS, smem, s>>>(p);
+        else select_kernel<CSAW_BIAS_EDGE_WEIGHT, false><<<blocks, SEL_THREADS, smem, s>>>(p);
+        break;
+    default:
+        if (wide) select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE, true><<<blocks, SEL_THREADS, smem, s>>>(p);
+        else select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE, false><<<blocks, SEL_THREADS, smem, s>>>(p);
+        break;
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "select_kernel");
     return CSAW_OK;
@@ -1092,70 +1301,41 @@ static csaw_status launch_select(const SelParams& p, int blocks, cudaStream_t s,
 template <int KIND>
 static csaw_status launch_count(const CountParams& p, uint64_t n, int sm_count, cudaStream_t s)
 {
-    count_kernel<KIND><<<grid_for((n + 31) / 32 * 32, 256, sm_count), 256, 0, s>>>(p);
+    count_kernel<KIND><<<grid_for(n, COUNT_THREADS, sm_count), COUNT_THREADS, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "count_kernel");
     return CSAW_OK;
 }
 
 // Resident blocks of the selection kernel per SM (occupancy limit).
-static int select_occupancy(int kind)
+static int select_occupancy(int kind, bool wide)
 {
-    // looked up once per kind; the attribute is set before the value is
-    // published, so a thread that reads it may launch (calls may come from
+    // looked up once per kind and width; the attribute is set before the value
+    // is published, so a thread that reads it may launch (calls may come from
     // several threads, e.g. the request server's slots)
-    static std::atomic<int> cached[4];
-    const int have = cached[kind].load(std::memory_order_acquire);
-    if (have) return have;
-    {
-        int per_sm = 1;
-        cudaError_t e = cudaSuccess;
-        switch (kind) {
-        case CSAW_BIAS_UNIFORM:
-            cudaFuncSetAttribute(select_kernel<CSAW_BIAS_UNIFORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_DYN_SMEM);
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_UNIFORM>, SEL_THREADS, SEL_DYN_SMEM);
-            break;
-        case CSAW_BIAS_EDGE_WEIGHT:
-            cudaFuncSetAttribute(select_kernel<CSAW_BIAS_EDGE_WEIGHT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_DYN_SMEM);
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_EDGE_WEIGHT>, SEL_THREADS, SEL_DYN_SMEM);
-            break;
-        default:
-            cudaFuncSetAttribute(select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_DYN_SMEM);
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE>, SEL_THREADS, SEL_DYN_SMEM);
-            break;
-        }
-        if (e != cudaSuccess || per_sm < 1) per_sm = 1;
-        cached[kind].store(per_sm, std::memory_order_release);
-        return per_sm;
-    }
-}
-
-static int select_blocks(int kind, int sm_count)
-{
-    return sm_count * select_occupancy(kind);
-}
-
-// Resident blocks per SM of a launch with warp items only (SEL_WARP_SMEM).
-static int select_occupancy_warp(int kind)
-{
-    static std::atomic<int> cached[4];
-    const int have = cached[kind].load(std::memory_order_acquire);
+    static std::atomic<int> cached[4][2];
+    const int have = cached[kind][wide].load(std::memory_order_acquire);
     if (have) return have;
     int per_sm = 1;
-    cudaError_t e = cudaSuccess;
-    switch (kind) {
-    case CSAW_BIAS_UNIFORM:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_UNIFORM>, SEL_THREADS, SEL_WARP_SMEM);
-        break;
-    case CSAW_BIAS_EDGE_WEIGHT:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_EDGE_WEIGHT>, SEL_THREADS, SEL_WARP_SMEM);
-        break;
-    default:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel<CSAW_BIAS_NEIGHBOR_DEGREE>, SEL_THREADS, SEL_WARP_SMEM);
-        break;
-    }
+    const void* fn = select_fn(kind, wide);
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SEL_DYN_SMEM);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SEL_THREADS, SEL_DYN_SMEM);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
-    cached[kind].store(per_sm, std::memory_order_release);
+    cached[kind][wide].store(per_sm, std::memory_order_release);
+    return per_sm;
+}
+
+// Resident blocks per SM of a launch with warp items only (sel_warp_smem).
+static int select_occupancy_warp(int kind, bool wide)
+{
+    static std::atomic<int> cached[4][2];
+    const int have = cached[kind][wide].load(std::memory_order_acquire);
+    if (have) return have;
+    int per_sm = 1;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_fn(kind, wide), SEL_THREADS,
+                                                                        sel_warp_smem(wide));
+    if (e != cudaSuccess || per_sm < 1) per_sm = 1;
+    cached[kind][wide].store(per_sm, std::memory_order_release);
     return per_sm;
 }
 
@@ -1165,7 +1345,7 @@ static void select_shape(const csaw_graph* g, int kind, uint32_t* theta_w, int* 
 {
     const uint32_t tw = g->tune_theta_w[kind];
     *theta_w = (tw == 0 || tw > WARP_MAX_DEG) ? WARP_MAX_DEG : tw;
-    const int occ = select_occupancy(kind);
+    const int occ = select_occupancy(kind, select_wide(g, kind));
     int per = (int)g->tune_blocks_per_sm[kind];
     if (per <= 0 || per > occ) per = occ;
     *blocks = g->sm_count * per;
@@ -1182,10 +1362,10 @@ enum : int {
     CT_WORDS = CT_LAYER + L_WORDS * CSAW_MAX_DEPTH,
 };
 // per layer: frontier entries, edges, item counts (warp, CTA, hub) and their
-// work counters, distinct hubs, their edges, hubs built by a whole CTA and
-// the two build counters
+// work counters, distinct hubs, their edges, hubs built by a whole CTA, the
+// two build counters and the whole-row entries
 enum : int { L_N = 0, L_TOTAL = 1, L_ITEMS = 2, L_NEXT = 5, L_NH = 8, L_HUBE = 9, L_NBIG = 10,
-             L_HNEXT = 11 };
+             L_HNEXT = 11, L_TAKE = 13 };
 
 // ---------------------------------------------------------------------------
 // Layer sampling (Sec. II-A; Fig. 2(b) with the whole frontier as the current
@@ -1779,10 +1959,12 @@ struct Pipeline {
     uint64_t vmask = 1;
     int sel_blocks = 1;
     uint32_t theta_w = WARP_MAX_DEG;
-    bool cached = false;                 // selection over a cached cumulative array
+    bool cached = false;                 // selection over a cached cumulative or packed array
+    const uint64_t* pack = nullptr;      // the packed array: the graph's, or one built in the run
+    bool take = true;                    // whole short rows by take_all_kernel
     bool hub_path = false;               // shared hub arrays per layer (static bias, streamed)
     bool hub_order = false;              // cached static bias: hub items visited in vertex order
-    bool cta_slots = false;              // CTA items may exceed CTA_SMEM_DEG: global slots
+    bool any_big_k = false;              // some layer takes more than PICK_MAX picks
     uint32_t attempt_cap = CSAW_ATTEMPT_CAP;
     uint32_t k0 = 0, k1 = 0;
     const uint32_t* key_dev = nullptr;   // plan mode: Philox key in device memory
@@ -1836,19 +2018,39 @@ struct Pipeline {
                     (kind == CSAW_BIAS_NEIGHBOR_DEGREE && g->zero_degree_target);
         select_shape(g, kind, &theta_w, &sel_blocks);
         cached = cached_cdf_usable(g, kind);
+        if (cached && kind != CSAW_BIAS_UNIFORM) pack = g->pack[kind];
+        paths();
+        bool big_k = false;
+        for (uint32_t l = 0; l < dep; ++l) big_k |= fan[l] > PICK_MAX && fan[l] != CSAW_FANOUT_ALL;
+        any_big_k = big_k;
+        k0 = (uint32_t)seed;
+        k1 = (uint32_t)(seed >> 32);
+    }
+
+    // A packed array built in the run (words) takes the place of the hub
+    // arrays and of streamed short rows.
+    void use_pack(const uint64_t* words)
+    {
+        pack = words;
+        cached = true;
+        paths();
+    }
+
+    void paths()
+    {
         // shared hub arrays pay when several instances can reach the same
         // hub; a single instance's frontier holds each vertex once, and its
         // long rows take the CTA path without the grouping kernels
         hub_path = !cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE);
         // vertex order pays only when several instances can hold the same hub
         hub_order = cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE);
-        // CTA items exist for picks above PICK_MAX (or, without the hub
-        // path, any long row); only rows above CTA_SMEM_DEG need a slot
-        bool big_k = false;
-        for (uint32_t l = 0; l < dep; ++l) big_k |= fan[l] > PICK_MAX && fan[l] != CSAW_FANOUT_ALL;
-        cta_slots = g->max_degree > CTA_SMEM_DEG && (big_k || (!cached && !hub_path));
-        k0 = (uint32_t)seed;
-        k1 = (uint32_t)(seed >> 32);
+    }
+
+    // CTA items exist for picks above PICK_MAX (or, without the hub path, any
+    // long row); only rows above CTA_SMEM_DEG need a slot.
+    bool cta_slots() const
+    {
+        return g->max_degree > CTA_SMEM_DEG && (any_big_k || (!cached && !hub_path));
     }
 
     // Capacities of a layer's per-entry and edge arrays.
@@ -1858,6 +2060,32 @@ struct Pipeline {
         return f * k;
     }
 };
+
+// Whether a run should build the packed array and draw long rows from it (and
+// read degrees from it).  The array takes about 4.3 ps per edge of the graph
+// and 20 us.  Against it, in ps: with several instances, the grouping of hub
+// items and the hubs' own prefix sums (150 us in small runs, and 150 per
+// frontier entry in large ones: RMAT s12 to s22); with one, whose long rows a
+// block each would scan, about 2 per neighbour of a row reached by an edge
+// (see walk_array_pays).  A frontier is taken as eight times the one before,
+// most rows being short.  The batched s22 plan (2048 instances, 32 M edges of
+// frontier) draws its long rows in 4.9 ms, with 0.6 for the array, against 8.3
+// over shared hub arrays.
+static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
+{
+    const csaw_graph* g = P.g;
+    if (P.kind == CSAW_BIAS_UNIFORM || P.cached || P.zero_bias || !pack_fits(g, P.kind) || n_seeds == 0) return false;
+    const double visited = std::sqrt((double)g->E / (double)g->V * (double)g->max_degree);
+    double entries = 0, reached = 0, f = (double)n_seeds;
+    for (uint32_t l = 0; l < P.depth; ++l) {
+        entries += f;
+        if (l) reached += f;
+        f *= std::min<double>(P.fanout[l], 8.0);
+        f = std::min(f, (double)P.n_inst * (double)g->V);
+    }
+    const double cost = 4.3 * (double)g->E + 20e6;
+    return P.n_inst > 1 ? 150e6 + 150.0 * entries >= cost : 2.0 * reached * visited >= cost + 40e6;
+}
 
 // Layer-0 frontier: sorted distinct (instance, seed) keys.
 static csaw_status enqueue_frontier0(Pipeline& P, const uint32_t* seeds, const uint64_t* inst_off,
@@ -1935,10 +2163,12 @@ static csaw_status enqueue_classify(Pipeline& P, uint32_t l, uint32_t v_lo, uint
     cp.k = P.fanout[l]; cp.theta_w = P.theta_w; cp.cached = P.cached; cp.zero_bias = P.zero_bias;
     cp.cnt = B.cnt; cp.warp_list = B.wlist; cp.cta_list = B.clist;
     cp.n_items = (unsigned long long*)P.lc(l, L_ITEMS);
-    cp.hub_list = P.hub_path || P.hub_order ? P.hlist : nullptr;
+    cp.hub_list = P.hub_path || P.hub_order || P.pack ? P.hlist : nullptr;
     cp.inst_k = P.inst_fan ? P.inst_fan + (uint64_t)l * P.n_inst : nullptr;
     cp.vbits = (uint32_t)P.vbits;
     cp.v_lo = v_lo; cp.v_hi = v_hi; cp.write_cnt = write_cnt;
+    cp.take_end = P.take ? B.f_cap : 0;
+    cp.n_take = (unsigned long long*)P.lc(l, L_TAKE);
     if (B.f_cap) {
         switch (P.kind) {
         case CSAW_BIAS_UNIFORM: CSAW_TRY(launch_count<CSAW_BIAS_UNIFORM>(cp, B.f_cap, g->sm_count, s)); break;
@@ -1976,43 +2206,53 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
         sp.out_src = B.src; sp.out_dst = B.dst; sp.out_cand = (l + 1 < P.depth) ? B.cand : nullptr;
         sp.scratch_S = P.hub_S; sp.scratch_bits = P.hub_bits; sp.scratch_stride = g->max_degree;
         sp.cdf = P.cached && P.kind != CSAW_BIAS_UNIFORM ? g->cdf[P.kind] : nullptr;
-    sp.cv = cdf_view(sp.cdf, g->E, g->V);
-        sp.skip_warp_items = P.cached;
+        sp.cv = cdf_view(sp.cdf, g->E, g->V);
+        sp.pk = pack_view(P.pack, g->E, g->V);
+        sp.skip_warp_items = P.cached && !P.pack;
         sp.attempt_cap = P.attempt_cap;
         sp.inst_key = P.inst_key; sp.inst_id = P.inst_id;
         sp.inst_k = P.inst_fan ? P.inst_fan + (uint64_t)l * P.n_inst : nullptr;
+        if (P.take) {
+            take_all_kernel<<<grid_for(B.f_cap, SEL_THREADS, g->sm_count), SEL_THREADS, 0, s>>>(
+                sp, B.wlist + B.f_cap, (const unsigned long long*)P.lc(l, L_TAKE));
+            CSAW_CUDA(cudaGetLastError());
+        }
         if (P.cached) {
             // warp items over the cached array; CTA items (more than PICK_MAX
             // picks) by the streaming kernel below
+            const bool half = P.fanout[l] <= 16;   // two items per warp
             const int blocks = g->sm_count * 8;
-            if (P.kind == CSAW_BIAS_UNIFORM) select_cdf_kernel<true><<<blocks, SEL_THREADS, 0, s>>>(sp);
-            else select_cdf_kernel<false, true><<<blocks, SEL_THREADS, 0, s>>>(sp);
-            if (P.hub_order) {
-                // the hub items in vertex order, over the same array
-                SelParams hs = sp;
-                hs.item_e = P.item_e;
-                if (P.fanout[l] <= 16) select_cdf_kernel<false, true, 16><<<blocks, SEL_THREADS, 0, s>>>(hs);
-                else select_cdf_kernel<false, true><<<blocks, SEL_THREADS, 0, s>>>(hs);
+            SelParams hs = sp;   // hub items, in vertex order where several instances can hold a hub
+            hs.item_e = P.hub_order ? P.item_e : P.hlist;
+            if (P.kind == CSAW_BIAS_UNIFORM) {
+                if (half) select_cdf_kernel<SRC_IMPLICIT, 16><<<blocks, SEL_THREADS, 0, s>>>(sp);
+                else select_cdf_kernel<SRC_IMPLICIT><<<blocks, SEL_THREADS, 0, s>>>(sp);
+            } else if (P.pack) {
+                if (half) select_cdf_kernel<SRC_PACK, 16><<<blocks, SEL_THREADS, 0, s>>>(hs);
+                else select_cdf_kernel<SRC_PACK><<<blocks, SEL_THREADS, 0, s>>>(hs);
+            } else {
+                select_cdf_kernel<SRC_LEAF><<<blocks, SEL_THREADS, 0, s>>>(sp);
+                if (P.hub_order && half) select_cdf_kernel<SRC_LEAF, 16><<<blocks, SEL_THREADS, 0, s>>>(hs);
+                else if (P.hub_order) select_cdf_kernel<SRC_LEAF><<<blocks, SEL_THREADS, 0, s>>>(hs);
             }
             CSAW_CUDA(cudaGetLastError());
         }
         // with shared hub arrays a CTA item needs more than PICK_MAX picks: a
         // layer whose fanout is at most that holds warp items only, launched
         // with their slots alone (more resident blocks hide the gathers)
-        const bool warp_only = P.hub_path && P.fanout[l] <= PICK_MAX;
+        const bool few = P.fanout[l] <= PICK_MAX || P.fanout[l] == CSAW_FANOUT_ALL;
+        const bool warp_only = (P.hub_path || P.pack) && few;
+        const bool wide = select_wide(g, P.kind);
         int blocks = P.sel_blocks;
         size_t smem = SEL_DYN_SMEM;
         if (warp_only) {
-            const int occ = select_occupancy_warp(P.kind);
+            const int occ = select_occupancy_warp(P.kind, wide);
             const int per = (int)g->tune_blocks_per_sm[P.kind];
             blocks = g->sm_count * (per > 0 && per < occ ? per : occ);
-            smem = SEL_WARP_SMEM;
+            smem = sel_warp_smem(wide);
         }
-        switch (P.kind) {
-        case CSAW_BIAS_UNIFORM: CSAW_TRY(launch_select<CSAW_BIAS_UNIFORM>(sp, blocks, s, smem)); break;
-        case CSAW_BIAS_EDGE_WEIGHT: CSAW_TRY(launch_select<CSAW_BIAS_EDGE_WEIGHT>(sp, blocks, s, smem)); break;
-        default: CSAW_TRY(launch_select<CSAW_BIAS_NEIGHBOR_DEGREE>(sp, blocks, s, smem)); break;
-        }
+        // without short rows to draw from only entries with more than PICK_MAX picks are left
+        if (!sp.skip_warp_items || !few) CSAW_TRY(launch_select(P.kind, wide, sp, blocks, s, smem));
         if (P.hub_path) {
             // the layer's distinct hubs: prefix sums built once each, then
             // every hub item draws from them
@@ -2031,8 +2271,8 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             hs.item_e = P.item_e; hs.item_h = P.item_h; hs.hub_off = P.hub_off; hs.hubS = P.hubS;
             hs.hubS_cap = P.hubS_cap; hs.err = (uint32_t*)(P.ctr + CT_ERR);
             // hub rows are long, so with at most 16 picks two items share a warp
-            if (P.fanout[l] <= 16) select_cdf_kernel<false, false, 16><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
-            else select_cdf_kernel<false><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
+            if (P.fanout[l] <= 16) select_cdf_kernel<SRC_HUB, 16><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
+            else select_cdf_kernel<SRC_HUB><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
             CSAW_CUDA(cudaGetLastError());
         }
     }
@@ -2086,7 +2326,7 @@ static csaw_status alloc_common(Pipeline& P, Alloc&& get)
     CSAW_TRY(get((void**)&P.ctr, sizeof(uint64_t) * CT_WORDS));
     CSAW_TRY(get(&P.scan_scr, scan_scratch_bytes(0)));
     CSAW_TRY(get(&P.sort_scr, sort_scratch_bytes(0)));
-    if (P.cta_slots) {
+    if (P.cta_slots()) {
         CSAW_TRY(get((void**)&P.hub_S, sizeof(uint64_t) * (size_t)P.sel_blocks * P.g->max_degree));
         CSAW_TRY(get((void**)&P.hub_bits, sizeof(uint32_t) * (size_t)P.sel_blocks * ((P.g->max_degree + 31) / 32)));
     }
@@ -2101,18 +2341,21 @@ static csaw_status alloc_common(Pipeline& P, Alloc&& get)
     return CSAW_OK;
 }
 
-// Hub grouping buffers for layers of up to `cap` frontier entries.
+// Hub buffers for layers of up to `cap` frontier entries: the list, the sort
+// into vertex order, and the grouping of shared hub arrays, as the path needs.
 template <class Alloc>
 static csaw_status alloc_hub(Pipeline& P, uint64_t cap, Alloc&& get)
 {
     P.hub_cap = cap;
     const uint64_t c = cap ? cap : 1;
     CSAW_TRY(get((void**)&P.hlist, sizeof(uint32_t) * c));
+    if (!P.hub_path && !P.hub_order) return CSAW_OK;
     CSAW_TRY(get((void**)&P.hkeys, sizeof(uint64_t) * c));
     CSAW_TRY(get((void**)&P.halt, sizeof(uint64_t) * c));
+    CSAW_TRY(get((void**)&P.item_e, sizeof(uint32_t) * c));
+    if (!P.hub_path) return CSAW_OK;
     CSAW_TRY(get((void**)&P.hflag, sizeof(uint32_t) * c));
     CSAW_TRY(get((void**)&P.hpos, sizeof(uint64_t) * (c + 1)));
-    CSAW_TRY(get((void**)&P.item_e, sizeof(uint32_t) * c));
     CSAW_TRY(get((void**)&P.item_h, sizeof(uint32_t) * c));
     CSAW_TRY(get((void**)&P.hubH, sizeof(uint32_t) * c));
     CSAW_TRY(get((void**)&P.hubD, sizeof(uint32_t) * c));
@@ -2300,6 +2543,18 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
         P.inst_id = tabs->inst_id;
         P.inst_fan = tabs->inst_fan;
     }
+    if (!layer_mode && sample_array_pays(P, n_seeds)) {
+        uint64_t* words = nullptr;
+        const csaw_status st = get((void**)&words, sizeof(uint64_t) * pack_layout(g->E, g->V).words);
+        if (st == CSAW_OK) {
+            CSAW_TRY(enqueue_pack_build(g, kind, words, s));
+            P.use_pack(words);
+        } else if (st == CSAW_ERR_NOMEM) {
+            clear_error();   // no room: streamed
+        } else {
+            return st;
+        }
+    }
     CSAW_TRY(alloc_common(P, get));
     CSAW_CUDA(cudaMemsetAsync(P.ctr, 0, sizeof(uint64_t) * CT_WORDS, s));
     CSAW_TRY(alloc_entries(P, 0, n_seeds, get));
@@ -2307,7 +2562,7 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
     R->src.assign(depth, nullptr);
     R->dst.assign(depth, nullptr);
     R->layer_edges.assign(depth, 0);
-    const bool hubs = (P.hub_path || P.hub_order) && !layer_mode;
+    const bool hubs = (P.hub_path || P.hub_order || P.pack) && !layer_mode;
     // layer sampling: the graph's packed array, or one built for the call
     const uint64_t* pack = nullptr;
     if (layer_mode && P.kind != CSAW_BIAS_UNIFORM && !P.zero_bias && attempt_cap >= LD_MIN_CAP) {
@@ -2633,6 +2888,12 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
         pl->allocs.push_back(*p);
         return CSAW_OK;
     };
+    // the packed array of a large plan, built in every run
+    uint64_t* pack = nullptr;
+    if (sample_array_pays(P, max_seeds)) {
+        if (get((void**)&pack, sizeof(uint64_t) * pack_layout(g->E, g->V).words) == CSAW_OK) P.use_pack(pack);
+        else clear_error();   // no room: streamed
+    }
     csaw_status st = alloc_common(P, get);
     // Upper bounds: a layer emits at most min(k, max degree) edges per
     // frontier vertex; a frontier is at most the previous layer's edges and
@@ -2646,7 +2907,7 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
         if (st == CSAW_OK) st = alloc_edges(P, l, e, get, get);
         f = e < fmax ? e : fmax;
     }
-    if (st == CSAW_OK && P.hub_order) st = alloc_hub(P, f_max, get);   // vertex order of hub items
+    if (st == CSAW_OK && (P.hub_order || P.pack)) st = alloc_hub(P, f_max, get);   // hub items over an array
     if (st == CSAW_OK && P.hub_path) {
         // shared hub prefix sums: at most every edge of the rows above
         // theta_w, and at most max degree per hub item
@@ -2679,6 +2940,7 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
     if (e == cudaSuccess) {
         e = cudaMemsetAsync(P.ctr, 0, sizeof(uint64_t) * CT_WORDS, cs);
         if (e != cudaSuccess) st = cuda_fail(e, "memset");
+        if (st == CSAW_OK && pack) st = enqueue_pack_build(g, kind, pack, cs);
         if (st == CSAW_OK) st = enqueue_frontier0(P, pl->in_seeds, pl->in_io, cs);
         for (uint32_t l = 0; st == CSAW_OK && l < depth; ++l) {
             st = enqueue_count(P, l, cs);
@@ -3023,6 +3285,7 @@ extern "C" csaw_status csaw_sample_oom(const uint64_t* row_offsets, const uint32
 
         Pipeline P;
         P.init(&view, eff_kind, n_instances, depth, fanout, rng_seed);
+        P.take = false;   // whole rows are listed with the loaded partition's warp items
         P.seeds_cap = n_seeds;
         st = alloc_common(P, get);
         if (st == CSAW_OK) {
@@ -3222,7 +3485,7 @@ extern "C" csaw_status csaw_autotune_select(csaw_graph* g, const uint32_t* seeds
     CSAW_TRY(check_bias(g, bias, false, &kind));
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t thetas[] = {32, 64, 128, 256};
-    const int occ = select_occupancy(kind);
+    const int occ = select_occupancy(kind, select_wide(g, kind));
     cudaEvent_t e0, e1;
     CSAW_CUDA(cudaEventCreate(&e0));
     CSAW_CUDA(cudaEventCreate(&e1));
@@ -3381,7 +3644,7 @@ extern "C" csaw_status csaw_select_noalloc(csaw_graph* g, const uint32_t* vertic
     if (device != g->device)
         return fail(CSAW_ERR_INVALID, "the current device (%d) is not the graph's device (%d)", device,
                     g->device);
-    int sel_blocks = select_blocks(kind, g->sm_count);
+    int sel_blocks = g->sm_count * select_occupancy(kind, select_wide(g, kind));
     if (g->max_degree > CTA_SMEM_DEG) {
         const uint64_t slot = (uint64_t)g->max_degree * 8 + ((uint64_t)g->max_degree + 31) / 32 * 4;
         const uint64_t slots = (CSAW_NOALLOC_SCRATCH_BYTES - NA_HUB) / slot;
@@ -3447,11 +3710,7 @@ extern "C" csaw_status csaw_select_noalloc(csaw_graph* g, const uint32_t* vertic
         sp.scratch_bits = (uint32_t*)(hub + (size_t)sel_blocks * g->max_degree * 8);
         sp.scratch_stride = g->max_degree;
         sp.cdf = nullptr; sp.skip_warp_items = false; sp.attempt_cap = CSAW_ATTEMPT_CAP;
-        switch (kind) {
-        case CSAW_BIAS_UNIFORM: CSAW_TRY(launch_select<CSAW_BIAS_UNIFORM>(sp, sel_blocks, s)); break;
-        case CSAW_BIAS_EDGE_WEIGHT: CSAW_TRY(launch_select<CSAW_BIAS_EDGE_WEIGHT>(sp, sel_blocks, s)); break;
-        default: CSAW_TRY(launch_select<CSAW_BIAS_NEIGHBOR_DEGREE>(sp, sel_blocks, s)); break;
-        }
+        CSAW_TRY(launch_select(kind, select_wide(g, kind), sp, sel_blocks, s));
     }
     return CSAW_OK;
 }
