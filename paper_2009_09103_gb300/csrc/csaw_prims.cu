@@ -5,17 +5,16 @@
 // fixed grid whose blocks each own a contiguous range of tiles.  Frontier
 // compaction (Update, Eq. 4: the next frontier is the sorted set of picks
 // minus the visited set) is built from these two.
-#include "csaw_internal.cuh"
+#include "csaw_scan.cuh"
 
 namespace csaw {
 
 // ---------------------------------------------------------------- scan
-constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = 8;
-constexpr uint64_t SCAN_TILE = (uint64_t)SCAN_THREADS * SCAN_ITEMS;
-constexpr int SCAN_MAX_BLOCKS = 1024;
+// Up to this many tiles one block scans in about the time that a second
+// launch takes.
+constexpr int SCAN_ONE_TILES = 4;
 
-static int scan_blocks(uint64_t n_max)
+int scan_blocks(uint64_t n_max)
 {
     uint64_t tiles = (n_max + SCAN_TILE - 1) / SCAN_TILE;
     if (tiles < 1) tiles = 1;
@@ -23,37 +22,6 @@ static int scan_blocks(uint64_t n_max)
 }
 
 size_t scan_scratch_bytes(uint64_t) { return sizeof(uint64_t) * (SCAN_MAX_BLOCKS + 1); }
-
-__device__ __forceinline__ void block_range(uint64_t n, uint64_t tile, uint64_t* lo, uint64_t* hi)
-{
-    const uint64_t tiles = (n + tile - 1) / tile;
-    const uint64_t per = (tiles + gridDim.x - 1) / gridDim.x;
-    uint64_t b = (uint64_t)blockIdx.x * per * tile;
-    uint64_t e = b + per * tile;
-    *lo = b < n ? b : n;
-    *hi = e < n ? e : n;
-}
-
-// Block-wide exclusive scan of one uint64 per thread; returns the block total.
-__device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* excl, uint64_t* s_warp)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint64_t incl = warp_inclusive_scan_u64(v, lane);
-    if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        uint64_t t = lane < nw ? s_warp[lane] : 0;
-        const uint64_t ti = warp_inclusive_scan_u64(t, lane);
-        if (lane < nw) s_warp[lane] = ti - t;
-        if (lane == nw - 1) s_warp[32] = ti;
-    }
-    __syncthreads();
-    *excl = s_warp[wid] + incl - v;
-    const uint64_t total = s_warp[32];
-    __syncthreads();
-    return total;
-}
 
 __global__ void scan_reduce_kernel(const uint32_t* __restrict__ in, const uint64_t* __restrict__ n_dev,
                                    uint64_t* __restrict__ bsum)
@@ -68,46 +36,41 @@ __global__ void scan_reduce_kernel(const uint32_t* __restrict__ in, const uint64
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
-__global__ void scan_top_kernel(uint64_t* __restrict__ bsum, int nblocks, uint64_t* __restrict__ total_out)
-{
-    __shared__ uint64_t s_warp[33];
-    // nblocks <= 1024 = blockDim: one value per thread
-    const uint64_t v = (int)threadIdx.x < nblocks ? bsum[threadIdx.x] : 0;
-    uint64_t excl;
-    const uint64_t total = block_exclusive_scan(v, &excl, s_warp);
-    if ((int)threadIdx.x < nblocks) bsum[threadIdx.x] = excl;
-    if (threadIdx.x == 0 && total_out) *total_out = total;
-}
-
-__global__ void scan_down_kernel(const uint32_t* __restrict__ in, const uint64_t* __restrict__ n_dev,
-                                 const uint64_t* __restrict__ boff, uint64_t* __restrict__ out)
+// Each block adds up the totals of the blocks before it itself (at most 1,024
+// words from L2), which is cheaper than a launch between the two passes.
+__global__ void __launch_bounds__(SCAN_THREADS) scan_down_kernel(const uint32_t* __restrict__ in,
+                                                                 const uint64_t* __restrict__ n_dev,
+                                                                 const uint64_t* __restrict__ bsum,
+                                                                 uint64_t* __restrict__ out,
+                                                                 uint64_t* __restrict__ total_out)
 {
     __shared__ uint64_t s_warp[33];
     const uint64_t n = *n_dev;
     uint64_t lo, hi;
     block_range(n, SCAN_TILE, &lo, &hi);
-    uint64_t base = boff[blockIdx.x];
-    for (uint64_t t0 = lo; t0 < hi; t0 += SCAN_TILE) {
-        const uint64_t my = t0 + (uint64_t)threadIdx.x * SCAN_ITEMS;
-        uint32_t v[SCAN_ITEMS];
-        uint64_t s = 0;
-#pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-            v[j] = (my + j < hi) ? in[my + j] : 0u;
-            s += v[j];
-        }
-        uint64_t excl;
-        const uint64_t total = block_exclusive_scan(s, &excl, s_warp);
-        uint64_t run = base + excl;
-#pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-            if (my + j < hi) out[my + j] = run;
-            run += v[j];
-        }
-        base += total;
-    }
+    uint64_t base = sum_before(bsum, blockIdx.x, s_warp);
+    for (uint64_t t0 = lo; t0 < hi; t0 += SCAN_TILE) base += scan_tile(in, t0, hi, base, out, s_warp);
     // the last block writes out[n] = grand total
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = base;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        out[n] = base;
+        if (total_out) *total_out = base;
+    }
+}
+
+// The whole scan by one block.
+__global__ void __launch_bounds__(SCAN_THREADS) scan_one_kernel(const uint32_t* __restrict__ in,
+                                                                const uint64_t* __restrict__ n_dev,
+                                                                uint64_t* __restrict__ out,
+                                                                uint64_t* __restrict__ total_out)
+{
+    __shared__ uint64_t s_warp[33];
+    const uint64_t n = *n_dev;
+    uint64_t base = 0;
+    for (uint64_t t0 = 0; t0 < n; t0 += SCAN_TILE) base += scan_tile(in, t0, n, base, out, s_warp);
+    if (threadIdx.x == 0) {
+        out[n] = base;
+        if (total_out) *total_out = base;
+    }
 }
 
 // out[i] = sum of in[0..i) for i <= n; *total_out (optional, device) = out[n].
@@ -116,9 +79,12 @@ csaw_status scan_u32(const uint32_t* in, uint64_t* out, const uint64_t* n_dev, u
 {
     const int nb = scan_blocks(n_max);
     uint64_t* bsum = (uint64_t*)scratch;
-    scan_reduce_kernel<<<nb, SCAN_THREADS, 0, s>>>(in, n_dev, bsum);
-    scan_top_kernel<<<1, SCAN_MAX_BLOCKS, 0, s>>>(bsum, nb, total_out);
-    scan_down_kernel<<<nb, SCAN_THREADS, 0, s>>>(in, n_dev, bsum, out);
+    if (nb <= SCAN_ONE_TILES) {
+        scan_one_kernel<<<1, SCAN_THREADS, 0, s>>>(in, n_dev, out, total_out);
+    } else {
+        scan_reduce_kernel<<<nb, SCAN_THREADS, 0, s>>>(in, n_dev, bsum);
+        scan_down_kernel<<<nb, SCAN_THREADS, 0, s>>>(in, n_dev, bsum, out, total_out);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "scan kernels");
     return CSAW_OK;
@@ -136,6 +102,9 @@ constexpr int SORT_ROUNDS = 8;                                       // 32-key r
 constexpr uint64_t SORT_TILE = (uint64_t)SORT_THREADS * SORT_ROUNDS; // 2048 keys
 constexpr int SORT_MAX_BLOCKS = 1024;
 constexpr int RADIX = 256;
+// Up to this many blocks the scatter adds the blocks' counts up itself (so
+// many loads a thread, in flight together) instead of after a scan launch.
+constexpr int SORT_DIRECT_BLOCKS = 64;
 
 static int sort_blocks(uint64_t n_max, int sm_count)
 {
@@ -150,7 +119,8 @@ size_t sort_scratch_bytes(uint64_t) { return sizeof(uint32_t) * ((size_t)RADIX *
 
 __global__ void __launch_bounds__(SORT_THREADS) sort_hist_kernel(const uint64_t* __restrict__ keys,
                                                                  const uint64_t* __restrict__ n_dev,
-                                                                 int shift, uint32_t* __restrict__ hist)
+                                                                 int shift, uint32_t* __restrict__ hist,
+                                                                 bool direct)
 {
     __shared__ uint32_t s_h[RADIX];
     for (int i = threadIdx.x; i < RADIX; i += SORT_THREADS) s_h[i] = 0;
@@ -160,7 +130,8 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_hist_kernel(const uint64_t*
     for (uint64_t i = lo + threadIdx.x; i < hi; i += SORT_THREADS)
         atomicAdd(&s_h[(keys[i] >> shift) & (RADIX - 1)], 1u);
     __syncthreads();
-    for (int d = threadIdx.x; d < RADIX; d += SORT_THREADS) hist[(size_t)d * gridDim.x + blockIdx.x] = s_h[d];
+    for (int d = threadIdx.x; d < RADIX; d += SORT_THREADS)
+        hist[direct ? (size_t)blockIdx.x * RADIX + d : (size_t)d * gridDim.x + blockIdx.x] = s_h[d];
 }
 
 // Exclusive scan of each digit's per-block counts, in place (one CTA per
@@ -187,7 +158,7 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_scatter_kernel(const uint64
                                                                     const uint64_t* __restrict__ n_dev,
                                                                     int shift,
                                                                     const uint32_t* __restrict__ hist,
-                                                                    const uint32_t* __restrict__ dtot)
+                                                                    const uint32_t* __restrict__ dtot, bool direct)
 {
     __shared__ uint32_t s_base[RADIX];             // next output slot of each digit for this block
     __shared__ uint32_t s_cnt[SORT_WARPS][RADIX];  // per-warp digit counts, then warp offsets
@@ -196,9 +167,23 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_scatter_kernel(const uint64
     {
         // start of each digit = earlier digits' totals + earlier blocks' counts
         static_assert(SORT_THREADS == RADIX, "one digit per thread");
+        uint32_t total, before;
+        if (direct) {
+            // few blocks: every one adds their counts up itself
+            total = before = 0;
+#pragma unroll 8
+            for (uint32_t k = 0; k < gridDim.x; ++k) {
+                const uint32_t c = hist[(size_t)k * RADIX + threadIdx.x];
+                before += k < blockIdx.x ? c : 0u;
+                total += c;
+            }
+        } else {
+            total = dtot[threadIdx.x];
+            before = hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x];
+        }
         uint64_t digit_base;
-        block_exclusive_scan(dtot[threadIdx.x], &digit_base, s_warp);
-        s_base[threadIdx.x] = (uint32_t)digit_base + hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x];
+        block_exclusive_scan(total, &digit_base, s_warp);
+        s_base[threadIdx.x] = (uint32_t)digit_base + before;
     }
     uint64_t lo, hi;
     block_range(*n_dev, SORT_TILE, &lo, &hi);
@@ -257,14 +242,15 @@ csaw_status radix_sort_u64(uint64_t* keys, uint64_t* alt, const uint64_t* n_dev,
 {
     if (n_max >= 0xFFFFFFFFull) return fail(CSAW_ERR_INVALID, "radix sort limited to 2^32-1 keys");
     const int nb = sort_blocks(n_max, sm_count);
+    const bool direct = nb <= SORT_DIRECT_BLOCKS;
     uint32_t* hist = (uint32_t*)scratch;
     uint32_t* dtot = hist + (size_t)RADIX * SORT_MAX_BLOCKS;
     uint64_t* src = keys;
     uint64_t* dst = alt;
     for (int shift = 0; shift < bits; shift += 8) {
-        sort_hist_kernel<<<nb, SORT_THREADS, 0, s>>>(src, n_dev, shift, hist);
-        sort_scan_kernel<<<RADIX, 256, 0, s>>>(hist, nb, dtot);
-        sort_scatter_kernel<<<nb, SORT_THREADS, 0, s>>>(src, dst, n_dev, shift, hist, dtot);
+        sort_hist_kernel<<<nb, SORT_THREADS, 0, s>>>(src, n_dev, shift, hist, direct);
+        if (!direct) sort_scan_kernel<<<RADIX, 256, 0, s>>>(hist, nb, dtot);
+        sort_scatter_kernel<<<nb, SORT_THREADS, 0, s>>>(src, dst, n_dev, shift, hist, dtot, direct);
         uint64_t* t = src; src = dst; dst = t;
     }
     cudaError_t e = cudaGetLastError();

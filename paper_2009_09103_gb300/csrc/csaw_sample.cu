@@ -38,7 +38,7 @@
 #include <type_traits>
 #include <vector>
 
-#include "csaw_internal.cuh"
+#include "csaw_scan.cuh"
 
 namespace csaw {
 
@@ -1115,38 +1115,74 @@ struct Visited {
     int n;
 };
 
-// kept[i] = 1 for the first of each run of equal sorted keys that no earlier
-// frontier of its instance holds.
-__global__ void unique_filter_kernel(const uint64_t* __restrict__ sorted, const uint64_t* n_dev,
-                                     Visited vis, uint32_t vbits, uint32_t* __restrict__ kept)
+// Whether an earlier frontier of its instance holds key.
+__device__ __forceinline__ bool visited_before(const Visited& vis, uint64_t key, uint32_t vbits)
 {
-    const uint64_t n = *n_dev;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t key = sorted[i];
-        bool keep = i == 0 || sorted[i - 1] != key;
-        const uint32_t inst = (uint32_t)(key >> vbits);
-        for (int j = 0; j < vis.n && keep; ++j) {
-            uint64_t lo = vis.foff[j][inst], hi = vis.foff[j][inst + 1];
-            const uint64_t end = hi;
-            while (lo < hi) {
-                const uint64_t mid = lo + ((hi - lo) >> 1);
-                if (vis.keys[j][mid] < key) lo = mid + 1; else hi = mid;
-            }
-            if (lo < end && vis.keys[j][lo] == key) keep = false;
+    const uint32_t inst = (uint32_t)(key >> vbits);
+    for (int j = 0; j < vis.n; ++j) {
+        uint64_t lo = vis.foff[j][inst], hi = vis.foff[j][inst + 1];
+        const uint64_t end = hi;
+        while (lo < hi) {
+            const uint64_t mid = lo + ((hi - lo) >> 1);
+            if (vis.keys[j][mid] < key) lo = mid + 1; else hi = mid;
         }
-        kept[i] = keep ? 1u : 0u;
+        if (lo < end && vis.keys[j][lo] == key) return true;
     }
+    return false;
 }
 
-__global__ void scatter_kept_kernel(const uint64_t* __restrict__ sorted, const uint64_t* n_dev,
-                                    const uint32_t* __restrict__ kept, const uint64_t* __restrict__ kpos,
-                                    uint64_t* __restrict__ out)
+// kept[i] = 1 for the first of each run of equal sorted keys that no earlier
+// frontier of its instance holds; bsum: how many each block's range keeps.
+__global__ void __launch_bounds__(SCAN_THREADS) frontier_flag_kernel(const uint64_t* __restrict__ sorted,
+                                                                     const uint64_t* n_dev, Visited vis,
+                                                                     uint32_t vbits, uint32_t* __restrict__ kept,
+                                                                     uint64_t* __restrict__ bsum)
 {
-    const uint64_t n = *n_dev;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        if (kept[i]) out[kpos[i]] = sorted[i];
+    __shared__ uint64_t s_warp[33];
+    uint64_t lo, hi, count = 0, excl;
+    block_range(*n_dev, SCAN_TILE, &lo, &hi);
+    for (uint64_t i = lo + threadIdx.x; i < hi; i += SCAN_THREADS) {
+        const uint64_t key = sorted[i];
+        const bool keep = (i == 0 || sorted[i - 1] != key) && !visited_before(vis, key, vbits);
+        kept[i] = keep ? 1u : 0u;
+        count += keep;
+    }
+    const uint64_t total = block_exclusive_scan(count, &excl, s_warp);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = total;
+}
+
+// The kept keys, in order, to out; *n_out: how many.
+__global__ void __launch_bounds__(SCAN_THREADS) frontier_scatter_kernel(const uint64_t* __restrict__ sorted,
+                                                                        const uint64_t* n_dev,
+                                                                        const uint32_t* __restrict__ kept,
+                                                                        const uint64_t* __restrict__ bsum,
+                                                                        uint64_t* __restrict__ out,
+                                                                        uint64_t* __restrict__ n_out)
+{
+    __shared__ uint64_t s_warp[33];
+    __shared__ uint32_t s_cnt[2][SCAN_THREADS / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t lo, hi;
+    block_range(*n_dev, SCAN_TILE, &lo, &hi);
+    uint64_t base = sum_before(bsum, blockIdx.x, s_warp);
+    int flip = 0;
+    for (uint64_t t0 = lo; t0 < hi; t0 += SCAN_THREADS, flip ^= 1) {
+        const uint64_t i = t0 + threadIdx.x;
+        const bool keep = i < hi && kept[i];
+        const uint32_t bal = __ballot_sync(CSAW_FULL_MASK, keep);
+        if (lane == 0) s_cnt[flip][wid] = __popc(bal);
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int k = 0; k < SCAN_THREADS / 32; ++k) {
+            const uint32_t c = s_cnt[flip][k];
+            before += k < wid ? c : 0u;
+            total += c;
+        }
+        if (keep) out[base + before + __popc(bal & lanemask_lt())] = sorted[i];
+        base += total;
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_out = base;
 }
 
 // foff[i] = first position of instance i in the sorted frontier, i <= n_inst.
@@ -1181,6 +1217,172 @@ __global__ void layer_offsets_kernel(const uint64_t* __restrict__ foff, const ui
         eoff[i] = e;
         if (i < n_inst) fsize[i] = foff[i + 1] - foff[i];
         else *next_base = e;
+    }
+}
+
+// The positions of a layer's picks and the layer's offsets (scan_u32 and
+// layer_offsets_kernel) by one block, for small frontiers.
+constexpr uint64_t SMALL_SCAN = 4 * SCAN_TILE;
+
+__global__ void __launch_bounds__(SCAN_THREADS) small_offsets_kernel(
+    const uint32_t* __restrict__ cnt, const uint64_t* n_dev, uint64_t* pos, uint64_t* __restrict__ total_out,
+    const uint64_t* __restrict__ foff, uint32_t n_inst, const uint64_t* __restrict__ base_dev,
+    uint64_t* __restrict__ eoff, uint64_t* __restrict__ fsize, uint64_t* __restrict__ next_base)
+{
+    __shared__ uint64_t s_warp[33];
+    const uint64_t n = *n_dev, first = *base_dev;
+    uint64_t total = 0;
+    for (uint64_t t0 = 0; t0 < n; t0 += SCAN_TILE) total += scan_tile(cnt, t0, n, total, pos, s_warp);
+    if (threadIdx.x == 0) {
+        pos[n] = total;
+        *total_out = total;
+    }
+    __syncthreads();
+    for (uint64_t i = threadIdx.x; i <= n_inst; i += SCAN_THREADS) {
+        const uint64_t a = foff[i], e = first + pos[a];
+        eoff[i] = e;
+        if (i < n_inst) fsize[i] = foff[i + 1] - a;
+        else *next_base = e;
+    }
+}
+
+// A whole frontier from at most SF_KEYS seeds or picks by one block: keys,
+// stable radix sort in shared memory, first of equal keys that the instance
+// has not visited, in order, and the instances' bounds.  A small frontier is
+// all launches otherwise (14 for the seeds, 11 and more for a layer): a plan of
+// 256 seeds and two layers on RMAT s12 takes 71 us with this and the offsets
+// in one block, 109 us without.
+constexpr int SF_THREADS = 1024, SF_WARPS = SF_THREADS / 32;
+constexpr uint32_t SF_KEYS = 4096;
+constexpr int SF_PER = (int)SF_KEYS / SF_THREADS;
+constexpr size_t SF_SMEM = 2 * SF_KEYS * sizeof(uint64_t) + SF_WARPS * 256 * sizeof(uint16_t) + 256 * sizeof(uint32_t);
+
+struct SmallFrontier {
+    const uint32_t* seeds = nullptr;      // layer 0: seeds and their instances' offsets
+    const uint64_t* inst_off = nullptr;
+    uint64_t cap = 0;                     // at most this many seeds
+    uint64_t* n_seeds = nullptr;          // receives their number
+    uint32_t V = 0;
+    uint32_t* err = nullptr;
+    const uint64_t* cand = nullptr;       // later layers: candidate keys and their number
+    const uint64_t* n_cand = nullptr;
+    Visited vis;
+    uint32_t n_inst = 0, vbits = 0;
+    int kbits = 0;
+    uint64_t* F = nullptr;
+    uint64_t* FO = nullptr;
+    uint64_t* n_out = nullptr;
+};
+
+__global__ void __launch_bounds__(SF_THREADS) small_frontier_kernel(SmallFrontier p)
+{
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    uint64_t* a = (uint64_t*)s_dyn;
+    uint64_t* b = a + SF_KEYS;
+    uint16_t (*cnt)[256] = (uint16_t (*)[256])(b + SF_KEYS);        // per warp: digit counts, then offsets
+    uint32_t* dbase = (uint32_t*)(cnt + SF_WARPS);
+    __shared__ uint64_t s_warp[33];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    uint32_t n;
+    if (p.seeds || p.inst_off) {
+        uint64_t total = p.inst_off[p.n_inst];
+        if (tid == 0) {
+            if (p.inst_off[0] != 0) atomicOr(p.err, 2u);
+            if (total > p.cap) atomicOr(p.err, 4u);
+            *p.n_seeds = total < p.cap ? total : p.cap;
+        }
+        for (uint64_t i = tid; i < p.n_inst; i += SF_THREADS)
+            if (p.inst_off[i + 1] < p.inst_off[i]) atomicOr(p.err, 2u);
+        n = (uint32_t)(total < p.cap ? total : p.cap);
+        for (uint32_t j = tid; j < n; j += SF_THREADS) {
+            uint32_t lo = 0, hi = p.n_inst;   // instance = last i with inst_off[i] <= j
+            while (lo < hi) {
+                const uint32_t mid = (uint32_t)(((uint64_t)lo + hi + 1) >> 1);
+                if (p.inst_off[mid] <= j) lo = mid; else hi = mid - 1;
+            }
+            const uint32_t sd = p.seeds[j];
+            if (sd >= p.V) atomicOr(p.err, 1u);
+            a[j] = ((uint64_t)lo << p.vbits) | (sd < p.V ? sd : 0u);
+        }
+    } else {
+        n = (uint32_t)*p.n_cand;
+        for (uint32_t j = tid; j < n; j += SF_THREADS) a[j] = p.cand[j];
+    }
+    const uint32_t lt = lanemask_lt();
+    for (int shift = 0; shift < p.kbits; shift += 8) {
+        for (int i = tid; i < SF_WARPS * 256 / 2; i += SF_THREADS) ((uint32_t*)cnt)[i] = 0u;
+        __syncthreads();
+        // a warp ranks 32 * SF_PER consecutive keys, 32 at a time
+        uint64_t k[SF_PER];
+        uint32_t dig[SF_PER], loc[SF_PER];
+#pragma unroll
+        for (int r = 0; r < SF_PER; ++r) {
+            const uint32_t i = (uint32_t)(wid * SF_PER + r) * 32u + lane;
+            dig[r] = 256u;
+            if ((uint32_t)(wid * SF_PER + r) * 32u >= n) continue;   // the whole warp
+            k[r] = i < n ? a[i] : 0;
+            if (i < n) dig[r] = (uint32_t)(k[r] >> shift) & 255u;
+            const uint32_t peers = __match_any_sync(CSAW_FULL_MASK, dig[r]);
+            const int leader = __ffs(peers) - 1;
+            uint32_t before = 0;
+            if (lane == leader && dig[r] < 256u) {
+                before = cnt[wid][dig[r]];
+                cnt[wid][dig[r]] = (uint16_t)(before + __popc(peers));
+            }
+            before = __shfl_sync(CSAW_FULL_MASK, before, leader);
+            loc[r] = before + __popc(peers & lt);
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t run = 0;
+        if (tid < 256)
+            for (int w = 0; w < SF_WARPS; ++w) {
+                const uint32_t c = cnt[w][tid];
+                cnt[w][tid] = (uint16_t)run;
+                run += c;
+            }
+        uint64_t excl;
+        block_exclusive_scan(tid < 256 ? run : 0u, &excl, s_warp);
+        if (tid < 256) dbase[tid] = (uint32_t)excl;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SF_PER; ++r)
+            if (dig[r] < 256u) b[dbase[dig[r]] + cnt[wid][dig[r]] + loc[r]] = k[r];
+        __syncthreads();
+        uint64_t* t = a;
+        a = b;
+        b = t;
+    }
+    __syncthreads();
+    // distinct and not visited, compacted into b and the frontier
+    bool keep[SF_PER];
+    uint32_t mine = 0;
+#pragma unroll
+    for (int r = 0; r < SF_PER; ++r) {
+        const uint32_t i = (uint32_t)tid * SF_PER + r;
+        keep[r] = i < n && (i == 0 || a[i - 1] != a[i]) && !visited_before(p.vis, a[i], p.vbits);
+        mine += keep[r];
+    }
+    uint64_t at;
+    const uint32_t kept = (uint32_t)block_exclusive_scan(mine, &at, s_warp);
+#pragma unroll
+    for (int r = 0; r < SF_PER; ++r)
+        if (keep[r]) {
+            const uint64_t key = a[tid * SF_PER + r];
+            b[at] = key;
+            p.F[at] = key;
+            ++at;
+        }
+    if (tid == 0) *p.n_out = kept;
+    __syncthreads();
+    for (uint64_t i = tid; i <= p.n_inst; i += SF_THREADS) {
+        uint32_t lo = 0, hi = kept;
+        const uint64_t key = i << p.vbits;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (b[mid] < key) lo = mid + 1; else hi = mid;
+        }
+        p.FO[i] = i == p.n_inst ? kept : lo;
     }
 }
 
@@ -1935,6 +2137,7 @@ __global__ void __launch_bounds__(LD_THREADS) layer_draw_kernel(LayerSelParams P
 
 struct LayerBufs {
     uint64_t f_cap = 0, e_cap = 0;
+    bool offsets_done = false;   // with the edge positions (small frontiers)
     uint64_t* F = nullptr;       // frontier keys [f_cap], sorted
     uint64_t* FO = nullptr;      // instance bounds [n_inst + 1]
     uint32_t* cnt = nullptr;     // [f_cap]
@@ -1946,7 +2149,6 @@ struct LayerBufs {
     uint64_t* cand = nullptr;    // [e_cap] candidate keys (not on the last layer)
     uint64_t* cand_alt = nullptr;
     uint32_t* kept = nullptr;
-    uint64_t* kpos = nullptr;    // [e_cap + 1]
 };
 
 struct Pipeline {
@@ -1983,7 +2185,6 @@ struct Pipeline {
     uint64_t* seed_keys = nullptr;       // [seeds_cap]
     uint64_t* seed_alt = nullptr;
     uint32_t* seed_kept = nullptr;
-    uint64_t* seed_kpos = nullptr;       // [seeds_cap + 1]
     LayerBufs L[CSAW_MAX_DEPTH];
     // hub grouping of one layer at a time (hub_cap items), and the shared
     // hub prefix sums (hubS_cap entries)
@@ -2087,12 +2288,46 @@ static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
     return P.n_inst > 1 ? 150e6 + 150.0 * entries >= cost : 2.0 * reached * visited >= cost + 40e6;
 }
 
+// The frontier from n_max sorted keys at most: flags and block sums, then the
+// kept keys in order.
+static void launch_frontier(const uint64_t* sorted, const uint64_t* n_dev, uint64_t n_max, const Visited& vis,
+                            uint32_t vbits, uint32_t* kept, void* scratch, uint64_t* F, uint64_t* n_out,
+                            cudaStream_t s)
+{
+    const int nb = scan_blocks(n_max);
+    frontier_flag_kernel<<<nb, SCAN_THREADS, 0, s>>>(sorted, n_dev, vis, vbits, kept, (uint64_t*)scratch);
+    frontier_scatter_kernel<<<nb, SCAN_THREADS, 0, s>>>(sorted, n_dev, kept, (const uint64_t*)scratch, F, n_out);
+}
+
+// Layer l's frontier by one block.
+static csaw_status launch_small_frontier(const Pipeline& P, SmallFrontier& sf, uint32_t l, cudaStream_t s)
+{
+    sf.n_inst = P.n_inst; sf.vbits = (uint32_t)P.vbits; sf.kbits = P.kbits;
+    sf.F = P.L[l].F; sf.FO = P.L[l].FO; sf.n_out = P.lc(l, L_N);
+    // the attribute is set before the flag is published: calls may come from several threads
+    static std::atomic<bool> ready{false};
+    if (!ready.load(std::memory_order_acquire)) {
+        CSAW_CUDA(cudaFuncSetAttribute(small_frontier_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SF_SMEM));
+        ready.store(true, std::memory_order_release);
+    }
+    small_frontier_kernel<<<1, SF_THREADS, SF_SMEM, s>>>(sf);
+    CSAW_CUDA(cudaGetLastError());
+    return CSAW_OK;
+}
+
 // Layer-0 frontier: sorted distinct (instance, seed) keys.
 static csaw_status enqueue_frontier0(Pipeline& P, const uint32_t* seeds, const uint64_t* inst_off,
                                      cudaStream_t s)
 {
     csaw_graph* g = P.g;
     const uint64_t cap = P.seeds_cap;
+    if (cap <= SF_KEYS) {
+        SmallFrontier sf;
+        sf.seeds = seeds; sf.inst_off = inst_off; sf.cap = cap; sf.n_seeds = P.ctr + CT_NSEEDS;
+        sf.V = g->V; sf.err = (uint32_t*)(P.ctr + CT_ERR);
+        sf.vis.n = 0;
+        return launch_small_frontier(P, sf, 0, s);
+    }
     check_inst_off_kernel<<<grid_for(P.n_inst, 256, g->sm_count), 256, 0, s>>>(inst_off, P.n_inst, (uint32_t*)(P.ctr + CT_ERR));
     seed_keys_kernel<<<grid_for(cap, 256, g->sm_count), 256, 0, s>>>(
         seeds, inst_off, P.n_inst, cap, g->V, P.vbits, P.seed_keys, (uint32_t*)(P.ctr + CT_ERR), P.ctr + CT_NSEEDS);
@@ -2100,9 +2335,7 @@ static csaw_status enqueue_frontier0(Pipeline& P, const uint32_t* seeds, const u
     if (cap) CSAW_TRY(radix_sort_u64(P.seed_keys, P.seed_alt, P.ctr + CT_NSEEDS, cap, P.kbits, g->sm_count, P.sort_scr, s, &sorted));
     Visited none;
     none.n = 0;
-    unique_filter_kernel<<<grid_for(cap, 256, g->sm_count), 256, 0, s>>>(sorted, P.ctr + CT_NSEEDS, none, P.vbits, P.seed_kept);
-    CSAW_TRY(scan_u32(P.seed_kept, P.seed_kpos, P.ctr + CT_NSEEDS, cap, P.scan_scr, P.lc(0, L_N), s));
-    scatter_kept_kernel<<<grid_for(cap, 256, g->sm_count), 256, 0, s>>>(sorted, P.ctr + CT_NSEEDS, P.seed_kept, P.seed_kpos, P.L[0].F);
+    launch_frontier(sorted, P.ctr + CT_NSEEDS, cap, none, P.vbits, P.seed_kept, P.scan_scr, P.L[0].F, P.lc(0, L_N), s);
     inst_bounds_kernel<<<grid_for((uint64_t)P.n_inst + 1, 256, g->sm_count), 256, 0, s>>>(P.L[0].F, P.lc(0, L_N), P.n_inst, P.vbits, P.L[0].FO);
     CSAW_CUDA(cudaGetLastError());
     return CSAW_OK;
@@ -2179,15 +2412,36 @@ static csaw_status enqueue_classify(Pipeline& P, uint32_t l, uint32_t v_lo, uint
     return CSAW_OK;
 }
 
+// The edge positions of layer l's entries, and for small frontiers its offsets.
+static csaw_status enqueue_positions(Pipeline& P, uint32_t l, cudaStream_t s)
+{
+    LayerBufs& B = P.L[l];
+    if (B.f_cap > SMALL_SCAN)
+        return scan_u32(B.cnt, B.pos, P.lc(l, L_N), B.f_cap, P.scan_scr, P.lc(l, L_TOTAL), s);
+    small_offsets_kernel<<<1, SCAN_THREADS, 0, s>>>(B.cnt, P.lc(l, L_N), B.pos, P.lc(l, L_TOTAL), B.FO, P.n_inst,
+                                                    P.ctr + CT_BASE + l, P.eoff + (uint64_t)l * P.n_inst,
+                                                    P.fsize + (uint64_t)l * P.n_inst, P.ctr + CT_BASE + l + 1);
+    CSAW_CUDA(cudaGetLastError());
+    B.offsets_done = true;
+    return CSAW_OK;
+}
+
 // Count/classify and the edge-position scan of layer l.
 static csaw_status enqueue_count(Pipeline& P, uint32_t l, cudaStream_t s)
 {
     LayerBufs& B = P.L[l];
     CSAW_TRY(enqueue_classify(P, l, 0, 0xFFFFFFFFu, true, s));
-    CSAW_TRY(scan_u32(B.cnt, B.pos, P.lc(l, L_N), B.f_cap, P.scan_scr, P.lc(l, L_TOTAL), s));
+    CSAW_TRY(enqueue_positions(P, l, s));
     if (P.hub_path && B.f_cap) CSAW_TRY(enqueue_hub_groups(P, l, s));
     if (P.hub_order && B.f_cap) CSAW_TRY(enqueue_hub_order(P, l, s));
     return CSAW_OK;
+}
+
+// Blocks of a persistent grid for at most n items, `per` at a time each.
+static int blocks_for(uint64_t n, int per, int most)
+{
+    const uint64_t b = (n + per - 1) / per;
+    return b < 1 ? 1 : b < (uint64_t)most ? (int)b : most;
 }
 
 // The selection kernels of layer l (its listed items) into its edge buffers.
@@ -2221,7 +2475,7 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             // warp items over the cached array; CTA items (more than PICK_MAX
             // picks) by the streaming kernel below
             const bool half = P.fanout[l] <= 16;   // two items per warp
-            const int blocks = g->sm_count * 8;
+            const int blocks = blocks_for(B.f_cap, half ? 2 * SEL_WARPS : SEL_WARPS, g->sm_count * 8);
             SelParams hs = sp;   // hub items, in vertex order where several instances can hold a hub
             hs.item_e = P.hub_order ? P.item_e : P.hlist;
             if (P.kind == CSAW_BIAS_UNIFORM) {
@@ -2251,6 +2505,7 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             blocks = g->sm_count * (per > 0 && per < occ ? per : occ);
             smem = sel_warp_smem(wide);
         }
+        blocks = blocks_for(B.f_cap, warp_only ? SEL_WARPS : 1, blocks);
         // without short rows to draw from only entries with more than PICK_MAX picks are left
         if (!sp.skip_warp_items || !few) CSAW_TRY(launch_select(P.kind, wide, sp, blocks, s, smem));
         if (P.hub_path) {
@@ -2263,7 +2518,7 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             hp.big_list = P.hubBig; hp.n_big = (const unsigned long long*)P.lc(l, L_NBIG);
             hp.next = (unsigned long long*)P.lc(l, L_HNEXT); hp.S = P.hubS;
             hp.S_cap = P.hubS_cap; hp.err = (uint32_t*)(P.ctr + CT_ERR);
-            const int blocks = g->sm_count * 8;
+            const int blocks = blocks_for(B.f_cap, 1, g->sm_count * 8);
             if (P.kind == CSAW_BIAS_EDGE_WEIGHT) hub_cdf_kernel<CSAW_BIAS_EDGE_WEIGHT><<<blocks, SEL_THREADS, 0, s>>>(hp);
             else hub_cdf_kernel<CSAW_BIAS_NEIGHBOR_DEGREE><<<blocks, SEL_THREADS, 0, s>>>(hp);
             SelParams hs = sp;
@@ -2271,8 +2526,9 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             hs.item_e = P.item_e; hs.item_h = P.item_h; hs.hub_off = P.hub_off; hs.hubS = P.hubS;
             hs.hubS_cap = P.hubS_cap; hs.err = (uint32_t*)(P.ctr + CT_ERR);
             // hub rows are long, so with at most 16 picks two items share a warp
-            if (P.fanout[l] <= 16) select_cdf_kernel<SRC_HUB, 16><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
-            else select_cdf_kernel<SRC_HUB><<<g->sm_count * 8, SEL_THREADS, 0, s>>>(hs);
+            const int draws = blocks_for(B.f_cap, P.fanout[l] <= 16 ? 2 * SEL_WARPS : SEL_WARPS, g->sm_count * 8);
+            if (P.fanout[l] <= 16) select_cdf_kernel<SRC_HUB, 16><<<draws, SEL_THREADS, 0, s>>>(hs);
+            else select_cdf_kernel<SRC_HUB><<<draws, SEL_THREADS, 0, s>>>(hs);
             CSAW_CUDA(cudaGetLastError());
         }
     }
@@ -2284,6 +2540,7 @@ static csaw_status enqueue_layer_offsets(Pipeline& P, uint32_t l, cudaStream_t s
 {
     csaw_graph* g = P.g;
     LayerBufs& B = P.L[l];
+    if (B.offsets_done) return CSAW_OK;
     layer_offsets_kernel<<<grid_for((uint64_t)P.n_inst + 1, 256, g->sm_count), 256, 0, s>>>(
         B.FO, B.pos, P.n_inst, P.ctr + CT_BASE + l, P.eoff + (uint64_t)l * P.n_inst,
         P.fsize + (uint64_t)l * P.n_inst, P.ctr + CT_BASE + l + 1);
@@ -2296,7 +2553,6 @@ static csaw_status enqueue_select(Pipeline& P, uint32_t l, cudaStream_t s)
 {
     CSAW_TRY(enqueue_select_items(P, l, s));
     return enqueue_layer_offsets(P, l, s);
-    return CSAW_OK;
 }
 
 // Update (Eq. 4): next frontier = sorted distinct picks of layer l that the
@@ -2306,14 +2562,18 @@ static csaw_status enqueue_compact(Pipeline& P, uint32_t l, cudaStream_t s)
     csaw_graph* g = P.g;
     LayerBufs& B = P.L[l];
     LayerBufs& N = P.L[l + 1];
-    uint64_t* sorted = B.cand;
-    if (B.e_cap) CSAW_TRY(radix_sort_u64(B.cand, B.cand_alt, P.lc(l, L_TOTAL), B.e_cap, P.kbits, g->sm_count, P.sort_scr, s, &sorted));
     Visited vis;
     vis.n = (int)l + 1;
     for (uint32_t j = 0; j <= l; ++j) { vis.keys[j] = P.L[j].F; vis.foff[j] = P.L[j].FO; }
-    unique_filter_kernel<<<grid_for(B.e_cap, 256, g->sm_count), 256, 0, s>>>(sorted, P.lc(l, L_TOTAL), vis, P.vbits, B.kept);
-    CSAW_TRY(scan_u32(B.kept, B.kpos, P.lc(l, L_TOTAL), B.e_cap, P.scan_scr, P.lc(l + 1, L_N), s));
-    scatter_kept_kernel<<<grid_for(B.e_cap, 256, g->sm_count), 256, 0, s>>>(sorted, P.lc(l, L_TOTAL), B.kept, B.kpos, N.F);
+    if (B.e_cap <= SF_KEYS) {
+        SmallFrontier sf;
+        sf.cand = B.cand; sf.n_cand = P.lc(l, L_TOTAL);
+        sf.vis = vis;
+        return launch_small_frontier(P, sf, l + 1, s);
+    }
+    uint64_t* sorted = B.cand;
+    if (B.e_cap) CSAW_TRY(radix_sort_u64(B.cand, B.cand_alt, P.lc(l, L_TOTAL), B.e_cap, P.kbits, g->sm_count, P.sort_scr, s, &sorted));
+    launch_frontier(sorted, P.lc(l, L_TOTAL), B.e_cap, vis, P.vbits, B.kept, P.scan_scr, N.F, P.lc(l + 1, L_N), s);
     inst_bounds_kernel<<<grid_for((uint64_t)P.n_inst + 1, 256, g->sm_count), 256, 0, s>>>(N.F, P.lc(l + 1, L_N), P.n_inst, P.vbits, N.FO);
     CSAW_CUDA(cudaGetLastError());
     return CSAW_OK;
@@ -2337,7 +2597,6 @@ static csaw_status alloc_common(Pipeline& P, Alloc&& get)
     CSAW_TRY(get((void**)&P.seed_keys, sizeof(uint64_t) * sc));
     CSAW_TRY(get((void**)&P.seed_alt, sizeof(uint64_t) * sc));
     CSAW_TRY(get((void**)&P.seed_kept, sizeof(uint32_t) * sc));
-    CSAW_TRY(get((void**)&P.seed_kpos, sizeof(uint64_t) * (sc + 1)));
     return CSAW_OK;
 }
 
@@ -2396,7 +2655,6 @@ static csaw_status alloc_edges(Pipeline& P, uint32_t l, uint64_t e_cap, Alloc&& 
         CSAW_TRY(get((void**)&B.cand, sizeof(uint64_t) * e));
         CSAW_TRY(get((void**)&B.cand_alt, sizeof(uint64_t) * e));
         CSAW_TRY(get((void**)&B.kept, sizeof(uint32_t) * e));
-        CSAW_TRY(get((void**)&B.kpos, sizeof(uint64_t) * (e + 1)));
     }
     return CSAW_OK;
 }
@@ -2451,7 +2709,7 @@ static csaw_status enqueue_layer_count(Pipeline& P, uint32_t l, cudaStream_t s)
         }
         CSAW_CUDA(cudaGetLastError());
     }
-    return scan_u32(B.cnt, B.pos, P.lc(l, L_N), B.f_cap, P.scan_scr, P.lc(l, L_TOTAL), s);
+    return enqueue_positions(P, l, s);
 }
 
 // Whether layer l is drawn by layer_draw_kernel: every bias positive, the
@@ -2512,11 +2770,7 @@ static csaw_status enqueue_layer_select(Pipeline& P, uint32_t l, uint64_t* VP, u
         }
         CSAW_CUDA(cudaGetLastError());
     }
-    layer_offsets_kernel<<<grid_for((uint64_t)P.n_inst + 1, 256, g->sm_count), 256, 0, s>>>(
-        B.FO, B.pos, P.n_inst, P.ctr + CT_BASE + l, P.eoff + (uint64_t)l * P.n_inst,
-        P.fsize + (uint64_t)l * P.n_inst, P.ctr + CT_BASE + l + 1);
-    CSAW_CUDA(cudaGetLastError());
-    return CSAW_OK;
+    return enqueue_layer_offsets(P, l, s);
 }
 
 // csaw_sample: exact edge buffers, one wait per layer.
@@ -3071,8 +3325,8 @@ extern "C" csaw_status csaw_sample_plan_get_info(const csaw_sample_plan* pl, uin
         // sizes are not recorded per allocation; report capacities
         const Pipeline& P = pl->P;
         for (uint32_t l = 0; l < P.depth; ++l)
-            b += P.L[l].f_cap * 28 + P.L[l].e_cap * (8 + (l + 1 < P.depth ? 28 : 0));
-        b += P.seeds_cap * 28 + pl->max_seeds * 4;
+            b += P.L[l].f_cap * 28 + P.L[l].e_cap * (8 + (l + 1 < P.depth ? 20 : 0));
+        b += P.seeds_cap * 20 + pl->max_seeds * 4;
         *device_bytes = b;
     }
     if (theta_warp) *theta_warp = pl->P.theta_w;
