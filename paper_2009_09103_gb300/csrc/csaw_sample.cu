@@ -2203,6 +2203,8 @@ struct Pipeline {
     uint64_t* hubS = nullptr;            // [hubS_cap]
 
     uint64_t* lc(uint32_t l, int w) const { return ctr + CT_LAYER + L_WORDS * l + w; }
+    // counters, then eoff, then fsize
+    uint64_t host_words() const { return CT_WORDS + 2 * ((uint64_t)depth * n_inst + 1); }
 
     void init(csaw_graph* gr, int k, uint32_t ninst, uint32_t dep, const uint32_t* fan, uint64_t seed)
     {
@@ -2579,24 +2581,54 @@ static csaw_status enqueue_compact(Pipeline& P, uint32_t l, cudaStream_t s)
     return CSAW_OK;
 }
 
+// Several buffers in one allocation: each is 256-byte aligned in it.  (A call
+// makes a dozen allocations instead of fifty.)
+struct Carve {
+    struct Part {
+        void** p;
+        size_t at;
+    };
+    std::vector<Part> parts;
+    size_t bytes = 0;
+    template <class T>
+    void add(T** p, uint64_t count)
+    {
+        parts.push_back({(void**)p, bytes});
+        bytes = (bytes + sizeof(T) * count + 255) & ~(size_t)255;
+    }
+    template <class Alloc>
+    csaw_status commit(Alloc&& get)
+    {
+        if (!bytes) return CSAW_OK;
+        char* base = nullptr;
+        CSAW_TRY(get((void**)&base, bytes));
+        for (const Part& q : parts) *q.p = base + q.at;
+        return CSAW_OK;
+    }
+};
+
 // Buffers shared by every layer (counters, scratch, offsets, seed arrays).
+// The counters, edge offsets and frontier sizes are one run of words
+// (host_words), so that the host reads them with one copy.
 template <class Alloc>
 static csaw_status alloc_common(Pipeline& P, Alloc&& get)
 {
-    CSAW_TRY(get((void**)&P.ctr, sizeof(uint64_t) * CT_WORDS));
-    CSAW_TRY(get(&P.scan_scr, scan_scratch_bytes(0)));
-    CSAW_TRY(get(&P.sort_scr, sort_scratch_bytes(0)));
+    Carve c;
+    c.add(&P.ctr, P.host_words());
+    c.add((char**)&P.scan_scr, scan_scratch_bytes(0));
+    c.add((char**)&P.sort_scr, sort_scratch_bytes(0));
     if (P.cta_slots()) {
-        CSAW_TRY(get((void**)&P.hub_S, sizeof(uint64_t) * (size_t)P.sel_blocks * P.g->max_degree));
-        CSAW_TRY(get((void**)&P.hub_bits, sizeof(uint32_t) * (size_t)P.sel_blocks * ((P.g->max_degree + 31) / 32)));
+        c.add(&P.hub_S, (uint64_t)P.sel_blocks * P.g->max_degree);
+        c.add(&P.hub_bits, (uint64_t)P.sel_blocks * ((P.g->max_degree + 31) / 32));
     }
-    const uint64_t ng = (uint64_t)P.depth * P.n_inst + 1;
-    CSAW_TRY(get((void**)&P.eoff, sizeof(uint64_t) * ng));
-    CSAW_TRY(get((void**)&P.fsize, sizeof(uint64_t) * ng));
-    const uint64_t sc = P.seeds_cap ? P.seeds_cap : 1;
-    CSAW_TRY(get((void**)&P.seed_keys, sizeof(uint64_t) * sc));
-    CSAW_TRY(get((void**)&P.seed_alt, sizeof(uint64_t) * sc));
-    CSAW_TRY(get((void**)&P.seed_kept, sizeof(uint32_t) * sc));
+    if (P.seeds_cap > SF_KEYS) {
+        c.add(&P.seed_keys, P.seeds_cap);
+        c.add(&P.seed_alt, P.seeds_cap);
+        c.add(&P.seed_kept, P.seeds_cap);
+    }
+    CSAW_TRY(c.commit(get));
+    P.eoff = P.ctr + CT_WORDS;
+    P.fsize = P.eoff + (uint64_t)P.depth * P.n_inst + 1;
     return CSAW_OK;
 }
 
@@ -2606,21 +2638,24 @@ template <class Alloc>
 static csaw_status alloc_hub(Pipeline& P, uint64_t cap, Alloc&& get)
 {
     P.hub_cap = cap;
-    const uint64_t c = cap ? cap : 1;
-    CSAW_TRY(get((void**)&P.hlist, sizeof(uint32_t) * c));
-    if (!P.hub_path && !P.hub_order) return CSAW_OK;
-    CSAW_TRY(get((void**)&P.hkeys, sizeof(uint64_t) * c));
-    CSAW_TRY(get((void**)&P.halt, sizeof(uint64_t) * c));
-    CSAW_TRY(get((void**)&P.item_e, sizeof(uint32_t) * c));
-    if (!P.hub_path) return CSAW_OK;
-    CSAW_TRY(get((void**)&P.hflag, sizeof(uint32_t) * c));
-    CSAW_TRY(get((void**)&P.hpos, sizeof(uint64_t) * (c + 1)));
-    CSAW_TRY(get((void**)&P.item_h, sizeof(uint32_t) * c));
-    CSAW_TRY(get((void**)&P.hubH, sizeof(uint32_t) * c));
-    CSAW_TRY(get((void**)&P.hubD, sizeof(uint32_t) * c));
-    CSAW_TRY(get((void**)&P.hubBig, sizeof(uint32_t) * c));
-    CSAW_TRY(get((void**)&P.hub_off, sizeof(uint64_t) * (c + 1)));
-    return CSAW_OK;
+    const uint64_t n = cap ? cap : 1;
+    Carve c;
+    c.add(&P.hlist, n);
+    if (P.hub_path || P.hub_order) {
+        c.add(&P.hkeys, n);
+        c.add(&P.halt, n);
+        c.add(&P.item_e, n);
+    }
+    if (P.hub_path) {
+        c.add(&P.hflag, n);
+        c.add(&P.hpos, n + 1);
+        c.add(&P.item_h, n);
+        c.add(&P.hubH, n);
+        c.add(&P.hubD, n);
+        c.add(&P.hubBig, n);
+        c.add(&P.hub_off, n + 1);
+    }
+    return c.commit(get);
 }
 
 // Per-entry arrays of layer l (frontier capacity f_cap) and its frontier keys.
@@ -2630,13 +2665,14 @@ static csaw_status alloc_entries(Pipeline& P, uint32_t l, uint64_t f_cap, Alloc&
     LayerBufs& B = P.L[l];
     B.f_cap = f_cap;
     const uint64_t f = f_cap ? f_cap : 1;
-    CSAW_TRY(get((void**)&B.F, sizeof(uint64_t) * f));
-    CSAW_TRY(get((void**)&B.FO, sizeof(uint64_t) * ((uint64_t)P.n_inst + 1)));
-    CSAW_TRY(get((void**)&B.cnt, sizeof(uint32_t) * f));
-    CSAW_TRY(get((void**)&B.wlist, sizeof(uint32_t) * f));
-    CSAW_TRY(get((void**)&B.clist, sizeof(uint32_t) * f));
-    CSAW_TRY(get((void**)&B.pos, sizeof(uint64_t) * (f + 1)));
-    return CSAW_OK;
+    Carve c;
+    c.add(&B.F, f);
+    c.add(&B.FO, (uint64_t)P.n_inst + 1);
+    c.add(&B.cnt, f);
+    c.add(&B.wlist, f);
+    c.add(&B.clist, f);
+    c.add(&B.pos, f + 1);
+    return c.commit(get);
 }
 
 // Edge arrays of layer l (capacity e_cap); src/dst come from `get_out`.
@@ -2652,9 +2688,13 @@ static csaw_status alloc_edges(Pipeline& P, uint32_t l, uint64_t e_cap, Alloc&& 
         if (e_cap >= 0xFFFFFFFFull)
             return fail(CSAW_ERR_INVALID, "layer %u may produce %llu edges; frontier compaction sorts "
                         "at most 2^32-1", l, (unsigned long long)e_cap);
-        CSAW_TRY(get((void**)&B.cand, sizeof(uint64_t) * e));
-        CSAW_TRY(get((void**)&B.cand_alt, sizeof(uint64_t) * e));
-        CSAW_TRY(get((void**)&B.kept, sizeof(uint32_t) * e));
+        Carve c;
+        c.add(&B.cand, e);
+        if (e_cap > SF_KEYS) {
+            c.add(&B.cand_alt, e);
+            c.add(&B.kept, e);
+        }
+        CSAW_TRY(c.commit(get));
     }
     return CSAW_OK;
 }
@@ -2845,17 +2885,18 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
         };
         if (hubs) CSAW_TRY(alloc_hub(P, P.L[l].f_cap, get_layer));
         CSAW_TRY(layer_mode ? enqueue_layer_count(P, l, s) : enqueue_count(P, l, s));
-        uint64_t h[3] = {0, 0, 0};
-        CSAW_CUDA(cudaMemcpyAsync(&h[0], P.ctr + CT_ERR, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-        CSAW_CUDA(cudaMemcpyAsync(&h[1], P.lc(l, L_TOTAL), sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        // the errors and this layer's counters, in one copy
         const bool shared = hubs && P.hub_path;   // shared hub arrays (streamed biases)
-        if (shared) CSAW_CUDA(cudaMemcpyAsync(&h[2], P.lc(l, L_HUBE), sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        uint64_t words[CT_WORDS];
+        CSAW_CUDA(cudaMemcpyAsync(words, P.ctr, sizeof(uint64_t) * (CT_LAYER + L_WORDS * (l + 1)),
+                                  cudaMemcpyDeviceToHost, s));
         CSAW_CUDA(cudaStreamSynchronize(s));
-        CSAW_TRY(check_errors(h[0]));
-        const uint64_t total = h[1];
+        CSAW_TRY(check_errors(words[CT_ERR]));
+        const uint64_t* h = words + CT_LAYER + L_WORDS * l;
+        const uint64_t total = h[L_TOTAL];
         if (shared) {
-            P.hubS_cap = h[2];
-            CSAW_TRY(get_layer((void**)&P.hubS, sizeof(uint64_t) * (h[2] ? h[2] : 1)));
+            P.hubS_cap = h[L_HUBE];
+            CSAW_TRY(get_layer((void**)&P.hubS, sizeof(uint64_t) * (P.hubS_cap ? P.hubS_cap : 1)));
         }
         R->layer_edges[l] = total;
         CSAW_TRY(alloc_edges(P, l, total, get, get_out));
@@ -2884,16 +2925,13 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
         }
     }
     const uint64_t ng = (uint64_t)depth * n_inst;
-    R->edge_offsets.assign(ng + 1, 0);
-    R->frontier_sizes.assign(ng, 0);
-    if (ng) {
-        CSAW_CUDA(cudaMemcpyAsync(R->edge_offsets.data(), P.eoff, sizeof(uint64_t) * (ng + 1), cudaMemcpyDeviceToHost, s));
-        CSAW_CUDA(cudaMemcpyAsync(R->frontier_sizes.data(), P.fsize, sizeof(uint64_t) * ng, cudaMemcpyDeviceToHost, s));
-    }
-    uint64_t err_end = 0;
-    CSAW_CUDA(cudaMemcpyAsync(&err_end, P.ctr + CT_ERR, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    std::vector<uint64_t> words(P.host_words());
+    CSAW_CUDA(cudaMemcpyAsync(words.data(), P.ctr, sizeof(uint64_t) * words.size(), cudaMemcpyDeviceToHost, s));
     CSAW_CUDA(cudaStreamSynchronize(s));
-    CSAW_TRY(check_errors(err_end));
+    CSAW_TRY(check_errors(words[CT_ERR]));
+    const uint64_t* eoff = words.data() + CT_WORDS;
+    R->edge_offsets.assign(eoff, eoff + ng + 1);
+    R->frontier_sizes.assign(eoff + ng + 1, eoff + 2 * ng + 1);
     uint64_t total = 0;
     for (uint32_t l = 0; l < depth; ++l) total += R->layer_edges[l];
     R->n_edges = total;
@@ -3080,6 +3118,8 @@ extern "C" csaw_status csaw_sample_copy_edges(csaw_sample_result* r, uint32_t* s
 // CUDA graph.  Each run copies new seeds in and launches the graph: no host
 // waits, no allocation, one launch for all instances and layers.
 
+static constexpr size_t PLAN_STAGE_BYTES = 256 << 10;
+
 struct csaw_sample_plan {
     uint32_t magic = 0x43504c4eu;   // "CPLN"
     csaw::Pipeline P;
@@ -3093,12 +3133,15 @@ struct csaw_sample_plan {
     cudaGraphExec_t exec = nullptr;
     cudaStream_t last = nullptr;
     bool ran = false;
+    bool collected = false;      // the last run's counters and offsets are in h_eoff ...
+    uint64_t* h_words = nullptr; // page-locked: host_words(), then PLAN_STAGE_BYTES for small results
     std::vector<uint64_t> h_eoff, h_fsize, h_layer_edges;
     std::vector<const uint32_t*> src_c, dst_c;
     ~csaw_sample_plan()
     {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
+        if (h_words) cudaFreeHost(h_words);
         for (void* p : allocs) csaw::free_with(alloc, p, nullptr);
     }
 };
@@ -3187,6 +3230,10 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
     if (st == CSAW_OK) st = get((void**)&pl->in_key, 2 * sizeof(uint32_t));
     if (st != CSAW_OK) { delete pl; return st; }
     P.key_dev = pl->in_key;
+    if (cudaHostAlloc((void**)&pl->h_words, sizeof(uint64_t) * P.host_words() + PLAN_STAGE_BYTES, 0) != cudaSuccess) {
+        cudaGetLastError();
+        pl->h_words = nullptr;
+    }
     cudaStream_t cs;
     cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) { delete pl; return cuda_fail(e, "cudaStreamCreate"); }
@@ -3257,6 +3304,7 @@ extern "C" csaw_status csaw_sample_plan_run(csaw_sample_plan* pl, const uint32_t
     CSAW_CUDA(cudaGraphLaunch(pl->exec, s));
     pl->last = s;
     pl->ran = true;
+    pl->collected = false;
     return CSAW_OK;
 }
 
@@ -3264,21 +3312,28 @@ extern "C" csaw_status csaw_sample_plan_run(csaw_sample_plan* pl, const uint32_t
 static csaw_status plan_collect(csaw_sample_plan* pl)
 {
     if (!pl->ran) return fail(CSAW_ERR_INVALID, "the plan has not run");
+    if (pl->collected) return CSAW_OK;
     Pipeline& P = pl->P;
-    CSAW_CUDA(cudaStreamSynchronize(pl->last));
     const uint64_t ng = (uint64_t)P.depth * P.n_inst;
-    pl->h_eoff.assign(ng + 1, 0);
-    pl->h_fsize.assign(ng ? ng : 1, 0);
-    std::vector<uint64_t> ctr(CT_WORDS, 0);
-    CSAW_CUDA(cudaMemcpy(ctr.data(), P.ctr, sizeof(uint64_t) * CT_WORDS, cudaMemcpyDeviceToHost));
-    CSAW_TRY(check_errors(ctr[CT_ERR]));
-    CSAW_CUDA(cudaMemcpy(pl->h_eoff.data(), P.eoff, sizeof(uint64_t) * (ng + 1), cudaMemcpyDeviceToHost));
-    if (ng) CSAW_CUDA(cudaMemcpy(pl->h_fsize.data(), P.fsize, sizeof(uint64_t) * ng, cudaMemcpyDeviceToHost));
+    std::vector<uint64_t> own;
+    uint64_t* words = pl->h_words;   // page-locked, where that could be had
+    if (!words) {
+        own.resize(P.host_words());
+        words = own.data();
+    }
+    CSAW_CUDA(cudaMemcpyAsync(words, P.ctr, sizeof(uint64_t) * P.host_words(), cudaMemcpyDeviceToHost, pl->last));
+    CSAW_CUDA(cudaStreamSynchronize(pl->last));
+    CSAW_TRY(check_errors(words[CT_ERR]));
+    const uint64_t* eoff = words + CT_WORDS;
+    pl->h_eoff.assign(eoff, eoff + ng + 1);
+    pl->h_fsize.assign(eoff + ng + 1, eoff + 2 * ng + 1);
+    if (!ng) pl->h_fsize.assign(1, 0);
     pl->h_layer_edges.assign(P.depth, 0);
-    for (uint32_t l = 0; l < P.depth; ++l) pl->h_layer_edges[l] = ctr[CT_LAYER + L_WORDS * l + L_TOTAL];
+    for (uint32_t l = 0; l < P.depth; ++l) pl->h_layer_edges[l] = words[CT_LAYER + L_WORDS * l + L_TOTAL];
     pl->src_c.assign(P.depth, nullptr);
     pl->dst_c.assign(P.depth, nullptr);
     for (uint32_t l = 0; l < P.depth; ++l) { pl->src_c[l] = P.L[l].src; pl->dst_c[l] = P.L[l].dst; }
+    pl->collected = true;
     return CSAW_OK;
 }
 
@@ -3302,15 +3357,25 @@ extern "C" csaw_status csaw_sample_plan_copy_edges(csaw_sample_plan* pl, uint32_
     clear_error();
     if (!pl) return fail(CSAW_ERR_INVALID, "plan is NULL");
     CSAW_TRY(plan_collect(pl));
+    const uint64_t total = pl->h_eoff.back();
+    if (total && (!src || !dst)) return fail(CSAW_ERR_INVALID, "NULL output");
+    // a small result through the page-locked words, in one wait
+    const bool staged = pl->h_words && 2 * total * sizeof(uint32_t) <= PLAN_STAGE_BYTES;
+    uint32_t* to_src = staged ? (uint32_t*)(pl->h_words + pl->P.host_words()) : src;
+    uint32_t* to_dst = staged ? to_src + total : dst;
     uint64_t at = 0;
     for (uint32_t l = 0; l < pl->P.depth; ++l) {
         const uint64_t n = pl->h_layer_edges[l];
         if (n) {
-            if (!src || !dst) return fail(CSAW_ERR_INVALID, "NULL output");
-            CSAW_CUDA(cudaMemcpy(src + at, pl->P.L[l].src, n * sizeof(uint32_t), cudaMemcpyDeviceToHost));
-            CSAW_CUDA(cudaMemcpy(dst + at, pl->P.L[l].dst, n * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+            CSAW_CUDA(cudaMemcpyAsync(to_src + at, pl->P.L[l].src, n * sizeof(uint32_t), cudaMemcpyDeviceToHost, pl->last));
+            CSAW_CUDA(cudaMemcpyAsync(to_dst + at, pl->P.L[l].dst, n * sizeof(uint32_t), cudaMemcpyDeviceToHost, pl->last));
         }
         at += n;
+    }
+    CSAW_CUDA(cudaStreamSynchronize(pl->last));
+    if (staged && total) {
+        std::memcpy(src, to_src, total * sizeof(uint32_t));
+        std::memcpy(dst, to_dst, total * sizeof(uint32_t));
     }
     return CSAW_OK;
 }
