@@ -453,7 +453,7 @@ __device__ void cta_item(const SelParams& p, uint32_t e, uint64_t* S, uint32_t* 
 }
 
 template <int KIND, bool WIDE>
-__global__ void __launch_bounds__(SEL_THREADS, 6) select_kernel(SelParams p)
+__global__ void __launch_bounds__(SEL_THREADS, 8) select_kernel(SelParams p)
 {
     if (p.key_dev) {
         p.k0 = p.key_dev[0];
@@ -525,7 +525,7 @@ __device__ __forceinline__ uint64_t cdf_at(const uint64_t* __restrict__ row, boo
 enum : int { SRC_IMPLICIT = 0, SRC_LEAF = 1, SRC_HUB = 2, SRC_PACK = 3 };
 
 template <int SRC, int G = 32>
-__global__ void __launch_bounds__(SEL_THREADS, SRC == SRC_PACK ? 5 : SRC == SRC_LEAF ? 6 : 8) select_cdf_kernel(SelParams p)
+__global__ void __launch_bounds__(SEL_THREADS, SRC == SRC_PACK || SRC == SRC_LEAF ? 6 : 8) select_cdf_kernel(SelParams p)
 {
     static_assert(G == 32 || G == 16, "16 or 32 lanes per item");
     constexpr bool IMPLICIT = SRC == SRC_IMPLICIT;
@@ -2206,9 +2206,11 @@ struct Pipeline {
     // counters, then eoff, then fsize
     uint64_t host_words() const { return CT_WORDS + 2 * ((uint64_t)depth * n_inst + 1); }
 
-    void init(csaw_graph* gr, int k, uint32_t ninst, uint32_t dep, const uint32_t* fan, uint64_t seed)
+    void init(csaw_graph* gr, int k, uint32_t ninst, uint32_t dep, const uint32_t* fan, uint64_t seed,
+              uint64_t max_seeds)
     {
         g = gr;
+        seeds_cap = max_seeds;
         kind = k;
         n_inst = ninst;
         depth = dep;
@@ -2245,8 +2247,13 @@ struct Pipeline {
         // hub; a single instance's frontier holds each vertex once, and its
         // long rows take the CTA path without the grouping kernels
         hub_path = !cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE);
-        // vertex order pays only when several instances can hold the same hub
-        hub_order = cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE);
+        // vertex order pays only when several instances can hold the same hub,
+        // and over the packed array only where its rows do not stay in L2 (8.6
+        // bytes per edge) and there are items enough: RMAT s20, 1024 instances,
+        // 1 M seeds 3.56 ms in order, 3.67 without; 64 K seeds 0.68 and 0.63;
+        // s16, 1 M seeds 2.67 and 2.63; the s22 plan 14.4 and 15.5
+        hub_order = cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE) &&
+                    (!pack || (seeds_cap >= (1u << 19) && g->E >= (1u << 24)));
     }
 
     // CTA items exist for picks above PICK_MAX (or, without the hub path, any
@@ -2829,9 +2836,8 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
     if (const DevAllocator* a = current_allocator()) R->alloc = *a;
     R->stream = s;
     Pipeline P;
-    P.init(g, kind, n_inst, depth, fanout, rng_seed);
+    P.init(g, kind, n_inst, depth, fanout, rng_seed, n_seeds);
     P.attempt_cap = attempt_cap;
-    P.seeds_cap = n_seeds;
     if (tabs) {
         P.inst_key = tabs->inst_key;
         P.inst_id = tabs->inst_id;
@@ -3175,9 +3181,8 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
     csaw_sample_plan* pl = new (std::nothrow) csaw_sample_plan();
     if (!pl) return fail(CSAW_ERR_NOMEM, "host allocation failed");
     Pipeline& P = pl->P;
-    P.init(g, kind, n_instances, depth, fanout, 0);
+    P.init(g, kind, n_instances, depth, fanout, 0, max_seeds);
     P.attempt_cap = opts ? opts->attempt_cap : CSAW_ATTEMPT_CAP;
-    P.seeds_cap = max_seeds;
     pl->max_seeds = max_seeds;
     pl->alloc = g->allocator;
     auto get = [&](void** p, size_t bytes) -> csaw_status {
@@ -3603,7 +3608,7 @@ extern "C" csaw_status csaw_sample_oom(const uint64_t* row_offsets, const uint32
         view.w = weighted ? slot[0].w : nullptr;
 
         Pipeline P;
-        P.init(&view, eff_kind, n_instances, depth, fanout, rng_seed);
+        P.init(&view, eff_kind, n_instances, depth, fanout, rng_seed, n_seeds);
         P.take = false;   // whole rows are listed with the loaded partition's warp items
         P.seeds_cap = n_seeds;
         st = alloc_common(P, get);
