@@ -236,21 +236,23 @@ __host__ __device__ inline CdfView cdf_view(const uint64_t* base, uint64_t E, ui
 // edges 0 .. e, over all rows; a row's own prefix sums are P[e] - P[start - 1].
 //   pack[g][16]  per 8-edge group its biases, then its columns (64 bytes)
 //   s1[g]        P at the group's end less P at its 64-edge block's start, 32 bits
-//   s2[h]        P at the end of block h
+//   s2[k][4]     per window of three blocks: P before it, and at its blocks'
+//                ends (one sector; past the last block: the largest value)
 //   rec[v]       {off[v], P before off[v]}, v <= V
 //   sums[c]      scratch of the build, one word per chunk
 // Edges are padded with zero biases to whole chunks.
 constexpr uint64_t PACK_CHUNK = 8192;
 struct PackLayout {
-    uint64_t chunks, s1, s2, rec, sums, words;   // word (8-byte) offsets and the total; pack at word 0
+    uint64_t chunks, blocks, s1, s2, rec, sums, words;   // counts, word (8-byte) offsets, total; pack at word 0
 };
 __host__ __device__ inline PackLayout pack_layout(uint64_t E, uint64_t V)
 {
     PackLayout L;
     L.chunks = (E + PACK_CHUNK - 1) / PACK_CHUNK;
+    L.blocks = L.chunks * (PACK_CHUNK / 64);
     L.s1 = L.chunks * PACK_CHUNK;
     L.s2 = L.s1 + L.chunks * (PACK_CHUNK / 16);
-    L.rec = L.s2 + L.chunks * (PACK_CHUNK / 64);
+    L.rec = L.s2 + 4 * (L.blocks / 3 + 1);
     L.sums = L.rec + 2 * (V + 1);
     L.words = L.sums + L.chunks;
     return L;
@@ -272,6 +274,9 @@ __host__ __device__ inline PackView pack_view(const uint64_t* words, uint64_t E,
     k.rec = words + L.rec;
     return k;
 }
+// The word of s2 that holds P before block h (and P at the end of block h - 1).
+__host__ __device__ inline uint64_t pack_before(uint32_t h) { return 4ull * (h / 3u) + h % 3u; }
+
 // Whether the kind's biases fit the packed array: weights or degrees below
 // 2^26, so that a block's sums fit 32 bits.
 bool pack_fits(const csaw_graph* g, int kind);
@@ -616,9 +621,9 @@ __device__ __forceinline__ uint64_t w_search(const CdfView& c, const uint32_t* _
 // [P[beg - 1], P[end - 1]): its column, its number, P before it and its bias.
 // P does not decrease over all edges, so the search is over all blocks,
 // started at edge `guess` (of the row), where the draw would fall if the row's
-// biases were equal: four block ends are read at once (one sector, and
-// the end before them), which holds the answer for most rows; otherwise a
-// galloping search goes on from there.  Then one sector of the block's group
+// biases were equal: a window of three blocks is read at once (one sector),
+// which holds the answer for most rows; otherwise a galloping search goes on
+// from there.  Then one sector of the block's group
 // sums and the group's biases and columns: four dependent loads a step, with
 // the record, against ten or so for the bisected summaries (cdf_group), and
 // one 64-byte line per pick where weights and column were two.
@@ -628,18 +633,17 @@ struct PackHit {
 };
 __device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, uint64_t end, uint64_t guess, uint64_t y)
 {
-    uint64_t at = guess >> 8;   // 256-edge window
+    uint32_t at = (uint32_t)(guess >> 6) / 3u;   // window
     uint64_t v[4];
-    ld256(k.s2 + 4 * at, v);
-    uint64_t before = at ? __ldg(k.s2 + 4 * at - 1) : 0ull;
-    if (before > y || v[3] <= y) {
+    ld256(k.s2 + 4ull * at, v);
+    if (v[0] > y || v[3] <= y) {
         // first window whose end exceeds y, in [lo, hi]
-        uint64_t lo = beg >> 8, hi = (end - 1) >> 8;
+        uint32_t lo = (uint32_t)(beg >> 6) / 3u, hi = (uint32_t)((end - 1) >> 6) / 3u;
         if (v[3] <= y) {
             lo = at + 1;
-            for (uint64_t step = 1; lo + step - 1 < hi; step <<= 1) {
-                const uint64_t q = lo + step - 1;
-                if (__ldg(k.s2 + 4 * q + 3) > y) {
+            for (uint32_t step = 1; lo + step - 1 < hi; step <<= 1) {
+                const uint32_t q = lo + step - 1;
+                if (__ldg(k.s2 + 4ull * q + 3) > y) {
                     hi = q;
                     break;
                 }
@@ -647,9 +651,9 @@ __device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, ui
             }
         } else {
             hi = at - 1;
-            for (uint64_t step = 1; lo < hi; step <<= 1) {
-                const uint64_t q = hi - (step < hi - lo ? step : hi - lo);
-                if (__ldg(k.s2 + 4 * q + 3) <= y) {
+            for (uint32_t step = 1; lo < hi; step <<= 1) {
+                const uint32_t q = hi - min(step, hi - lo);
+                if (__ldg(k.s2 + 4ull * q + 3) <= y) {
                     lo = q + 1;
                     break;
                 }
@@ -657,15 +661,13 @@ __device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, ui
             }
         }
         while (lo < hi) {
-            const uint64_t mid = lo + ((hi - lo) >> 1);
-            if (__ldg(k.s2 + 4 * mid + 3) > y) hi = mid; else lo = mid + 1;
+            const uint32_t mid = lo + ((hi - lo) >> 1);
+            if (__ldg(k.s2 + 4ull * mid + 3) > y) hi = mid; else lo = mid + 1;
         }
         at = lo;
-        ld256(k.s2 + 4 * at, v);
-        before = at ? __ldg(k.s2 + 4 * at - 1) : 0ull;
+        ld256(k.s2 + 4ull * at, v);
     }
-    uint64_t h = 4 * at;
-    if (v[0] <= y) { before = v[0]; ++h; }
+    uint64_t before = v[0], h = 3ull * at;
     if (v[1] <= y) { before = v[1]; ++h; }
     if (v[2] <= y) { before = v[2]; ++h; }
     uint32_t x = (uint32_t)(y - before);
@@ -703,7 +705,7 @@ __device__ __forceinline__ PackHit pack_pick(const PackView& k, uint64_t beg, ui
 __device__ __forceinline__ uint64_t pack_prefix(const PackView& k, uint64_t e)
 {
     const uint64_t g = e >> 3;
-    uint64_t sum = g >= 8 ? __ldg(k.s2 + (g >> 3) - 1) : 0ull;
+    uint64_t sum = __ldg(k.s2 + pack_before((uint32_t)(g >> 3)));
     if (g & 7) sum += __ldg(k.s1 + g - 1);
     for (uint32_t j = 0; j < (uint32_t)(e & 7); ++j) sum += __ldg(k.pack + 16 * g + j);
     return sum;

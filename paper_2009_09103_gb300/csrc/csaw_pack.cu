@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(PK_THREADS) pack_groups_kernel(const uint32_t*
             if (k < wid) before += t;
             running += t;
         }
-        if ((lane & 7) == 7) s2[g >> 3] = before + incl;
+        if ((lane & 7) == 7) s2[pack_before((uint32_t)(g >> 3)) + 1] = before + incl;
     }
     if (threadIdx.x == 0) chunk_sum[blockIdx.x] = running;
 }
@@ -108,10 +108,18 @@ __global__ void __launch_bounds__(1024) pack_carry_kernel(uint64_t* __restrict__
     }
 }
 
+// The blocks' ends from all edges; a window's first word is the end before it.
 __global__ void pack_ends_kernel(const uint64_t* __restrict__ chunk_sum, uint64_t blocks, uint64_t* __restrict__ s2)
 {
-    for (uint64_t h = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; h < blocks; h += (uint64_t)gridDim.x * blockDim.x)
-        s2[h] += __ldg(chunk_sum + h / (PACK_CHUNK / 64));
+    for (uint64_t h = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; h < blocks; h += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t at = pack_before((uint32_t)h) + 1;
+        const uint64_t end = s2[at] + __ldg(chunk_sum + h / (PACK_CHUNK / 64));
+        s2[at] = end;
+        if (h % 3 == 2) s2[at + 1] = end;
+        if (h == 0) s2[0] = 0;
+        if (h + 1 == blocks)
+            for (uint64_t q = at + (h % 3 == 2 ? 2 : 1); q < 4 * (blocks / 3 + 1); ++q) s2[q] = ~0ull;
+    }
 }
 
 // rec[v] = {off[v], the sum of all edges before it}, v <= V.
@@ -121,7 +129,7 @@ __global__ void pack_rows_kernel(const uint64_t* __restrict__ off, uint32_t V, c
 {
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= V; v += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t e = __ldg(off + v), g = e >> 3;
-        uint64_t before = g >= 8 ? s2[(g >> 3) - 1] : 0ull;
+        uint64_t before = s2[pack_before((uint32_t)(g >> 3))];
         if (g & 7) before += s1[g - 1];
         for (uint32_t j = 0; j < (uint32_t)(e & 7); ++j) before += pack[16 * g + j];
         reinterpret_cast<ulonglong2*>(rec)[v] = make_ulonglong2(e, before);
@@ -143,12 +151,11 @@ csaw_status enqueue_pack_build(const csaw_graph* g, int kind, uint64_t* words, c
         pack_groups_kernel<CSAW_BIAS_NEIGHBOR_DEGREE><<<(unsigned)L.chunks, PK_THREADS, 0, s>>>(g->col, g->w, g->deg,
                                                                                                 g->E, pack, s1, s2, cs);
     pack_carry_kernel<<<1, 1024, 0, s>>>(cs, L.chunks);
-    const uint64_t blocks = L.chunks * (PACK_CHUNK / 64);
     const auto grid = [&](uint64_t n) {
         const uint64_t b = (n + 255) / 256, cap = (uint64_t)g->sm_count * 16;
         return (unsigned)(b < cap ? b : cap);
     };
-    pack_ends_kernel<<<grid(blocks), 256, 0, s>>>(cs, blocks, s2);
+    pack_ends_kernel<<<grid(L.blocks), 256, 0, s>>>(cs, L.blocks, s2);
     pack_rows_kernel<<<grid((uint64_t)g->V + 1), 256, 0, s>>>(g->off, g->V, pack, s1, s2, rec);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? CSAW_OK : cuda_fail(e, "packed array launch");

@@ -30,12 +30,13 @@ namespace csaw {
 // without pushing the summaries out.
 //
 // Over the packed array (WC_PACK) the walk of RMAT s20 (1 M walkers x 80
-// steps) takes 1.46 ms and its construction 0.11, against 2.88 and 0.15 over
+// steps) takes 1.39 ms and its construction 0.11, against 2.88 and 0.15 over
 // summaries and weights: 133 DRAM bytes a step instead of 276 (a missing
 // sector is fetched as 64 bytes, so what one pick needs lies in one such
-// line), four dependent loads instead of ten.  Bound by their latency (DRAM
-// 4.5 TB/s, L2 65 % busy) at six blocks per SM; seven spill (1.90 ms), five
-// are even.
+// line), four dependent loads instead of ten.  Bound by scattered sectors (six
+// a step; a seventh cost 0.1 ms; DRAM 4.5 TB/s, L2 65 % busy), not by lanes:
+// leaving out the walkers that cannot move (38 %) made it slower.  Six blocks
+// per SM; seven spill (1.90 ms), five are even.
 constexpr int WC_THREADS = 256;
 constexpr int WC_WARPS = WC_THREADS / 32;
 constexpr int WC_TILE = 16;                  // path entries staged per walker
