@@ -26,7 +26,7 @@
 // row only costs a few more steps.  The index (4 bytes per edge + 40 per
 // vertex) and the weight summaries (csaw_graph.cu) are built in the call.
 //
-// Measured (RMAT s20 ef32, 1 M walkers, 40 steps): 157 ms with the index's
+// Measured (RMAT s20 ef32, 1 M walkers, 40 steps): 150 ms with the index's
 // construction (2.6 ms) against 459 ms for the streaming kernel.  Bound by
 // instruction issue and dependent loads together (issue active 59 %, DRAM 35 %
 // at 32 warps per SM; 24 or 40 warps are 7-9 % slower).
@@ -45,6 +45,8 @@ constexpr int N2V_B = 2;                      // look-ups per lane and batch
 constexpr uint32_t N2V_BATCH = 32 * N2V_B;
 constexpr uint32_t N2V_PREV = 0xFFFFFFFFu, N2V_NONE = 0xFFFFFFFEu;   // queue marks: prev itself, no entry
 constexpr uint32_t N2V_QUEUE = 32 * N2V_U + N2V_BATCH;
+constexpr uint32_t N2V_HOLD = 4;               // batches whose common neighbours are held
+constexpr uint32_t N2V_HELD = N2V_HOLD * N2V_BATCH;
 
 // Row v's index: the ids' span [first, first + span] in at most 2^k ranges of
 // 2^shift ids, k = floor(log2(d)) + N2V_SPREAD, in words {ids before the word,
@@ -206,25 +208,26 @@ __device__ __forceinline__ uint64_t n2v_sum(uint32_t x)
 }
 
 // A warp's shared buffers.
+template <bool WIDE>
 struct N2vShared {
     uint64_t cum[N2V_SLOTS];      // weight sum of the common neighbours up to the slot's end
-    uint64_t jw[N2V_BATCH];        // common neighbours held: running weight sum and position in N(cur)
+    typename N2vAcc<WIDE>::T jw[N2V_HELD];   // common neighbours held: running weight sum and position in N(cur)
     // ids whose bit is set, their index in the list (N2V_PREV: prev itself)
     // and the first position to compare
     uint2 at[N2V_QUEUE];
     uint32_t id[N2V_QUEUE];
     uint32_t pos[N2V_SLOTS];      // 1 + position in N(cur) of the slot's last common neighbour
     uint32_t from[N2V_SLOTS];     // list index of the slot's first queue entry
-    uint32_t jpos[N2V_BATCH];
+    uint32_t jpos[N2V_HELD];
 };
 
 // One step: the position in N(cur) of the pick for draw r; false at a dead
 // end.  cur/prev: the two lists; total: the row's weight sum.
-// WIDE: the sum of 32 weights may pass 2^32.
+// WIDE: the sum of N2V_HELD weights may pass 2^32.
 //
 // The shorter list is read 32 * N2V_U ids at a time; ids whose bit is
 // set in the longer list's index queue up, and N2V_BATCH queued ids at a time are
-// looked up exactly.  The common neighbours of the first batch are held, and
+// looked up exactly.  The common neighbours of the first N2V_HOLD batches are held, and
 // the pick is searched with them.  A step with more batches keeps, per slot
 // of G batches, the running weight sum and the last common position, which is
 // enough to place the draw in one slot; that slot's batches are then formed
@@ -233,7 +236,7 @@ struct N2vShared {
 // together.
 template <bool WIDE>
 __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, const N2vRow& prev, uint32_t prev_id,
-                                         uint64_t total, uint64_t r, N2vShared& sh, int lane, uint32_t* idx)
+                                         uint64_t total, uint64_t r, N2vShared<WIDE>& sh, int lane, uint32_t* idx)
 {
     const bool own = cur.d <= prev.d;
     const uint32_t* list = own ? cur.a : prev.a;
@@ -245,6 +248,7 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
     const uint64_t m2 = p.m2;
     const uint64_t dm1 = (uint64_t)p.m1 - m2;   // wrapping differences
     uint64_t run = 0, dp = 0, x = 0, before = 0;
+    typename N2vAcc<WIDE>::T held = 0;   // weight sum of those held
     uint32_t pp = 0xFFFFFFFFu, last_pos = 0, batch = 0, n_batches = 0, j0 = 0, from = 0, to = cur.d, nj = 0;
     auto S_at = [&](uint32_t pe, uint64_t cum) -> uint64_t {   // S of the first pe positions
         return pe == 0 ? 0ull : m2 * n2v_W(p, cur.beg, pe - 1) + dm1 * cum + (pp < pe ? dp : 0ull);
@@ -401,8 +405,11 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
                         left = G;
                     }
                 }
-                if (phase == 0 ? batch == 1 : placed) {
-                    nj = 0;
+                if (phase == 0 ? batch <= N2V_HOLD : placed) {
+                    if (phase == 1) {
+                        nj = 0;
+                        held = 0;
+                    }
 #pragma unroll
                     for (int t = 0; t < N2V_B; ++t) {
                         if (jb[t] == 0) continue;
@@ -415,9 +422,9 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
                         if ((jb[t] >> lane) & 1u) {
                             const uint32_t k = nj + __popc(jb[t] & lt);
                             sh.jpos[k] = pos[t];
-                            sh.jw[k] = run + incl;
+                            sh.jw[k] = held + incl;
                         }
-                        run += __shfl_sync(CSAW_FULL_MASK, incl, 31);
+                        held += __shfl_sync(CSAW_FULL_MASK, incl, 31);
                         nj += __popc(jb[t]);
                     }
                 }
@@ -454,7 +461,7 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
         const uint64_t T = m2 * total + dm1 * run + dp;
         if (T == 0) return false;
         x = scale_draw(r, T);
-        if (batch <= 1) break;
+        if (batch <= N2V_HOLD) break;
         // the slot: the first whose end exceeds x (the last slot's end is T)
         const uint32_t n_slots = slot + (left < G ? 1u : 0u);
         if (lane == 0) sh.pos[n_slots - 1] = cur.d;
@@ -482,7 +489,7 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
             const uint32_t mid = (lo + hi) >> 1;
             if (sh.jpos[mid] <= i) lo = mid + 1; else hi = mid;
         }
-        return m2 * W + dm1 * (lo ? sh.jw[lo - 1] : before) + (pp <= i ? dp : 0ull);
+        return m2 * W + dm1 * (before + (lo ? (uint64_t)sh.jw[lo - 1] : 0ull)) + (pp <= i ? dp : 0ull);
     };
     // the 8-edge group (numbered from the row's first): S at a group's end
     // needs a summary entry alone
@@ -521,7 +528,7 @@ __device__ __forceinline__ bool n2v_pick(const N2vParams& p, const N2vRow& cur, 
 template <bool WIDE, bool TELE>
 __global__ void __launch_bounds__(N2V_THREADS, 4) walk_n2v_kernel(N2vParams p)
 {
-    __shared__ N2vShared s_warp[N2V_WARPS];
+    __shared__ N2vShared<WIDE> s_warp[N2V_WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t row_len = (uint64_t)p.L + 1;
     while (true) {
@@ -682,7 +689,7 @@ csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bi
         p.m0 = bias->n2v_mult[0]; p.m1 = bias->n2v_mult[1]; p.m2 = bias->n2v_mult[2];
         p.tele = tele; p.tele_q32 = tele_q32;
         p.next_walker = next_walker;
-        const bool wide = max_bias * 32 >= (1ull << 32);
+        const bool wide = max_bias * N2V_HELD >= (1ull << 32);
         if (st == CSAW_OK)
             st = tele ? (wide ? launch_n2v_k<true, true>(p, g->sm_count, s) : launch_n2v_k<false, true>(p, g->sm_count, s))
                       : (wide ? launch_n2v_k<true, false>(p, g->sm_count, s) : launch_n2v_k<false, false>(p, g->sm_count, s));
