@@ -249,6 +249,16 @@ def cached_walk_bytes(torch, off_t, path, length):
     return (32 + 32 + 32 + 4 + 4) * n_trans + 8 * probes + 4 * n + 4 * n * (length + 1)
 
 
+def packed_walk_bytes(torch, off_t, path, length):
+    """Algorithmic bytes of one walk launch over the packed array: per step 32
+    (two vertex records) + 32 (one window of block ends) + 32 (a block's group
+    sums) + 64 (the group's biases and columns) + 4 (path entry); per walker 4
+    (start) and 4 * (L + 1) (its path row)."""
+    n_trans = int((path[:, 1:] != -1).sum())
+    n = path.shape[0]
+    return (32 + 32 + 32 + 64 + 4) * n_trans + 4 * n + 4 * n * (length + 1)
+
+
 def walk_workload(args):
     from paper_2009_09103_gb300 import inputs
     if args.workload == "node2vec":
@@ -275,12 +285,13 @@ def walk_mode(args, wl):
     """How the main line's walk gets its cumulative bias arrays: "build" (a
     static bias: the call builds the array over all rows, then every step is a
     search of it -- the array's construction is inside every timed step),
-    "cached" (--cdf: built once per graph, before timing) or "streaming"
-    (--streaming, or node2vec's dynamic bias: every step streams its row)."""
+    "cached" (--cdf: built once per graph, before timing) or "plain"
+    (--streaming, or node2vec's dynamic bias: the default call, which streams
+    rows or, at these sizes, builds what it searches by itself)."""
     if args.cdf:
         return "cached"
     if args.streaming or wl.bias == "node2vec":
-        return "streaming"
+        return "plain"
     return "build"
 
 
@@ -332,7 +343,6 @@ def run_walk_bench(args, rank, world):
     torch.cuda.synchronize()
     off_t = torch.from_numpy(g.off.astype(np.int64)).to(dev)
     n_trans, alg_bytes = (node2vec_bytes if wl.bias == "node2vec" else walk_bytes)(torch, off_t, path)
-    sector_bytes = walk_sector_bytes(torch, off_t, path) if wl.bias == "edge_weight" else None
 
     clocks = Clocks(dev.index)
     evs = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
@@ -383,18 +393,13 @@ def run_walk_bench(args, rank, world):
 
     wl_name = f"{args.workload}_s{args.scale}"
     kernels = {}
-    if mode == "streaming":
-        kname = "walk_kernel<NODE2VEC>" if wl.bias == "node2vec" else "walk_kernel<EDGE_WEIGHT>"
-        roofline = roofline_block(kname, traffic_record("csaw_walk.cu", wl_name), ms_per_step, alg_bytes,
-                                  sector_bytes)
-    elif wl.bias == "node2vec":
-        roofline = roofline_block("walk_kernel<NODE2VEC>", traffic_record("csaw_walk.cu", wl_name + "_cdf"),
-                                  ms_per_step, alg_bytes)
+    if wl.bias == "node2vec":
+        roofline = roofline_block("walk_n2v_kernel", traffic_record("csaw_walk_n2v.cu", wl_name), ms_per_step, alg_bytes)
     else:
         # the step's phases timed by CUDA events on the step's stream inside
         # the call (the array's construction, then the walk kernels); the
         # paths checked against the graph's prebuilt array
-        cb = cached_walk_bytes(torch, off_t, path, wl.length)
+        cb = packed_walk_bytes(torch, off_t, path, wl.length)
         ms_walk = ms_per_step
         if mode == "build":
             ph = []
@@ -415,9 +420,9 @@ def run_walk_bench(args, rank, world):
             kernels = {"walk_cached_kernel_ms": ms_walk,
                        "cumulative_array_build_ms": ms_build,
                        "basis": "CUDA events on the step's stream around each phase inside the call (phase_ms)",
-                       "build_algorithmic_bytes": 4 * g.E + 9 * g.E // 8 + 40 * g.V,
+                       "build_algorithmic_bytes": 16 * g.E + 5 * g.E // 8 + 24 * g.V,
                        "identical_paths_graph_array": same}
-            recs = traffic_records("csaw_graph.cu", wl_name + "_build")
+            recs = traffic_records("csaw_pack.cu", wl_name + "_build")
             if recs and ms_build > 0:
                 peak, peak_kind = measured_peaks()
                 dram = sum(r["traffic_bytes_per_launch"] for r in recs)
@@ -425,14 +430,12 @@ def run_walk_bench(args, rank, world):
                 kernels["build_dram_gbs"] = round(dram / (ms_build / 1e3) / 1e9, 1)
                 kernels["build_dram_frac"] = round(dram / (ms_build / 1e3) / 1e9 / peak, 4)
                 kernels["build_kernels"] = sorted(r["kernel"] for r in recs)
-        kn = "walk_cached_kernel<WEIGHTS>" if mode == "build" else "walk_cached_kernel<LEAF>"
-        roofline = roofline_block(kn, traffic_record("csaw_walk_cdf.cu", wl_name + ("_build" if mode == "build" else "_cdf")),
+        roofline = roofline_block("walk_cached_kernel<PACK>", traffic_record("csaw_walk_cdf.cu", wl_name + "_pack"),
                                   ms_walk, cb)
-    cum = {"build": "built over all rows inside every step (segmented scan over edge tiles into summaries of the "
-                    "prefix sums and per-vertex records; each step bisects the summaries and sums one 32-byte "
-                    "group of weights)",
-           "cached": "cached per edge (built once per graph, before timing)",
-           "streaming": "computed per step (streamed over the row)"}[mode]
+    cum = {"build": "built over all rows inside every step (one running sum over all edges, biases packed beside "
+                    "columns; each step reads a window of block ends, a block's group sums and one group)",
+           "cached": "built once per graph, before timing",
+           "plain": "the default call's choice (at this size built inside the call)"}[mode]
     result = {
         "metric": METRIC, "value": value, "unit": "edges/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
@@ -443,7 +446,9 @@ def run_walk_bench(args, rank, world):
                    "l2": "flushed (512 MiB write) before every timed step",
                    "cumulative_array": cum,
                    "sampled_edges_per_step": n_trans},
-        "gpu_launches": args.steps * (4 if mode == "build" else 1),
+        # build: four kernels and the walk; node2vec: five for the weights'
+        # sums, two for the row index and the walk
+        "gpu_launches": args.steps * (8 if wl.bias == "node2vec" else 1 if mode == "cached" else 5),
         "roofline": roofline,
         "e2e": e2e,
     }
@@ -452,19 +457,15 @@ def run_walk_bench(args, rank, world):
     if clk:
         result["clocks"] = clk
     if mode == "build" and not args.no_variant:
-        # The per-visit streaming walk (each step streams its row's biases):
-        # the same paths, timed the same way.
+        # The default call (no build_cdf): the same paths, timed the same way.
         path3 = torch.empty_like(path)
         t_s = time_steps(torch, lambda: csaw.walk(G, starts, wl.length, wl.bias, seed, wl.n2v_mult,
                                                   path=path3, stream=stream),
                          args.steps, args.warmup, stream, flush)
         ms3 = sum(t_s) / len(t_s)
-        result["streaming_per_visit"] = {
+        result["plain_call"] = {
             "value": n_trans * world / (ms3 / 1e3), "unit": "edges/s", "ms_per_step": ms3,
-            "kernel": "walk_kernel", "identical_paths": bool(torch.equal(path, path3)),
-            "roofline": roofline_block("walk_kernel<EDGE_WEIGHT>", traffic_record("csaw_walk.cu", wl_name), ms3,
-                                       alg_bytes, sector_bytes)}
-        result["gpu_launches_streaming"] = args.steps
+            "identical_paths": bool(torch.equal(path, path3))}
     G.close()
     return result, (g, wl, n_trans)
 
@@ -832,7 +833,7 @@ def run_mdrw_bench(args):
                                "degree, EdgeBias = 1",
                    "l2": "flushed (512 MiB write) before every timed step", "sampled_edges_per_step": n_edges},
         "gpu_launches": args.steps,
-        "roofline": roofline_block("mdrw_kernel", tr, ms, alg),
+        "roofline": roofline_block("mdrw_chain_kernel", tr, ms, alg),
         "e2e": {"value": n_edges / e2e_s, "unit": "edges/s", "h2d_bytes_per_step": 4 * n * m,
                 "d2h_bytes_per_step": 8 * n * wl.steps, "matches_device_run": same},
     }
@@ -931,7 +932,7 @@ def run_layer_bench(args):
                                f"depth 2, {wl.fanout} picks per instance and layer, edge-weight bias",
                    "l2": "flushed (512 MiB write) before every timed step", "sampled_edges_per_step": edges,
                    "cumulative_array": "cached per edge" if args.cdf else "computed per selection"},
-        "roofline": roofline_block("layer_select_kernel", tr, ms, alg),
+        "roofline": roofline_block("layer_draw_kernel", tr, ms, alg),
         "e2e": {"value": edges / e2e_s, "unit": "edges/s", "h2d_bytes_per_step": 4 * len(wl.seeds) + 8 * (n_inst + 1),
                 "d2h_bytes_per_step": 8 * edges},
     }
@@ -1263,7 +1264,7 @@ def main():
                              "attempts"])
     ap.add_argument("--autotune", action="store_true", help="sampling workloads: autotune first")
     ap.add_argument("--no-variant", action="store_true",
-                    help="walks: skip the per-visit streaming walk measured after the main line")
+                    help="walks: skip the default call measured after the main line")
     ap.add_argument("--streaming", action="store_true",
                     help="walks: the main line streams each step's row (no cumulative array)")
     ap.add_argument("--cdf", action="store_true",

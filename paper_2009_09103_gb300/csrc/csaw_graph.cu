@@ -76,7 +76,9 @@ void free_with(const DevAllocator& a, void* p, cudaStream_t s)
 }
 
 // The library's own stream-ordered pool, one per device.  Freed blocks stay
-// in it (they are not returned at every synchronisation), and a block freed
+// in it, up to an eighth of the device's memory (what is above that goes back
+// at the next synchronisation: a walk over a large graph makes temporaries of
+// several bytes per edge), and a block freed
 // on one stream is reused on another only once that free has completed: the
 // pool never makes an allocation wait for work queued on another stream, so
 // one server slot's buffers never wait for another slot's kernels.
@@ -99,7 +101,13 @@ static cudaError_t lib_pool(cudaMemPool_t* out)
     cudaMemPool_t pool;
     e = cudaMemPoolCreate(&pool, &props);
     if (e != cudaSuccess) return e;
-    uint64_t keep = UINT64_MAX;
+    size_t free_bytes = 0, total_bytes = 0;
+    e = cudaMemGetInfo(&free_bytes, &total_bytes);
+    if (e != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+    }
+    uint64_t keep = total_bytes / 8;
     int no = 0;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);

@@ -2765,7 +2765,7 @@ static csaw_status enqueue_layer_count(Pipeline& P, uint32_t l, cudaStream_t s)
 // block where layer_select_kernel runs a warp per instance.
 static bool layer_draws(const Pipeline& P, uint32_t l, const uint64_t* pack)
 {
-    return !P.zero_bias && P.fanout[l] <= LD_MAX_K && P.attempt_cap >= LD_MIN_CAP &&
+    return !P.zero_bias && P.fanout[l] <= LD_MAX_K && P.attempt_cap >= LD_MIN_CAP && P.n_inst <= 0x7FFFFFFFu &&
            (pack || P.kind == CSAW_BIAS_UNIFORM);
 }
 
