@@ -4,6 +4,8 @@
 // graph object and error plumbing.  Everything here is written for sm_103a.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
@@ -184,6 +186,25 @@ csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bi
                      uint32_t length, uint64_t rng_seed, uint32_t tele, uint32_t tele_q32, uint32_t* path,
                      unsigned long long* next_walker, cudaStream_t s, bool* done);
 // Whether a call of n walks of `length` steps is large enough for it.
+// The mean degree of the rows that a walk or a sampled layer comes to, for the
+// rules that weigh streaming rows against building an array: sqrt(mean degree *
+// largest degree) where edges are followed by weight (RMAT s16 520 for 684
+// measured, s20 1393 for 2233, s20 ef32 2424 for 3315), nearer the largest
+// degree where they are followed by degree, and the degree itself on a regular
+// graph.
+inline double visited_degree(const csaw_graph* g, bool by_degree)
+{
+    const double avg = g->V ? (double)g->E / (double)g->V : 0.0, most = (double)g->max_degree;
+    return by_degree ? std::cbrt(avg * most * most) : std::sqrt(avg * most);
+}
+
+// The longest row that n walkers stand at in one step, for the same rules: a
+// call ends no sooner than the walker whose rows are longest.
+inline double longest_row(const csaw_graph* g, double n, bool by_degree)
+{
+    return std::min((double)g->max_degree, std::sqrt(n) * visited_degree(g, by_degree));
+}
+
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length);
 
 // Whether selection/walks of this kind can use a cached cumulative array:

@@ -2277,7 +2277,7 @@ struct Pipeline {
 // items and the hubs' own prefix sums (150 us in small runs, and 150 per
 // frontier entry in large ones: RMAT s12 to s22); with one, whose long rows a
 // block each would scan, about 2 per neighbour of a row reached by an edge
-// (see walk_array_pays).  A frontier is taken as eight times the one before,
+// (see visited_degree).  A frontier is taken as eight times the one before,
 // most rows being short.  The batched s22 plan (2048 instances, 32 M edges of
 // frontier) draws its long rows in 4.9 ms, with 0.6 for the array, against 8.3
 // over shared hub arrays.
@@ -2285,7 +2285,7 @@ static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
 {
     const csaw_graph* g = P.g;
     if (P.kind == CSAW_BIAS_UNIFORM || P.cached || P.zero_bias || !pack_fits(g, P.kind) || n_seeds == 0) return false;
-    const double visited = std::sqrt((double)g->E / (double)g->V * (double)g->max_degree);
+    const double visited = visited_degree(g, false);
     double entries = 0, reached = 0, f = (double)n_seeds;
     for (uint32_t l = 0; l < P.depth; ++l) {
         entries += f;
@@ -2771,21 +2771,27 @@ static bool layer_draws(const Pipeline& P, uint32_t l, const uint64_t* pack)
 
 // Whether building the packed array for one layer-sampling call pays.  In ps:
 // layer_select_kernel's pass over the pool takes about 5 per edge with the
-// chip full and its picks about 2 us each in turn (512 picks from 500 rows);
-// the array takes 4 per edge of the graph (8 where degrees are gathered) and
-// 25 us.  Rows of later layers are reached by degree (see walk_array_pays).
+// chip full, 9000 per edge of the instance's own pool, which one warp reads
+// (RMAT s20: 10,000 by weight, 28,000 by degree), and its picks about 2 us each
+// in turn (512 picks from 500 rows); the array takes 4 per edge of the graph (6
+// where degrees are gathered) and 25 us.  Rows of later layers are reached by
+// an edge.  Fanout [8, 8] of 16 instances of 16 seeds by degree, streamed and
+// over the array: RMAT s16 570 and 309 us, s20 1714 and 467; 1000 instances of
+// 64 seeds, [20, 20], s20 3679 and 643.
 static bool layer_array_pays(const Pipeline& P, uint64_t n_seeds)
 {
     const csaw_graph* g = P.g;
-    const double avg = (double)g->E / (double)g->V, visited = std::sqrt(avg * (double)g->max_degree);
+    const bool by_degree = P.kind == CSAW_BIAS_NEIGHBOR_DEGREE;
+    const double avg = (double)g->E / (double)g->V, n_inst = std::max<double>(P.n_inst, 1.0);
     double cost = 0, f = (double)n_seeds;
     bool any = false;
     for (uint32_t l = 0; l < P.depth; ++l) {
-        cost += 5.0 * f * (l ? visited : avg) + 2e6 * P.fanout[l];
-        f = (double)P.n_inst * P.fanout[l];
+        const double pool = f * (l ? visited_degree(g, by_degree) : avg);
+        cost += std::max(5.0 * pool, 9e3 * pool / n_inst) + 2e6 * P.fanout[l];
+        f = n_inst * P.fanout[l];
         any |= P.fanout[l] <= LD_MAX_K;
     }
-    return any && cost >= (P.kind == CSAW_BIAS_NEIGHBOR_DEGREE ? 8.0 : 4.0) * (double)g->E + 25e6;
+    return any && cost >= (by_degree ? 6.0 : 4.0) * (double)g->E + 25e6;
 }
 
 // Layer l of layer sampling: the picks of every instance, then the offsets.

@@ -622,17 +622,20 @@ static csaw_status launch_n2v_k(const N2vParams& p, int sm_count, cudaStream_t s
     return CSAW_OK;
 }
 
-// Streaming a step costs about 5.5 ps per neighbour of the row with the chip
-// full (RMAT s20 ef32: 18 ns per step at a mean visited degree of 3,315), the
-// index and summaries about 18 ps per edge and ten launches, and a step over
-// them about a third of a streamed one.  The mean visited degree is taken as
-// sqrt(mean degree * largest degree): 2,424 there, and the degree itself on a
-// regular graph.
+// In ps: streaming a step costs about 5.5 per neighbour of the row with the
+// chip full (RMAT s20 ef32: 18 ns per step at a mean visited degree of 3,315),
+// and a step of the walker at the longest row 4 us and 800 per neighbour
+// however few walk beside it; a step over the index takes about a third.  The
+// index and summaries take about 18 per edge, and 10 us of launches (40 where
+// too few walk to hide the first pass over them).  60 steps of 256 walkers,
+// streamed and over the index: RMAT s16 1161 and 556 us, s20 3088 and 1722.
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length)
 {
     if (g->E == 0 || g->max_degree > 0x7FFFFFFFu) return false;   // positions plus 8 fit 32 bits
-    const double visited = std::sqrt((double)g->E / (double)g->V * (double)g->max_degree);
-    return (double)n * (double)length * visited >= 5.0 * (double)g->E + 2e6;
+    const double full = 5.5 * (double)n * visited_degree(g, false);
+    const double longest = 4e6 + 800.0 * longest_row(g, (double)n, false);
+    const double gain = (double)length * 2.0 / 3.0, cost = 18.0 * (double)g->E;
+    return gain * full >= cost + 10e6 || gain * longest >= cost + 40e6;
 }
 
 csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,
