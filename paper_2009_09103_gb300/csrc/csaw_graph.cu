@@ -49,6 +49,14 @@ AllocScope::AllocScope(const csaw_graph* g) : prev(t_alloc)
 
 AllocScope::~AllocScope() { t_alloc = prev; }
 
+static thread_local uint64_t t_array_room = UINT64_MAX;
+
+uint64_t array_room() { return t_array_room; }
+
+ArrayRoom::ArrayRoom(uint64_t bytes) : prev(t_array_room) { t_array_room = bytes; }
+
+ArrayRoom::~ArrayRoom() { t_array_room = prev; }
+
 csaw_status alloc_with(const DevAllocator* a, void** p, size_t bytes, cudaStream_t s)
 {
     *p = nullptr;

@@ -87,6 +87,17 @@ struct AllocScope {
     ~AllocScope();
 };
 
+// Device bytes that an entry point on this thread may take for an array that
+// its caller did not ask for (built because the call is large enough that it
+// pays): all there are, except inside a scope that says less.  The request
+// server's batches may take what the budget has left beside the estimates.
+uint64_t array_room();
+struct ArrayRoom {
+    uint64_t prev;
+    explicit ArrayRoom(uint64_t bytes);
+    ~ArrayRoom();
+};
+
 // Allocation and release through an explicit allocator (null or empty:
 // cudaMalloc / cudaFree), for memory that outlives the call that made it.
 csaw_status alloc_with(const DevAllocator* a, void** p, size_t bytes, cudaStream_t s);
@@ -198,13 +209,17 @@ inline double visited_degree(const csaw_graph* g, bool by_degree)
     return by_degree ? std::cbrt(avg * most * most) : std::sqrt(avg * most);
 }
 
-// The longest row that n walkers stand at in one step, for the same rules: a
-// call ends no sooner than the walker whose rows are longest.
-inline double longest_row(const csaw_graph* g, double n, bool by_degree)
+// The neighbours that the slowest of n walkers streams in `length` steps, for
+// the same rules: a call ends no sooner than that walker, which meets rows far
+// longer than the mean (RMAT s20, 60 steps: fits 16 to 4,000 walkers' times).
+inline double slowest_walk(const csaw_graph* g, double n, double length, bool by_degree)
 {
-    return std::min((double)g->max_degree, std::sqrt(n) * visited_degree(g, by_degree));
+    const double visited = visited_degree(g, by_degree);
+    return length * visited + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * visited);
 }
 
+// Device bytes of node2vec's row index and sums, built for one call.
+uint64_t n2v_bytes(const csaw_graph* g);
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length);
 
 // Whether selection/walks of this kind can use a cached cumulative array:

@@ -2285,6 +2285,7 @@ static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
 {
     const csaw_graph* g = P.g;
     if (P.kind == CSAW_BIAS_UNIFORM || P.cached || P.zero_bias || !pack_fits(g, P.kind) || n_seeds == 0) return false;
+    if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const double visited = visited_degree(g, false);
     double entries = 0, reached = 0, f = (double)n_seeds;
     for (uint32_t l = 0; l < P.depth; ++l) {

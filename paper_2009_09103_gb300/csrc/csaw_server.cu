@@ -569,6 +569,21 @@ struct csaw_server {
         }
     }
 
+    // Device bytes set aside, beside the estimates, for an array that the batch
+    // may build: an array of this graph, where the budget has that much left
+    // and a slot's arrays stay below half its share.  Otherwise rows are
+    // streamed, within the estimate (RMAT s26: an array is 18 GB).  Called with
+    // mu held, the batch's estimates in in_use.
+    uint64_t reserve_array(const std::vector<Request*>& batch) const
+    {
+        const Request* head = batch[0];
+        const int kind = head->bias.kind;
+        if (kind == CSAW_BIAS_UNIFORM || (head->kind == CSAW_REQ_WALK && batch.size() > 1)) return 0;
+        const uint64_t bytes = kind == CSAW_BIAS_NODE2VEC ? n2v_bytes(g)
+                                                          : sizeof(uint64_t) * pack_layout(g->E, g->V).words;
+        return bytes <= budget / (2 * (uint64_t)slots) && bytes <= budget - in_use ? bytes : 0;
+    }
+
     void worker(uint32_t slot)
     {
         cudaSetDevice(g->device);
@@ -587,12 +602,18 @@ struct csaw_server {
                 rq->state = Request::RUNNING;
                 rq->result->t_admit_ns = t_admit;
             }
+            const uint64_t array = reserve_array(batch);
+            in_use += array;
             lk.unlock();
             const int64_t t_start = now_ns();
             for (Request* rq : batch) rq->result->t_start_ns = t_start;
-            execute(g, L, batch);
+            {
+                ArrayRoom room(array);
+                execute(g, L, batch);
+            }
             const int64_t t_finish = now_ns();
             lk.lock();
+            in_use -= array;
             for (Request* rq : batch) {
                 rq->result->t_finish_ns = t_finish;
                 in_use -= rq->estimate;

@@ -926,18 +926,20 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
 
 // Whether building the packed array for one call pays.  In ps: streaming a
 // step costs about 250 + 0.3 per neighbour of the row with the chip full (RMAT
-// s16 to s20; 1.0 and more where degrees are gathered), and a step of the
-// walker at the longest row 125 per neighbour however few walk beside it
-// (degrees 400); the array takes 4 per edge (degrees 5 to 6) and its launches
-// 25 us.  60 steps of 256 walkers on RMAT s20, streamed and over the array:
-// 363 and 269 us by weight, 1890 and 354 by degree; 10 steps by degree 371 and
-// 205.
+// s16 to s20; 1.0 and more where degrees are gathered), and the slowest walker
+// 750 per neighbour however few walk beside it (degrees 1300); the array takes
+// 4 per edge (degrees 5 to 6), its launches 25 us, and a few walkers half a us
+// a step more than streaming short rows.  60 steps of 256 walkers on RMAT s20,
+// streamed and over the array: 363 and 274 us by weight, 1890 and 358 by
+// degree; 10 steps by degree 371 and 205.
 static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length)
 {
+    if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const bool by_degree = kind == CSAW_BIAS_NEIGHBOR_DEGREE;
-    const double full = (double)n * (250.0 + (by_degree ? 1.0 : 0.3) * visited_degree(g, by_degree));
-    const double longest = (by_degree ? 400.0 : 125.0) * longest_row(g, (double)n, by_degree);
-    return (double)length * std::max(full, longest) >= (by_degree ? 6.0 : 4.0) * (double)g->E + 25e6;
+    const double full = (double)n * (double)length * (250.0 + (by_degree ? 1.0 : 0.3) * visited_degree(g, by_degree));
+    const double slowest = (by_degree ? 1300.0 : 750.0) * slowest_walk(g, (double)n, (double)length, by_degree);
+    const double cost = (by_degree ? 6.0 : 4.0) * (double)g->E + 25e6;
+    return full >= cost || slowest >= cost + 0.5e6 * (double)length;
 }
 
 // CUDA events around a call's phases, when the caller asks for their times:

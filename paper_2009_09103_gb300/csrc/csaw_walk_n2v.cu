@@ -622,20 +622,29 @@ static csaw_status launch_n2v_k(const N2vParams& p, int sm_count, cudaStream_t s
     return CSAW_OK;
 }
 
+uint64_t n2v_bytes(const csaw_graph* g)
+{
+    const uint64_t sums = g->w && !g->cdf[CSAW_BIAS_EDGE_WEIGHT] ? sizeof(uint64_t) * wsum_layout(g->E, g->V).words : 0;
+    return sums + sizeof(uint2) * n2v_index_words(g->E, g->V) + sizeof(uint64_t) * (4 * (uint64_t)g->V + 1) +
+           sizeof(uint32_t) * (g->E / N2V_BIG_ROW + 2);
+}
+
 // In ps: streaming a step costs about 5.5 per neighbour of the row with the
 // chip full (RMAT s20 ef32: 18 ns per step at a mean visited degree of 3,315),
-// and a step of the walker at the longest row 4 us and 800 per neighbour
-// however few walk beside it; a step over the index takes about a third.  The
-// index and summaries take about 18 per edge, and 10 us of launches (40 where
-// too few walk to hide the first pass over them).  60 steps of 256 walkers,
-// streamed and over the index: RMAT s16 1161 and 556 us, s20 3088 and 1722.
+// and a step of the slowest walker 4.5 us and 6000 per neighbour however few
+// walk beside it; a step over the index takes about a third of the first and
+// two fifths of the second.  The index and summaries take about 18 per edge,
+// and 10 us of launches (50 where too few walk to fill the chip).  60 steps of
+// 256 walkers, streamed and over the index: RMAT s16 1161 and 556 us, s20 3088
+// and 1726.
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length)
 {
     if (g->E == 0 || g->max_degree > 0x7FFFFFFFu) return false;   // positions plus 8 fit 32 bits
-    const double full = 5.5 * (double)n * visited_degree(g, false);
-    const double longest = 4e6 + 800.0 * longest_row(g, (double)n, false);
-    const double gain = (double)length * 2.0 / 3.0, cost = 18.0 * (double)g->E;
-    return gain * full >= cost + 10e6 || gain * longest >= cost + 40e6;
+    if (n2v_bytes(g) > array_room()) return false;
+    const double full = 5.5 * (double)n * (double)length * visited_degree(g, false);
+    const double slowest = 4.5e6 * (double)length + 6e3 * slowest_walk(g, (double)n, (double)length, false);
+    const double cost = 18.0 * (double)g->E;
+    return full * 2.0 / 3.0 >= cost + 10e6 || slowest * 0.6 >= cost + 50e6;
 }
 
 csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,
