@@ -192,7 +192,8 @@ struct ServerResult {
 // copy engine serves copies in the order they were issued, and a small walk's
 // would wait for those of large walks issued before it, whose kernels still
 // run.  A walk of 500 behind three of 32,768: 4 us after the last of them in
-// one run of seven by the copy engine, 150 us and more before it in all runs so.
+// one run of seven by the copy engine; so, a median of 170 us before it, and behind
+// it in none of 118 but for a process's first.
 __global__ void result_out_kernel(const uint32_t* __restrict__ src, uint64_t n, uint32_t* __restrict__ dst)
 {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
