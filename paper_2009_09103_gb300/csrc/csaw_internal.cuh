@@ -395,6 +395,7 @@ struct SampleTables {
     const uint32_t* inst_key;
     const uint32_t* inst_id;
     const uint32_t* inst_fan;
+    const uint32_t* fan_finite;   // host: per layer the largest fanout that is not CSAW_FANOUT_ALL
 };
 csaw_status sample_batch(csaw_graph* g, const uint32_t* d_seeds, const uint64_t* d_inst_off, uint32_t n_inst,
                          uint64_t n_seeds, uint32_t depth, const uint32_t* fan_max, const SampleTables& t,

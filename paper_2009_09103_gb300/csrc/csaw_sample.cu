@@ -2166,7 +2166,7 @@ struct Pipeline {
     bool take = true;                    // whole short rows by take_all_kernel
     bool hub_path = false;               // shared hub arrays per layer (static bias, streamed)
     bool hub_order = false;              // cached static bias: hub items visited in vertex order
-    bool any_big_k = false;              // some layer takes more than PICK_MAX picks
+    uint32_t finite[CSAW_MAX_DEPTH] = {};   // the largest fanout of a layer that is not CSAW_FANOUT_ALL
     uint32_t attempt_cap = CSAW_ATTEMPT_CAP;
     uint32_t k0 = 0, k1 = 0;
     const uint32_t* key_dev = nullptr;   // plan mode: Philox key in device memory
@@ -2225,9 +2225,7 @@ struct Pipeline {
         cached = cached_cdf_usable(g, kind);
         if (cached && kind != CSAW_BIAS_UNIFORM) pack = g->pack[kind];
         paths();
-        bool big_k = false;
-        for (uint32_t l = 0; l < dep; ++l) big_k |= fan[l] > PICK_MAX && fan[l] != CSAW_FANOUT_ALL;
-        any_big_k = big_k;
+        for (uint32_t l = 0; l < dep; ++l) finite[l] = fan[l] == CSAW_FANOUT_ALL ? 0u : fan[l];
         k0 = (uint32_t)seed;
         k1 = (uint32_t)(seed >> 32);
     }
@@ -2256,11 +2254,18 @@ struct Pipeline {
                     (!pack || (seeds_cap >= (1u << 19) && g->E >= (1u << 24)));
     }
 
+    // Whether no entry of layer l draws more than PICK_MAX picks.  Whole rows
+    // are no draws, so that is a matter of the finite fanouts: instances of
+    // several requests may take CSAW_FANOUT_ALL beside, say, 300.
+    bool few(uint32_t l) const { return finite[l] <= PICK_MAX; }
+
     // CTA items exist for picks above PICK_MAX (or, without the hub path, any
     // long row); only rows above CTA_SMEM_DEG need a slot.
     bool cta_slots() const
     {
-        return g->max_degree > CTA_SMEM_DEG && (any_big_k || (!cached && !hub_path));
+        bool big_k = false;
+        for (uint32_t l = 0; l < depth; ++l) big_k |= !few(l);
+        return g->max_degree > CTA_SMEM_DEG && (big_k || (!cached && !hub_path));
     }
 
     // Capacities of a layer's per-entry and edge arrays.
@@ -2501,10 +2506,10 @@ static csaw_status enqueue_select_items(Pipeline& P, uint32_t l, cudaStream_t s)
             }
             CSAW_CUDA(cudaGetLastError());
         }
-        // with shared hub arrays a CTA item needs more than PICK_MAX picks: a
-        // layer whose fanout is at most that holds warp items only, launched
-        // with their slots alone (more resident blocks hide the gathers)
-        const bool few = P.fanout[l] <= PICK_MAX || P.fanout[l] == CSAW_FANOUT_ALL;
+        // with shared hub arrays or the packed array a CTA item needs more than
+        // PICK_MAX picks: a layer without such draws holds warp items only,
+        // launched with their slots alone (more resident blocks hide the gathers)
+        const bool few = P.few(l);
         const bool warp_only = (P.hub_path || P.pack) && few;
         const bool wide = select_wide(g, P.kind);
         int blocks = P.sel_blocks;
@@ -2849,6 +2854,7 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
         P.inst_key = tabs->inst_key;
         P.inst_id = tabs->inst_id;
         P.inst_fan = tabs->inst_fan;
+        for (uint32_t l = 0; l < depth; ++l) P.finite[l] = tabs->fan_finite[l];
     }
     if (!layer_mode && sample_array_pays(P, n_seeds)) {
         uint64_t* words = nullptr;

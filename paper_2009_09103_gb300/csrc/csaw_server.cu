@@ -399,7 +399,7 @@ static csaw_status execute_samples(csaw_graph* g, Lane& L, std::vector<Request*>
     uint32_t* h_id = (uint32_t*)(L.pin + o_id);
     uint32_t* h_fan = (uint32_t*)(L.pin + o_fan);
     uint32_t* h_seeds = (uint32_t*)(L.pin + o_seeds);
-    std::vector<uint32_t> fan_max(depth, 0);
+    std::vector<uint32_t> fan_max(depth, 0), fan_finite(depth, 0);
     uint64_t i0 = 0, s0 = 0;
     for (Request* rq : batch) {
         for (uint32_t i = 0; i < rq->n_instances; ++i) {
@@ -410,8 +410,11 @@ static csaw_status execute_samples(csaw_graph* g, Lane& L, std::vector<Request*>
             for (uint32_t l = 0; l < depth; ++l)
                 h_fan[(uint64_t)l * N + i0 + i] = l < rq->fanout.size() ? rq->fanout[l] : 0u;
         }
-        for (uint32_t l = 0; l < rq->fanout.size(); ++l)
-            fan_max[l] = rq->fanout[l] > fan_max[l] ? rq->fanout[l] : fan_max[l];
+        for (uint32_t l = 0; l < rq->fanout.size(); ++l) {
+            const uint32_t k = rq->fanout[l];
+            if (k > fan_max[l]) fan_max[l] = k;
+            if (k != CSAW_FANOUT_ALL && k > fan_finite[l]) fan_finite[l] = k;
+        }
         if (!rq->seeds.empty()) std::memcpy(h_seeds + s0, rq->seeds.data(), 4 * rq->seeds.size());
         i0 += rq->n_instances;
         s0 += rq->seeds.size();
@@ -431,6 +434,7 @@ static csaw_status execute_samples(csaw_graph* g, Lane& L, std::vector<Request*>
         t.inst_key = (const uint32_t*)(d + o_key);
         t.inst_id = (const uint32_t*)(d + o_id);
         t.inst_fan = (const uint32_t*)(d + o_fan);
+        t.fan_finite = fan_finite.data();
         st = sample_batch(g, (const uint32_t*)(d + o_seeds), (const uint64_t*)(d + o_io), (uint32_t)N, S, depth,
                           fan_max.data(), t, kind, L.s, &R);
     }
