@@ -321,7 +321,8 @@ csaw_status csaw_walk_oom_ex(const uint64_t* row_offsets, const uint32_t* cols, 
  *   device_budget_bytes  the device memory of one partition slot: vertex
  *                 ranges are cut so that a range's columns, weights and the
  *                 prefix sums of its hub rows fit it (16 bytes per edge; see
- *                 csaw_oom_plan with weighted = 1)
+ *                 csaw_oom_plan with weighted = 1; the slot's arrays take 64
+ *                 bytes of padding each beyond it)
  *   seeds, inst_offsets, n_instances, depth, fanout, bias, rng_seed
  *                 host arrays and arguments as for csaw_sample (bias: uniform,
  *                 edge weight or neighbour degree)

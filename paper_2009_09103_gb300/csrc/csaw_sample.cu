@@ -3481,6 +3481,10 @@ struct OomSlot {
     cudaEvent_t freed = nullptr;       // the selection that read it is done
 };
 
+// Words of a slot's column and weight arrays: whole 32-byte sectors are read of
+// a row (sector_biases), so there are some past the last edge, as on a resident graph.
+uint64_t oom_slot_words(uint64_t slot_edges) { return slot_edges + CSAW_EDGE_PAD; }
+
 }  // namespace csaw
 
 extern "C" csaw_status csaw_sample_oom(const uint64_t* row_offsets, const uint32_t* cols, const uint32_t* weights,
@@ -3582,8 +3586,8 @@ extern "C" csaw_status csaw_sample_oom(const uint64_t* row_offsets, const uint32
         cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
         if (e != cudaSuccess) { st = cuda_fail(e, "cudaStreamCreate"); break; }
         for (auto& sl : slot) {
-            st = get((void**)&sl.col, sizeof(uint32_t) * slot_edges);
-            if (st == CSAW_OK && weighted) st = get((void**)&sl.w, sizeof(uint32_t) * slot_edges);
+            st = get((void**)&sl.col, sizeof(uint32_t) * oom_slot_words(slot_edges));
+            if (st == CSAW_OK && weighted) st = get((void**)&sl.w, sizeof(uint32_t) * oom_slot_words(slot_edges));
             if (st == CSAW_OK) st = get((void**)&sl.hubS, sizeof(uint64_t) * slot_edges);
             if (st != CSAW_OK) break;
             e = cudaEventCreateWithFlags(&sl.loaded, cudaEventDisableTiming);
