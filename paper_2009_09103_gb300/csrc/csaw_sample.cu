@@ -2833,10 +2833,12 @@ static csaw_status enqueue_layer_select(Pipeline& P, uint32_t l, uint64_t* VP, u
 }
 
 // csaw_sample: exact edge buffers, one wait per layer.
-static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64_t* inst_off,
+// may_build: whether the packed array may be built where it pays; *built: it was.
+static csaw_status run_layers(csaw_graph* g, const uint32_t* seeds, const uint64_t* inst_off,
                               uint32_t n_inst, uint64_t n_seeds, uint32_t depth, const uint32_t* fanout,
                               int kind, uint64_t rng_seed, uint32_t attempt_cap, bool layer_mode,
-                              cudaStream_t s, csaw_sample_result* R, const SampleTables* tabs = nullptr)
+                              cudaStream_t s, csaw_sample_result* R, const SampleTables* tabs, bool may_build,
+                              bool* built)
 {
     Temps tmp(s);
     auto get = [&](void** p, size_t bytes) -> csaw_status {
@@ -2856,10 +2858,11 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
         P.inst_fan = tabs->inst_fan;
         for (uint32_t l = 0; l < depth; ++l) P.finite[l] = tabs->fan_finite[l];
     }
-    if (!layer_mode && sample_array_pays(P, n_seeds)) {
+    if (may_build && !layer_mode && sample_array_pays(P, n_seeds)) {
         uint64_t* words = nullptr;
         const csaw_status st = get((void**)&words, sizeof(uint64_t) * pack_layout(g->E, g->V).words);
         if (st == CSAW_OK) {
+            *built = true;
             CSAW_TRY(enqueue_pack_build(g, kind, words, s));
             P.use_pack(words);
         } else if (st == CSAW_ERR_NOMEM) {
@@ -2880,10 +2883,11 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
     const uint64_t* pack = nullptr;
     if (layer_mode && P.kind != CSAW_BIAS_UNIFORM && !P.zero_bias && attempt_cap >= LD_MIN_CAP) {
         pack = g->pack[P.kind];
-        if (!pack && pack_fits(g, P.kind) && layer_array_pays(P, n_seeds)) {
+        if (!pack && may_build && pack_fits(g, P.kind) && layer_array_pays(P, n_seeds)) {
             uint64_t* words = nullptr;
             const csaw_status st = get((void**)&words, sizeof(uint64_t) * pack_layout(g->E, g->V).words);
             if (st == CSAW_OK) {
+                *built = true;
                 CSAW_TRY(enqueue_pack_build(g, P.kind, words, s));
                 pack = words;
             } else if (st != CSAW_ERR_NOMEM) {
@@ -2918,9 +2922,10 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
             CSAW_TRY(get_layer((void**)&P.hubS, sizeof(uint64_t) * (P.hubS_cap ? P.hubS_cap : 1)));
         }
         R->layer_edges[l] = total;
-        CSAW_TRY(alloc_edges(P, l, total, get, get_out));
-        R->src[l] = P.L[l].src;
+        const csaw_status edges = alloc_edges(P, l, total, get, get_out);
+        R->src[l] = P.L[l].src;   // the result's from here on, whatever fails
         R->dst[l] = P.L[l].dst;
+        CSAW_TRY(edges);
         if (layer_mode) {
             uint64_t *VP = nullptr, *p_eid = nullptr, *p_start = nullptr;
             uint32_t* p_bias = nullptr;
@@ -2958,6 +2963,27 @@ static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64
     R->src_c.assign(R->src.begin(), R->src.end());
     R->dst_c.assign(R->dst.begin(), R->dst.end());
     return CSAW_OK;
+}
+
+// An array that the caller did not ask for is given back where the buffers do
+// not fit beside it, and the run starts again without it.
+static csaw_status run_sample(csaw_graph* g, const uint32_t* seeds, const uint64_t* inst_off,
+                              uint32_t n_inst, uint64_t n_seeds, uint32_t depth, const uint32_t* fanout,
+                              int kind, uint64_t rng_seed, uint32_t attempt_cap, bool layer_mode,
+                              cudaStream_t s, csaw_sample_result* R, const SampleTables* tabs = nullptr)
+{
+    bool built = false;
+    const csaw_status st = run_layers(g, seeds, inst_off, n_inst, n_seeds, depth, fanout, kind, rng_seed, attempt_cap,
+                                      layer_mode, s, R, tabs, true, &built);
+    if (st != CSAW_ERR_NOMEM || !built) return st;
+    for (std::vector<uint32_t*>* arrs : {&R->src, &R->dst})
+        for (uint32_t*& p : *arrs) {
+            dfree(p, s);
+            p = nullptr;
+        }
+    clear_error();
+    return run_layers(g, seeds, inst_off, n_inst, n_seeds, depth, fanout, kind, rng_seed, attempt_cap, layer_mode, s,
+                      R, tabs, false, &built);
 }
 
 csaw_status sample_batch(csaw_graph* g, const uint32_t* d_seeds, const uint64_t* d_inst_off, uint32_t n_inst,

@@ -1,0 +1,92 @@
+"""Search arrays that a caller did not ask for never cost a call its success:
+where the caller's allocator has no room beside one, the call gives it back and
+goes on without it, with the same result."""
+import numpy as np
+import pytest
+
+from paper_2009_09103_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+SCALE = 14
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2009_09103_gb300 import build
+    build.build()
+    from paper_2009_09103_gb300 import csaw
+    g = inputs.rmat_csr(SCALE, 16, 255, 9)
+    G = csaw.Graph(g.off, g.col, g.w)
+    yield torch, csaw, g, G
+    G.use_own_allocator()
+    G.close()
+
+
+class Memory:
+    """PyTorch's allocator behind csaw_graph_set_allocator.  An array is a block of
+    exactly `array` bytes; while one is held, allocations from the `refuse`-th on
+    after it are refused."""
+
+    def __init__(self, env, array):
+        self.torch, self.csaw, _, self.G = env
+        self.array, self.refuse = array, None
+        self.live, self.arrays, self.refused, self.beside = {}, 0, 0, 0
+        self.cbs = (self.csaw.ALLOC_FN(self.alloc), self.csaw.FREE_FN(self.free))
+        st = self.csaw.lib().csaw_graph_set_allocator(self.G.handle, *self.cbs, None)
+        assert st == self.csaw.OK
+
+    def alloc(self, n, stream, ctx):
+        if self.array in self.live.values():
+            self.beside += 1
+            if self.refuse is not None and self.beside >= self.refuse:
+                self.refused += 1
+                return None
+        st = self.torch.cuda.ExternalStream(stream) if stream else None
+        p = self.torch.cuda.caching_allocator_alloc(int(n), stream=st)
+        self.live[p] = int(n)
+        if n == self.array:
+            self.arrays, self.beside = self.arrays + 1, 0
+        return p
+
+    def free(self, p, stream, ctx):
+        del self.live[p]
+        self.torch.cuda.caching_allocator_delete(p)
+
+    def check(self, call):
+        """call() alike at every place where memory may run out beside the array."""
+        ref = call()
+        assert self.arrays == 1, "the call is to build an array"
+        places = self.beside
+        assert places > 0
+        for k in range(1, places + 1):
+            self.refuse, self.arrays, self.beside, self.refused = k, 0, 0, 0
+            got = call()
+            assert self.refused > 0 and self.arrays == 1
+            assert len(got) == len(ref) and all(np.array_equal(a, b) for a, b in zip(got, ref)), k
+            assert not self.live, k
+        self.refuse = None
+
+
+def packed_bytes(g):
+    """The packed array: groups and their sums, windows of three 64-edge blocks, a
+    record per vertex and a word per chunk of 8192 edges."""
+    chunks = -(-g.E // 8192)
+    return 8 * (chunks * (8192 + 512 + 1) + 4 * (chunks * 128 // 3 + 1) + 2 * (g.V + 1))
+
+
+@pytest.mark.parametrize("layer", [False, True])
+@pytest.mark.parametrize("bias", ["edge_weight", "neighbor_degree"])
+def test_sampling(env, layer, bias):
+    torch, csaw, g, G = env
+    mem = Memory(env, packed_bytes(g))
+    seeds, io = inputs.distinct_seeds(np.full(300, 20, dtype=np.uint64), g.V, 4)
+    call = csaw.layer_sample if layer else csaw.sample
+
+    def run():
+        r = call(G, seeds, io, [12, 9], bias, 5)
+        return r.edge_offsets, r.frontier_sizes, r.src, r.dst
+    mem.check(run)
