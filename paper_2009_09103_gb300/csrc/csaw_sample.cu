@@ -3201,27 +3201,17 @@ static inline uint64_t sat_mul(uint64_t a, uint64_t b)
 
 }  // namespace csaw
 
-extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_instances, uint64_t max_seeds,
-                                                  uint32_t depth, const uint32_t* fanout, const csaw_bias* bias,
-                                                  const csaw_sample_opts* opts, csaw_sample_plan** out)
+// may_build: whether the plan may hold a packed array and build it in every
+// run, where that pays; *built: it does.
+static csaw_status plan_create(csaw_graph* g, uint32_t n_instances, uint64_t max_seeds, uint32_t depth,
+                               const uint32_t* fanout, int kind, uint32_t attempt_cap, bool may_build, bool* built,
+                               csaw_sample_plan** out)
 {
-    clear_error();
-    if (!out) return fail(CSAW_ERR_INVALID, "out is NULL");
-    *out = nullptr;
-    if (!g) return fail(CSAW_ERR_INVALID, "graph is NULL");
-    int kind;
-    CSAW_TRY(check_bias(g, bias, false, &kind));
-    if (depth < 1 || depth > CSAW_MAX_DEPTH) return fail(CSAW_ERR_INVALID, "depth must be 1..%u", CSAW_MAX_DEPTH);
-    if (!fanout) return fail(CSAW_ERR_INVALID, "fanout is NULL");
-    for (uint32_t l = 0; l < depth; ++l)
-        if (fanout[l] == 0) return fail(CSAW_ERR_INVALID, "fanout[%u] is 0", l);
-    if (n_instances == 0 || n_instances == 0xFFFFFFFFu) return fail(CSAW_ERR_INVALID, "bad instance count");
-    if (max_seeds == 0 || max_seeds >= 0xFFFFFFFFull) return fail(CSAW_ERR_INVALID, "bad seed budget");
     csaw_sample_plan* pl = new (std::nothrow) csaw_sample_plan();
     if (!pl) return fail(CSAW_ERR_NOMEM, "host allocation failed");
     Pipeline& P = pl->P;
     P.init(g, kind, n_instances, depth, fanout, 0, max_seeds);
-    P.attempt_cap = opts ? opts->attempt_cap : CSAW_ATTEMPT_CAP;
+    P.attempt_cap = attempt_cap;
     pl->max_seeds = max_seeds;
     pl->alloc = g->allocator;
     auto get = [&](void** p, size_t bytes) -> csaw_status {
@@ -3231,10 +3221,11 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
     };
     // the packed array of a large plan, built in every run
     uint64_t* pack = nullptr;
-    if (sample_array_pays(P, max_seeds)) {
+    if (may_build && sample_array_pays(P, max_seeds)) {
         if (get((void**)&pack, sizeof(uint64_t) * pack_layout(g->E, g->V).words) == CSAW_OK) P.use_pack(pack);
         else clear_error();   // no room: streamed
     }
+    *built = pack != nullptr;
     csaw_status st = alloc_common(P, get);
     // Upper bounds: a layer emits at most min(k, max degree) edges per
     // frontier vertex; a frontier is at most the previous layer's edges and
@@ -3309,6 +3300,33 @@ extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_inst
     if (st != CSAW_OK) { delete pl; return st; }
     *out = pl;
     return CSAW_OK;
+}
+
+extern "C" csaw_status csaw_sample_plan_create_ex(csaw_graph* g, uint32_t n_instances, uint64_t max_seeds,
+                                                  uint32_t depth, const uint32_t* fanout, const csaw_bias* bias,
+                                                  const csaw_sample_opts* opts, csaw_sample_plan** out)
+{
+    clear_error();
+    if (!out) return fail(CSAW_ERR_INVALID, "out is NULL");
+    *out = nullptr;
+    if (!g) return fail(CSAW_ERR_INVALID, "graph is NULL");
+    int kind;
+    CSAW_TRY(check_bias(g, bias, false, &kind));
+    if (depth < 1 || depth > CSAW_MAX_DEPTH) return fail(CSAW_ERR_INVALID, "depth must be 1..%u", CSAW_MAX_DEPTH);
+    if (!fanout) return fail(CSAW_ERR_INVALID, "fanout is NULL");
+    for (uint32_t l = 0; l < depth; ++l)
+        if (fanout[l] == 0) return fail(CSAW_ERR_INVALID, "fanout[%u] is 0", l);
+    if (n_instances == 0 || n_instances == 0xFFFFFFFFu) return fail(CSAW_ERR_INVALID, "bad instance count");
+    if (max_seeds == 0 || max_seeds >= 0xFFFFFFFFull) return fail(CSAW_ERR_INVALID, "bad seed budget");
+    const uint32_t attempt_cap = opts ? opts->attempt_cap : CSAW_ATTEMPT_CAP;
+    bool built = false;
+    csaw_status st = plan_create(g, n_instances, max_seeds, depth, fanout, kind, attempt_cap, true, &built, out);
+    if (st == CSAW_ERR_NOMEM && built) {
+        // its buffers do not fit beside the array: a plan without it
+        clear_error();
+        st = plan_create(g, n_instances, max_seeds, depth, fanout, kind, attempt_cap, false, &built, out);
+    }
+    return st;
 }
 
 extern "C" csaw_status csaw_sample_plan_create(csaw_graph* g, uint32_t n_instances, uint64_t max_seeds,

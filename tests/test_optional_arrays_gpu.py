@@ -90,3 +90,18 @@ def test_sampling(env, layer, bias):
         r = call(G, seeds, io, [12, 9], bias, 5)
         return r.edge_offsets, r.frontier_sizes, r.src, r.dst
     mem.check(run)
+
+
+@pytest.mark.parametrize("instances", [2, 300])
+def test_plans(env, instances):
+    torch, csaw, g, G = env
+    mem = Memory(env, packed_bytes(g))
+    seeds, io = inputs.distinct_seeds(np.full(instances, 6000 // instances, dtype=np.uint64), g.V, 4)
+
+    def run():
+        plan = csaw.SamplePlan(G, instances, len(seeds), [12, 9], "edge_weight")
+        plan.run(seeds, io, 5)
+        r = plan.result()
+        plan.close()
+        return r.edge_offsets, r.frontier_sizes, r.src, r.dst
+    mem.check(run)
