@@ -1011,8 +1011,11 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
     WalkArray arr;
     arr.tele = tele;
     arr.tele_q32 = tele != CSAW_TELEPORT_NONE ? opts->teleport_q32 : 0u;
-    void* tmp = nullptr;
+    void* tmp = nullptr;   // an array built for this call
+    void* a = nullptr;     // device starts and paths of a host call
+    void* b = nullptr;
     bool over_array = kind != CSAW_BIAS_NODE2VEC && (kept || build || pays);
+    const bool own = over_array && !kept && kind != CSAW_BIAS_UNIFORM;
     if (over_array && kept && kind != CSAW_BIAS_UNIFORM) {
         if (g->pack[kind]) {
             arr.mode = WC_PACK;
@@ -1023,52 +1026,58 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
         } else {
             over_array = false;
         }
-    } else if (over_array && kind != CSAW_BIAS_UNIFORM) {
-        if (pack_fits(g, kind)) {
-            csaw_status st = dalloc(&tmp, sizeof(uint64_t) * pack_layout(g->E, g->V).words, s);
-            if (st != CSAW_OK && st != CSAW_ERR_NOMEM) return st;
-            if (st == CSAW_OK) {
-                arr.mode = WC_PACK;
-                arr.k = pack_view((const uint64_t*)tmp, g->E, g->V);
-            }
-            clear_error();
-        }
-        if (!tmp && build) {
-            // edge weights keep only the summaries and records (the leaf level
-            // is formed from the weights); neighbour degree the whole array
-            const bool leaf = kind != CSAW_BIAS_EDGE_WEIGHT;
-            CSAW_TRY(dalloc(&tmp, sizeof(uint64_t) * (leaf ? cdf_words(g->E, g->V) : wsum_layout(g->E, g->V).words), s));
-            arr.mode = leaf ? WC_LEAF : WC_WEIGHTS;
-            arr.c = leaf ? cdf_view((const uint64_t*)tmp, g->E, g->V) : wsum_view((const uint64_t*)tmp, g->E, g->V);
-        }
-        if (!tmp) over_array = false;   // no room: the rows are streamed
     }
-    if (mem_kind == CSAW_MEM_HOST) {
-        // (over the array, the host starts are checked while the walk runs:
-        // the kernels stop a walker whose start is not a vertex)
-        for (uint64_t i = 0; !over_array && i < n_walkers; ++i)
+    // (over the array, the host starts are checked while the walk runs: the
+    // kernels stop a walker whose start is not a vertex)
+    const auto check_starts = [&]() -> csaw_status {
+        for (uint64_t i = 0; mem_kind == CSAW_MEM_HOST && !over_array && i < n_walkers; ++i)
             if (starts[i] >= g->V)
                 return fail(CSAW_ERR_INVALID, "start %llu of walker %llu out of range",
                             (unsigned long long)starts[i], (unsigned long long)i);
-        void* a = nullptr;
-        void* b = nullptr;
-        csaw_status st = dalloc(&a, sizeof(uint32_t) * n_walkers, s);
-        if (st == CSAW_OK) st = dalloc(&b, path_bytes, s);
-        if (st == CSAW_ERR_NOMEM && tmp && !build) {
-            // the buffers do not fit beside an array that was not asked for
-            dfree(tmp, s);
-            tmp = nullptr;
-            over_array = false;
-            for (uint64_t i = 0; i < n_walkers; ++i)
-                if (starts[i] >= g->V) {
-                    dfree(a, s);
-                    return fail(CSAW_ERR_INVALID, "start %llu of walker %llu out of range",
-                                (unsigned long long)starts[i], (unsigned long long)i);
-                }
-            st = a ? CSAW_OK : dalloc(&a, sizeof(uint32_t) * n_walkers, s);
+        return CSAW_OK;
+    };
+    // an array of so many words (0: none) and the host call's buffers, or neither
+    const auto memory = [&](uint64_t words) -> csaw_status {
+        csaw_status st = words ? dalloc(&tmp, sizeof(uint64_t) * words, s) : CSAW_OK;
+        if (st == CSAW_OK && mem_kind == CSAW_MEM_HOST) {
+            st = dalloc(&a, sizeof(uint32_t) * n_walkers, s);
             if (st == CSAW_OK) st = dalloc(&b, path_bytes, s);
         }
-        if (st != CSAW_OK) { dfree(a, s); dfree(tmp, s); return st; }
+        if (st != CSAW_OK) {
+            dfree(a, s);
+            dfree(tmp, s);
+            a = tmp = nullptr;
+        }
+        return st;
+    };
+    CSAW_TRY(check_starts());
+    // the largest array that fits beside the buffers: packed, then (build_cdf)
+    // the smaller one, then none, where the call did not ask for one
+    csaw_status got = CSAW_ERR_NOMEM;
+    if (own && pack_fits(g, kind)) {
+        got = memory(pack_layout(g->E, g->V).words);
+        if (got == CSAW_OK) {
+            arr.mode = WC_PACK;
+            arr.k = pack_view((const uint64_t*)tmp, g->E, g->V);
+        }
+    }
+    if (got == CSAW_ERR_NOMEM && build) {
+        // edge weights keep only the summaries and records (the leaf level
+        // is formed from the weights); neighbour degree the whole array
+        const bool leaf = kind != CSAW_BIAS_EDGE_WEIGHT;
+        got = memory(leaf ? cdf_words(g->E, g->V) : wsum_layout(g->E, g->V).words);
+        arr.mode = leaf ? WC_LEAF : WC_WEIGHTS;
+        arr.c = leaf ? cdf_view((const uint64_t*)tmp, g->E, g->V) : wsum_view((const uint64_t*)tmp, g->E, g->V);
+    } else if (got == CSAW_ERR_NOMEM) {
+        if (own) {
+            over_array = false;   // no room: the rows are streamed
+            CSAW_TRY(check_starts());
+        }
+        got = memory(0);
+    }
+    if (got != CSAW_OK) return got;
+    clear_error();
+    if (mem_kind == CSAW_MEM_HOST) {
         d_starts = (const uint32_t*)a;
         d_path = (uint32_t*)b;
         cudaError_t e = cudaMemcpyAsync(a, starts, sizeof(uint32_t) * n_walkers,

@@ -105,3 +105,20 @@ def test_plans(env, instances):
         plan.close()
         return r.edge_offsets, r.frontier_sizes, r.src, r.dst
     mem.check(run)
+
+
+@pytest.mark.parametrize("bias", ["edge_weight", "neighbor_degree"])
+@pytest.mark.parametrize("build", [False, True])
+def test_host_walks(env, bias, build):
+    torch, csaw, g, G = env
+    mem = Memory(env, packed_bytes(g))
+    starts = inputs.uniform_vertices(3000, g.V, 6)
+
+    def run():
+        phases = []
+        path = csaw.walk(G, starts, 40, bias, 8, build_cdf=build, phase_ms=phases)
+        # an array that was asked for is built all the same, by several launches
+        # (two events with nothing between are 3 us apart)
+        assert not build or phases[0] > 0.008
+        return (path,)
+    mem.check(run)
