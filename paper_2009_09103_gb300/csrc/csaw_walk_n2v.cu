@@ -662,15 +662,6 @@ csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bi
     if (st == CSAW_OK) st = dalloc(&index, index_bytes, s);
     if (st == CSAW_OK) st = dalloc(&rec, sizeof(uint64_t) * 4 * (uint64_t)g->V, s);
     if (st == CSAW_OK) st = dalloc(&big, sizeof(uint64_t) + sizeof(uint32_t) * n_big, s);
-    if (st == CSAW_ERR_NOMEM) {
-        // no room for the index: the caller streams the rows
-        dfree(sums, s);
-        dfree(index, s);
-        dfree(rec, s);
-        dfree(big, s);
-        clear_error();
-        return CSAW_OK;
-    }
     if (st == CSAW_OK && g->w) {
         p.c = kept ? cdf_view(kept, g->E, g->V) : wsum_view((const uint64_t*)sums, g->E, g->V);
         if (!kept)
@@ -711,6 +702,12 @@ csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bi
     dfree(rec, s);
     dfree(big, s);
     *done = st == CSAW_OK;
+    if (st == CSAW_ERR_NOMEM) {
+        // no room for the index, the sums or the sums' own temporaries: the
+        // caller streams the rows
+        clear_error();
+        return CSAW_OK;
+    }
     return st;
 }
 

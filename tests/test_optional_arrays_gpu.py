@@ -122,3 +122,10 @@ def test_host_walks(env, bias, build):
         assert not build or phases[0] > 0.008
         return (path,)
     mem.check(run)
+
+
+def test_node2vec_walks(env):
+    torch, csaw, g, G = env
+    mem = Memory(env, 8 * (g.E // 2 + g.V + 1))   # the row index: a word of 8 bytes per two edges and per vertex
+    starts = inputs.uniform_vertices(3000, g.V, 6)
+    mem.check(lambda: (csaw.walk(G, starts, 40, "node2vec", 8, (1, 2, 4)),))
