@@ -1223,6 +1223,12 @@ __global__ void layer_offsets_kernel(const uint64_t* __restrict__ foff, const ui
 // The positions of a layer's picks and the layer's offsets (scan_u32 and
 // layer_offsets_kernel) by one block, for small frontiers.
 constexpr uint64_t SMALL_SCAN = 4 * SCAN_TILE;
+// Up to this many instances one block also goes through all of them (most of
+// them empty, in a small frontier), which takes it 0.55 ns each, four times in
+// a plan of two layers; beyond, grids do (three launches more).  A plan of 100
+// seeds among 2,000 instances 0.097 ms by one block and 0.103 by grids, 4,000
+// 0.101 and 0.103, 16,000 0.129 and 0.102, two million 4.45 and 0.16.
+constexpr uint32_t SMALL_INSTANCES = 4096;
 
 __global__ void __launch_bounds__(SCAN_THREADS) small_offsets_kernel(
     const uint32_t* __restrict__ cnt, const uint64_t* n_dev, uint64_t* pos, uint64_t* __restrict__ total_out,
@@ -1270,7 +1276,7 @@ struct SmallFrontier {
     uint32_t n_inst = 0, vbits = 0;
     int kbits = 0;
     uint64_t* F = nullptr;
-    uint64_t* FO = nullptr;
+    uint64_t* FO = nullptr;               // null: the offsets' check and the bounds are left to grids
     uint64_t* n_out = nullptr;
 };
 
@@ -1291,7 +1297,7 @@ __global__ void __launch_bounds__(SF_THREADS) small_frontier_kernel(SmallFrontie
             if (total > p.cap) atomicOr(p.err, 4u);
             *p.n_seeds = total < p.cap ? total : p.cap;
         }
-        for (uint64_t i = tid; i < p.n_inst; i += SF_THREADS)
+        for (uint64_t i = tid; p.FO && i < p.n_inst; i += SF_THREADS)
             if (p.inst_off[i + 1] < p.inst_off[i]) atomicOr(p.err, 2u);
         n = (uint32_t)(total < p.cap ? total : p.cap);
         for (uint32_t j = tid; j < n; j += SF_THREADS) {
@@ -1375,7 +1381,7 @@ __global__ void __launch_bounds__(SF_THREADS) small_frontier_kernel(SmallFrontie
         }
     if (tid == 0) *p.n_out = kept;
     __syncthreads();
-    for (uint64_t i = tid; i <= p.n_inst; i += SF_THREADS) {
+    for (uint64_t i = tid; p.FO && i <= p.n_inst; i += SF_THREADS) {
         uint32_t lo = 0, hi = kept;
         const uint64_t key = i << p.vbits;
         while (lo < hi) {
@@ -2318,7 +2324,11 @@ static void launch_frontier(const uint64_t* sorted, const uint64_t* n_dev, uint6
 static csaw_status launch_small_frontier(const Pipeline& P, SmallFrontier& sf, uint32_t l, cudaStream_t s)
 {
     sf.n_inst = P.n_inst; sf.vbits = (uint32_t)P.vbits; sf.kbits = P.kbits;
-    sf.F = P.L[l].F; sf.FO = P.L[l].FO; sf.n_out = P.lc(l, L_N);
+    const bool bounds = P.n_inst <= SMALL_INSTANCES;
+    const int sms = P.g->sm_count;
+    sf.F = P.L[l].F; sf.FO = bounds ? P.L[l].FO : nullptr; sf.n_out = P.lc(l, L_N);
+    if (!bounds && sf.inst_off)
+        check_inst_off_kernel<<<grid_for(P.n_inst, 256, sms), 256, 0, s>>>(sf.inst_off, P.n_inst, sf.err);
     // the attribute is set before the flag is published: calls may come from several threads
     static std::atomic<bool> ready{false};
     if (!ready.load(std::memory_order_acquire)) {
@@ -2326,6 +2336,9 @@ static csaw_status launch_small_frontier(const Pipeline& P, SmallFrontier& sf, u
         ready.store(true, std::memory_order_release);
     }
     small_frontier_kernel<<<1, SF_THREADS, SF_SMEM, s>>>(sf);
+    if (!bounds)
+        inst_bounds_kernel<<<grid_for((uint64_t)P.n_inst + 1, 256, sms), 256, 0, s>>>(P.L[l].F, P.lc(l, L_N), P.n_inst,
+                                                                                      P.vbits, P.L[l].FO);
     CSAW_CUDA(cudaGetLastError());
     return CSAW_OK;
 }
@@ -2431,7 +2444,7 @@ static csaw_status enqueue_classify(Pipeline& P, uint32_t l, uint32_t v_lo, uint
 static csaw_status enqueue_positions(Pipeline& P, uint32_t l, cudaStream_t s)
 {
     LayerBufs& B = P.L[l];
-    if (B.f_cap > SMALL_SCAN)
+    if (B.f_cap > SMALL_SCAN || P.n_inst > SMALL_INSTANCES)
         return scan_u32(B.cnt, B.pos, P.lc(l, L_N), B.f_cap, P.scan_scr, P.lc(l, L_TOTAL), s);
     small_offsets_kernel<<<1, SCAN_THREADS, 0, s>>>(B.cnt, P.lc(l, L_N), B.pos, P.lc(l, L_TOTAL), B.FO, P.n_inst,
                                                     P.ctr + CT_BASE + l, P.eoff + (uint64_t)l * P.n_inst,
