@@ -1,5 +1,7 @@
 """Few seeds among very many instances, most of them empty: what goes through
 the instances is spread over the chip, and the results stay the oracle's."""
+import time
+
 import numpy as np
 import pytest
 
@@ -67,3 +69,30 @@ def test_time(env):
     plan.close()
     G.close()
     assert min(times) < 1.0, times
+
+
+def test_reading_the_offsets(env):
+    """The offsets and sizes of two million instances are read about as fast as their bytes
+    are copied into the same kind of host memory."""
+    torch, csaw = env
+    g = inputs.rmat_csr(12, 8, 20, 2)
+    G = csaw.Graph(g.off, g.col, g.w)
+    n = 2000000
+    seeds, io = inputs.uniform_vertices(100, g.V, 3), np.full(n + 1, 100, dtype=np.uint64)
+    io[0] = 0
+    plan = csaw.SamplePlan(G, n, 100, [5, 5], "edge_weight")
+    words = torch.zeros(4 * n, dtype=torch.int64, device="cuda")
+    host = torch.zeros(4 * n, dtype=torch.int64)
+    read, copy = [], []
+    for _ in range(6):
+        plan.run(seeds, io, 1)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        plan.n_edges()
+        t1 = time.perf_counter()
+        host.copy_(words)
+        read.append(t1 - t0)
+        copy.append(time.perf_counter() - t1)
+    plan.close()
+    G.close()
+    assert min(read) < 1.6 * min(copy), (read, copy)
