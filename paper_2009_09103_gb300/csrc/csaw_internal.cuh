@@ -218,6 +218,12 @@ inline double slowest_walk(const csaw_graph* g, double n, double length, bool by
     return length * visited + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * visited);
 }
 
+// Device bytes of the array that a plain walk call of n walkers, or a sampling
+// run, builds by itself because it pays (0: none), beside its other buffers.
+uint64_t walk_array_bytes(const csaw_graph* g, const csaw_bias* bias, uint64_t n, uint32_t length);
+uint64_t sample_array_bytes(csaw_graph* g, int kind, uint32_t n_inst, uint64_t n_seeds, uint32_t depth,
+                            const uint32_t* fanout);
+
 // Device bytes of node2vec's row index and sums, built for one call.
 uint64_t n2v_bytes(const csaw_graph* g);
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length);

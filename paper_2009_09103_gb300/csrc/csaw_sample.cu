@@ -2316,6 +2316,14 @@ static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
     return P.n_inst > 1 ? 150e6 + 150.0 * entries >= cost : 2.0 * reached * visited >= cost + 40e6;
 }
 
+uint64_t sample_array_bytes(csaw_graph* g, int kind, uint32_t n_inst, uint64_t n_seeds, uint32_t depth,
+                            const uint32_t* fanout)
+{
+    Pipeline P;
+    P.init(g, kind, n_inst, depth, fanout, 0, n_seeds);
+    return sample_array_pays(P, n_seeds) ? sizeof(uint64_t) * pack_layout(g->E, g->V).words : 0;
+}
+
 // The frontier from n_max sorted keys at most: flags and block sums, then the
 // kept keys in order.
 static void launch_frontier(const uint64_t* sorted, const uint64_t* n_dev, uint64_t n_max, const Visited& vis,

@@ -591,18 +591,31 @@ struct csaw_server {
         }
     }
 
-    // Device bytes set aside, beside the estimates, for an array that the batch
-    // may build: an array of this graph, where the budget has that much left
-    // and a slot's arrays stay below half its share.  Otherwise rows are
-    // streamed, within the estimate (RMAT s26: an array is 18 GB).  Called with
-    // mu held, the batch's estimates in in_use.
+    // Device bytes set aside, beside the estimates, for the array that the batch
+    // builds by the rules of csaw_walk and csaw_sample, where the budget has that
+    // much left and a slot's arrays stay below half its share.  Otherwise rows
+    // are streamed, within the estimate (RMAT s26: an array is 18 GB).  Called
+    // with mu held, the batch's estimates in in_use.
     uint64_t reserve_array(const std::vector<Request*>& batch) const
     {
         const Request* head = batch[0];
-        const int kind = head->bias.kind;
-        if (kind == CSAW_BIAS_UNIFORM || (head->kind == CSAW_REQ_WALK && batch.size() > 1)) return 0;
-        const uint64_t bytes = kind == CSAW_BIAS_NODE2VEC ? n2v_bytes(g)
-                                                          : sizeof(uint64_t) * pack_layout(g->E, g->V).words;
+        uint64_t bytes = 0;
+        if (head->kind == CSAW_REQ_WALK) {
+            // (several walks in one launch stream, or search a kept array)
+            if (batch.size() == 1) bytes = walk_array_bytes(g, &head->bias, head->starts.size(), head->length);
+        } else {
+            uint64_t n_inst = 0, n_seeds = 0;
+            uint32_t fan_max[CSAW_MAX_DEPTH] = {}, depth = 0;
+            for (const Request* rq : batch) {
+                n_inst += rq->n_instances;
+                n_seeds += rq->seeds.size();
+                depth = std::max(depth, (uint32_t)rq->fanout.size());
+                for (size_t l = 0; l < rq->fanout.size(); ++l) fan_max[l] = std::max(fan_max[l], rq->fanout[l]);
+            }
+            int kind;
+            if (check_bias(g, &head->bias, false, &kind) == CSAW_OK && n_inst < 0xFFFFFFFFull)
+                bytes = sample_array_bytes(g, kind, (uint32_t)n_inst, n_seeds, depth, fan_max);
+        }
         return bytes <= budget / (2 * (uint64_t)slots) && bytes <= budget - in_use ? bytes : 0;
     }
 

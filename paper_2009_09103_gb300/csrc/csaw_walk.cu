@@ -942,6 +942,15 @@ static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t 
     return full >= cost || slowest >= cost + 0.5e6 * (double)length;
 }
 
+uint64_t walk_array_bytes(const csaw_graph* g, const csaw_bias* bias, uint64_t n, uint32_t length)
+{
+    int kind;
+    if (check_bias(g, bias, true, &kind) != CSAW_OK) return 0;
+    if (kind == CSAW_BIAS_NODE2VEC) return n2v_index_pays(g, n, length) ? n2v_bytes(g) : 0;
+    const bool builds = !cached_cdf_usable(g, kind) && pack_fits(g, kind) && walk_array_pays(g, kind, n, length);
+    return builds ? sizeof(uint64_t) * pack_layout(g->E, g->V).words : 0;
+}
+
 // CUDA events around a call's phases, when the caller asks for their times:
 // [0] before the array's construction, [1] before the walk, [2] after it.
 struct PhaseTimer {
