@@ -398,7 +398,10 @@ csaw_status csaw_mdrw(csaw_graph* g, const uint32_t* pools, uint64_t n_instances
  * `stream` and waits on it once per layer (to size the next layer's buffers),
  * so it returns with the result complete.  The result lives on the device;
  * read it with csaw_sample_get_view or copy it with csaw_sample_copy_edges,
- * release it with csaw_result_free.
+ * release it with csaw_result_free.  A call large enough for it (csaw_sample
+ * and csaw_layer_sample) builds the packed array of the whole graph into a
+ * temporary, as csaw_walk does; where that does not fit beside its buffers, the
+ * rows are streamed.
  * Errors: CSAW_ERR_INVALID, CSAW_ERR_NOMEM, CSAW_ERR_CUDA. */
 csaw_status csaw_sample(csaw_graph* g, const uint32_t* seeds, const uint64_t* inst_offsets,
                         uint32_t n_instances, uint32_t depth, const uint32_t* fanout,
@@ -481,7 +484,9 @@ void csaw_result_free(void* result);
  * once at its upper bound and the pipeline captured into one CUDA graph.
  * Each run copies a new batch of seeds in and launches the graph: no host
  * waits, no allocation.  Results are identical to csaw_sample on the same
- * arguments.
+ * arguments.  Like csaw_sample, a large plan builds the packed array of its
+ * bias in every run (8.67 bytes per edge + 16 per vertex of its buffers); where
+ * that does not fit in memory, rows are streamed.
  * Upper bounds: layer l emits at most |F_l| * min(fanout[l], max degree)
  * edges; |F_0| <= max_seeds and |F_{l+1}| <= min(edges of layer l,
  * n_instances * n_vertices).  A plan whose non-last layer may produce 2^32 or
@@ -514,8 +519,8 @@ csaw_status csaw_sample_plan_get_view(csaw_sample_plan* p, csaw_sample_view* vie
  * host arrays of n_edges entries. */
 csaw_status csaw_sample_plan_copy_edges(csaw_sample_plan* p, uint32_t* src, uint32_t* dst);
 
-/* Capacity-based device bytes of the plan's buffers and its selection launch
- * shape (any pointer may be NULL). */
+/* Device bytes of the plan's buffers, a packed array of its own among them,
+ * and its selection launch shape (any pointer may be NULL). */
 csaw_status csaw_sample_plan_get_info(const csaw_sample_plan* p, uint64_t* device_bytes,
                                       uint32_t* theta_warp, uint32_t* select_blocks);
 

@@ -3215,6 +3215,7 @@ struct csaw_sample_plan {
     uint32_t magic = 0x43504c4eu;   // "CPLN"
     csaw::Pipeline P;
     std::vector<void*> allocs;
+    uint64_t device_bytes = 0;   // of allocs
     DevAllocator alloc;       // the allocator of the buffers (the graph's at creation)
     uint32_t* in_seeds = nullptr;
     uint64_t* in_io = nullptr;
@@ -3263,6 +3264,7 @@ static csaw_status plan_create(csaw_graph* g, uint32_t n_instances, uint64_t max
     auto get = [&](void** p, size_t bytes) -> csaw_status {
         CSAW_TRY(alloc_with(&pl->alloc, p, bytes ? bytes : 16, nullptr));
         pl->allocs.push_back(*p);
+        pl->device_bytes += bytes;
         return CSAW_OK;
     };
     // the packed array of a large plan, built in every run
@@ -3486,15 +3488,7 @@ extern "C" csaw_status csaw_sample_plan_get_info(const csaw_sample_plan* pl, uin
 {
     clear_error();
     if (!pl) return fail(CSAW_ERR_INVALID, "plan is NULL");
-    if (device_bytes) {
-        uint64_t b = 0;
-        // sizes are not recorded per allocation; report capacities
-        const Pipeline& P = pl->P;
-        for (uint32_t l = 0; l < P.depth; ++l)
-            b += P.L[l].f_cap * 28 + P.L[l].e_cap * (8 + (l + 1 < P.depth ? 20 : 0));
-        b += P.seeds_cap * 20 + pl->max_seeds * 4;
-        *device_bytes = b;
-    }
+    if (device_bytes) *device_bytes = pl->device_bytes;
     if (theta_warp) *theta_warp = pl->P.theta_w;
     if (select_blocks) *select_blocks = (uint32_t)pl->P.sel_blocks;
     return CSAW_OK;

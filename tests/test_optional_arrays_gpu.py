@@ -129,3 +129,14 @@ def test_node2vec_walks(env):
     mem = Memory(env, 8 * (g.E // 2 + g.V + 1))   # the row index: a word of 8 bytes per two edges and per vertex
     starts = inputs.uniform_vertices(3000, g.V, 6)
     mem.check(lambda: (csaw.walk(G, starts, 40, "node2vec", 8, (1, 2, 4)),))
+
+
+@pytest.mark.parametrize("bias", ["uniform", "edge_weight"])
+def test_plan_info_counts_every_buffer(env, bias):
+    torch, csaw, g, G = env
+    mem = Memory(env, packed_bytes(g))
+    plan = csaw.SamplePlan(G, 300, 6000, [12, 9], bias)
+    assert mem.arrays == (bias == "edge_weight")
+    assert sum(mem.live.values()) == plan.info()["device_bytes"]
+    plan.close()
+    assert not mem.live
