@@ -942,12 +942,19 @@ static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t 
     return full >= cost || slowest >= cost + 0.5e6 * (double)length;
 }
 
+// Whether the graph keeps an array that walks of the kind can search.  The
+// packed one takes zero biases as they are.
+static bool walk_array_kept(const csaw_graph* g, int kind)
+{
+    return cached_cdf_usable(g, kind) || g->pack[kind];
+}
+
 uint64_t walk_array_bytes(const csaw_graph* g, const csaw_bias* bias, uint64_t n, uint32_t length)
 {
     int kind;
     if (check_bias(g, bias, true, &kind) != CSAW_OK) return 0;
     if (kind == CSAW_BIAS_NODE2VEC) return n2v_index_pays(g, n, length) ? n2v_bytes(g) : 0;
-    const bool builds = !cached_cdf_usable(g, kind) && pack_fits(g, kind) && walk_array_pays(g, kind, n, length);
+    const bool builds = !walk_array_kept(g, kind) && pack_fits(g, kind) && walk_array_pays(g, kind, n, length);
     return builds ? sizeof(uint64_t) * pack_layout(g->E, g->V).words : 0;
 }
 
@@ -1013,7 +1020,7 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
     // a static bias: over the graph's kept array, or one built for this call
     // into a stream-ordered temporary (build_cdf, or because the call is large
     // enough that it pays); otherwise the rows are streamed
-    const bool kept = cached_cdf_usable(g, kind);
+    const bool kept = walk_array_kept(g, kind);
     const bool build = !kept && tele == CSAW_TELEPORT_NONE && opts && opts->build_cdf && cdf_kind_positive(g, kind);
     const bool pays = !kept && !build && kind != CSAW_BIAS_NODE2VEC && pack_fits(g, kind) &&
                       walk_array_pays(g, kind, n_walkers, length);

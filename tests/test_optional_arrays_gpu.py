@@ -4,6 +4,7 @@ goes on without it, with the same result."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2009_09103_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -140,3 +141,26 @@ def test_plan_info_counts_every_buffer(env, bias):
     assert sum(mem.live.values()) == plan.info()["device_bytes"]
     plan.close()
     assert not mem.live
+
+
+@pytest.mark.parametrize("bias", ["edge_weight", "neighbor_degree"])
+@pytest.mark.parametrize("tele", [{}, {"teleport": "restart", "teleport_q32": 1 << 29}])
+def test_kept_array_with_zero_biases(env, bias, tele):
+    """A kept packed array is searched, not built again, whatever the biases: here zero
+    weights, and edges into vertices that have none."""
+    torch, csaw, g, _ = env
+    off = np.minimum(g.off, g.off[g.V // 2])   # the upper half has no edges of its own
+    z = inputs.CSRGraph(off, g.col[:off[-1]], g.w[:off[-1]] & np.uint32(3))
+    starts = inputs.uniform_vertices(3000, g.V, 6)
+    Z = csaw.Graph(z.off, z.col, z.w)
+    mem = Memory((torch, csaw, z, Z), packed_bytes(z))
+    Z.build_cdf(bias)
+    assert mem.arrays == 1
+    got = csaw.walk(Z, starts, 40, bias, 8, **tele)
+    assert mem.arrays == 1
+    Z.drop_cdf(bias)
+    assert np.array_equal(got, csaw.walk(Z, starts, 40, bias, 8, **tele))
+    assert mem.arrays == 2
+    Z.use_own_allocator()
+    Z.close()
+    assert np.array_equal(got, oracle.walk(z, starts, 40, bias, 8, **tele))
