@@ -14,8 +14,8 @@
 // Rows that fit one round stay in registers and need one pass.
 //
 // Work distribution: a persistent grid; each warp takes the next walker from
-// a global counter and runs all its steps.  (Walks over a cached cumulative
-// array are in csaw_walk_cdf.cu.)  The path row is buffered one
+// a global counter and runs all its steps.  (Uniform walks, and walks over an
+// array of the biases, are in csaw_walk_cdf.cu.)  The path row is buffered one
 // 32-entry block per warp (lane j holds entry 32*blk + j) and written with
 // one coalesced store per block.
 #include <atomic>
@@ -575,10 +575,6 @@ __device__ __forceinline__ bool walk_pick(const WalkParams& p, const Row& row, c
             n2v_fast_pays(row.d, (uint32_t)(c.pend - c.pbeg)))
             return n2v_fast_pick(p, row, c, r, lane, s_jpos, s_jw, idx);
     }
-    if constexpr (KIND == CSAW_BIAS_UNIFORM) {
-        *idx = (uint32_t)scale_draw(r, row.d);   // b = 1: S[i] = i + 1, the pick is x itself
-        return true;
-    }
     if constexpr (KIND != CSAW_BIAS_NODE2VEC) {
         if (row.span <= TILE) {
             // One tile: lane l holds positions 4l .. 4l+3; its inclusive
@@ -698,8 +694,7 @@ __device__ __forceinline__ bool walk_pick(const WalkParams& p, const Row& row, c
 template <int KIND, bool WIDE, bool TELE, bool BATCH>
 constexpr int walk_min_blocks()
 {
-    return KIND == CSAW_BIAS_UNIFORM ? 5
-           : (KIND == CSAW_BIAS_EDGE_WEIGHT && !WIDE) ? CSAW_WALK_EW_BLOCKS
+    return (KIND == CSAW_BIAS_EDGE_WEIGHT && !WIDE) ? CSAW_WALK_EW_BLOCKS
            : KIND == CSAW_BIAS_NODE2VEC ? (TELE || BATCH ? 3 : CSAW_WALK_N2V_BLOCKS) : 4;
 }
 
@@ -849,7 +844,6 @@ static csaw_status launch_walk(int kind, uint64_t max_bias, const WalkParams& p,
 {
     const bool wide = max_bias * ROUND >= (1ull << 32);
     switch (kind) {
-    case CSAW_BIAS_UNIFORM: return launch_walk_kw<CSAW_BIAS_UNIFORM, false>(p, sm_count, s);
     case CSAW_BIAS_EDGE_WEIGHT:
         return wide ? launch_walk_kw<CSAW_BIAS_EDGE_WEIGHT, true>(p, sm_count, s)
                     : launch_walk_kw<CSAW_BIAS_EDGE_WEIGHT, false>(p, sm_count, s);
@@ -870,7 +864,6 @@ static csaw_status launch_walk_batch(int kind, uint64_t max_bias, const WalkPara
 {
     const bool wide = max_bias * ROUND >= (1ull << 32);
     switch (kind) {
-    case CSAW_BIAS_UNIFORM: return launch_walk_kwt<CSAW_BIAS_UNIFORM, false, false, true>(p, sm_count, s);
     case CSAW_BIAS_EDGE_WEIGHT:
         return wide ? launch_walk_kwt<CSAW_BIAS_EDGE_WEIGHT, true, false, true>(p, sm_count, s)
                     : launch_walk_kwt<CSAW_BIAS_EDGE_WEIGHT, false, false, true>(p, sm_count, s);
