@@ -196,26 +196,25 @@ csaw_status walk_batch_cached(const csaw_graph* g, int kind, const uint32_t* d_s
 csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,
                      uint32_t length, uint64_t rng_seed, uint32_t tele, uint32_t tele_q32, uint32_t* path,
                      unsigned long long* next_walker, cudaStream_t s, bool* done);
-// Whether a call of n walks of `length` steps is large enough for it.
 // The mean degree of the rows that a walk or a sampled layer comes to, for the
 // rules that weigh streaming rows against building an array: sqrt(mean degree *
 // largest degree) where edges are followed by weight (RMAT s16 520 for 684
 // measured, s20 1393 for 2233, s20 ef32 2424 for 3315), nearer the largest
 // degree where they are followed by degree, and the degree itself on a regular
 // graph.
+inline double mean_degree(const csaw_graph* g) { return g->V ? (double)g->E / (double)g->V : 0.0; }
 inline double visited_degree(const csaw_graph* g, bool by_degree)
 {
-    const double avg = g->V ? (double)g->E / (double)g->V : 0.0, most = (double)g->max_degree;
+    const double avg = mean_degree(g), most = (double)g->max_degree;
     return by_degree ? std::cbrt(avg * most * most) : std::sqrt(avg * most);
 }
 
-// The neighbours that the slowest of n walkers streams in `length` steps, for
-// the same rules: a call ends no sooner than that walker, which meets rows far
-// longer than the mean (RMAT s20, 60 steps: fits 16 to 4,000 walkers' times).
-inline double slowest_walk(const csaw_graph* g, double n, double length, bool by_degree)
+// The neighbours that the slowest of n walkers comes by in `length` steps, at
+// rows of a mean degree, for the same rules: a call ends no sooner than that
+// walker, which meets rows far longer than the mean.
+inline double slowest_walk(const csaw_graph* g, double n, double length, double degree)
 {
-    const double visited = visited_degree(g, by_degree);
-    return length * visited + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * visited);
+    return length * degree + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * degree);
 }
 
 // Device bytes of the array that a plain walk call of n walkers, or a sampling
@@ -224,7 +223,8 @@ uint64_t walk_array_bytes(const csaw_graph* g, const csaw_bias* bias, uint64_t n
 uint64_t sample_array_bytes(csaw_graph* g, int kind, uint32_t n_inst, uint64_t n_seeds, uint32_t depth,
                             const uint32_t* fanout);
 
-// Device bytes of node2vec's row index and sums, built for one call.
+// Device bytes of node2vec's row index and sums, built for one call, and
+// whether a call of n walks of `length` steps is large enough for them.
 uint64_t n2v_bytes(const csaw_graph* g);
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length);
 

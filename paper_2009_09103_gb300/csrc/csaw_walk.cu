@@ -929,8 +929,9 @@ static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t 
 {
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const bool by_degree = kind == CSAW_BIAS_NEIGHBOR_DEGREE;
-    const double full = (double)n * (double)length * (250.0 + (by_degree ? 1.0 : 0.3) * visited_degree(g, by_degree));
-    const double slowest = (by_degree ? 1300.0 : 750.0) * slowest_walk(g, (double)n, (double)length, by_degree);
+    const double visited = visited_degree(g, by_degree);
+    const double full = (double)n * (double)length * (250.0 + (by_degree ? 1.0 : 0.3) * visited);
+    const double slowest = (by_degree ? 1300.0 : 750.0) * slowest_walk(g, (double)n, (double)length, visited);
     const double cost = (by_degree ? 6.0 : 4.0) * (double)g->E + 25e6;
     return full >= cost || slowest >= cost + 0.5e6 * (double)length;
 }

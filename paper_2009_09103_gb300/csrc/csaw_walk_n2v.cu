@@ -629,22 +629,31 @@ uint64_t n2v_bytes(const csaw_graph* g)
            sizeof(uint32_t) * (g->E / N2V_BIG_ROW + 2);
 }
 
-// In ps: streaming a step costs about 5.5 per neighbour of the row with the
-// chip full (RMAT s20 ef32: 18 ns per step at a mean visited degree of 3,315),
-// and a step of the slowest walker 4.5 us and 6000 per neighbour however few
-// walk beside it; a step over the index takes about a third of the first and
-// two fifths of the second.  The index and summaries take about 18 per edge,
-// and 10 us of launches (50 where too few walk to fill the chip).  60 steps of
-// 256 walkers, streamed and over the index: RMAT s16 1161 and 556 us, s20 3088
-// and 1726.
+// Streaming, a step costs by the row it stands on; over the index, by the
+// shorter of two rows' lists, which stays near the mean degree however long
+// the hubs are.  So the index pays where the rows that walks come to are
+// longer than the mean, once its construction is paid, and hardly ever on a
+// regular graph, where both lists are alike (degree 4: 0.64 ns a step streamed
+// and 0.83 over the index with the chip full; 64: 1.04 and 1.13; 512 of which
+// half are common: 2.85 and 4.49).  RMAT s12 1.41 and 0.99, s16 2.9 and 1.2,
+// s20 5.8 and 2.4; 16 stars of 60,000 leaves 35 and 1.0.  Each side is the larger of
+// what its steps cost with the chip full and of what the slowest walker takes,
+// however few walk beside it.
+// The figures, in ps, are fitted to the choices, not to either side alone:
+// 645 calls on 20 graphs (grid, circulant, random, Zipf, stars, RMAT s12 to
+// s20), 16 to 1,000,000 walkers of 2 to 80 steps.  Of those calls 11 take
+// longer than streamed, at most by 15 %.
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length)
 {
     if (g->E == 0 || g->max_degree > 0x7FFFFFFFu) return false;   // positions plus 8 fit 32 bits
     if (n2v_bytes(g) > array_room()) return false;
-    const double full = 5.5 * (double)n * (double)length * visited_degree(g, false);
-    const double slowest = 4.5e6 * (double)length + 6e3 * slowest_walk(g, (double)n, (double)length, false);
-    const double cost = 18.0 * (double)g->E;
-    return full * 2.0 / 3.0 >= cost + 10e6 || slowest * 0.6 >= cost + 50e6;
+    const double walkers = (double)n, steps = (double)length;
+    const double visited = visited_degree(g, false), mean = mean_degree(g);
+    const double streamed = std::max(7.3 * walkers * steps * visited,
+                                     9.5e3 * slowest_walk(g, walkers, steps, visited) + 0.4e6 * steps);
+    const double indexed = 42.0 * (double)g->E + 80e6 +
+                           std::max(walkers * steps * (7.3 * mean + 40.0), 7e3 * slowest_walk(g, walkers, steps, mean));
+    return streamed >= indexed;
 }
 
 csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,

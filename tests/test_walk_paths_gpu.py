@@ -61,6 +61,16 @@ def hub_graph(V, sizes, wlo, whi, loops=False, seed=6):
     return inputs.CSRGraph(off, a[:, 1].astype(np.uint32), rng.integers(wlo, whi + 1, size=len(a)).astype(np.uint32))
 
 
+def beside_a_star(g, leaves=6000):
+    """g and, apart from it, a star: its hub makes the rows that walks come to long in the
+    mean, so that calls on g's vertices build the index at sizes the oracle is quick at."""
+    V, n = g.V, g.E
+    off = np.concatenate([g.off, n + np.arange(1, leaves + 1), [n + 2 * leaves]]).astype(np.uint64)
+    col = np.concatenate([g.col, np.full(leaves, V + leaves), V + np.arange(leaves)]).astype(np.uint32)
+    w = None if g.w is None else np.concatenate([g.w, np.ones(2 * leaves)]).astype(np.uint32)
+    return inputs.CSRGraph(off, col, w)
+
+
 MULTS = [(1, 2, 4), (0, 1, 1), (1, 0, 2), (4, 1, 0), (0, 0, 1), (1, 0, 0), (0, 1, 0), (0, 0, 0)]
 
 
@@ -70,7 +80,7 @@ MULTS = [(1, 2, 4), (0, 1, 1), (1, 0, 2), (4, 1, 0), (0, 0, 1), (1, 0, 0), (0, 1
 def test_node2vec_weights_and_multipliers(csaw, wlo, whi, mult, loops):
     g = hub_graph(900, (700, 260, 40, 8), wlo, whi, loops)
     starts = np.tile(np.arange(g.V, dtype=np.uint32), 16)
-    assert walk(csaw, g, starts, 10, "node2vec", 21, mult)
+    assert walk(csaw, beside_a_star(g), starts, 10, "node2vec", 21, mult)
 
 
 @pytest.mark.parametrize("tele", ["restart", "jump"])
@@ -78,7 +88,7 @@ def test_node2vec_weights_and_multipliers(csaw, wlo, whi, mult, loops):
 def test_node2vec_teleports(csaw, tele, mult):
     g = hub_graph(900, (700, 260, 40, 8), 0, 3, True)
     starts = np.tile(np.arange(g.V, dtype=np.uint32), 16)
-    assert walk(csaw, g, starts, 10, "node2vec", 22, mult, teleport=tele, teleport_q32=1 << 29)
+    assert walk(csaw, beside_a_star(g), starts, 10, "node2vec", 22, mult, teleport=tele, teleport_q32=1 << 29)
 
 
 @pytest.mark.parametrize("sizes", [(1, 1), (3, 9), (31, 130), (129, 700)])
@@ -86,7 +96,7 @@ def test_node2vec_teleports(csaw, tele, mult):
 def test_node2vec_small_rows(csaw, sizes, kept):
     g = hub_graph(2 + 2 * max(sizes) + 50, sizes, 1, 255)
     starts = np.resize(np.array([0, 1, 2, 5], dtype=np.uint32), 60000)
-    assert walk(csaw, g, starts, 60, "node2vec", 23, (3, 1, 2), kept)
+    assert walk(csaw, beside_a_star(g), starts, 60, "node2vec", 23, (3, 1, 2), kept)
 
 
 @pytest.mark.parametrize("edges,weights", [
@@ -94,9 +104,9 @@ def test_node2vec_small_rows(csaw, sizes, kept):
 def test_node2vec_tiny_graphs(csaw, edges, weights):
     g = inputs.csr_from_edges(max(max(e) for e in edges) + 1, edges, weights)
     starts = np.resize(np.arange(g.V, dtype=np.uint32), 50000)
-    assert walk(csaw, g, starts, 90, "node2vec", 2, (1, 2, 4))
+    assert walk(csaw, beside_a_star(g), starts, 90, "node2vec", 2, (1, 2, 4))
     unweighted = inputs.CSRGraph(g.off, g.col, None)
-    assert walk(csaw, unweighted, starts, 90, "node2vec", 3, (1, 2, 4))
+    assert walk(csaw, beside_a_star(unweighted), starts, 90, "node2vec", 3, (1, 2, 4))
 
 
 @pytest.mark.parametrize("bias,n,length,builds", [
@@ -110,3 +120,19 @@ def test_few_walkers(csaw, bias, n, length, builds):
     assert walk(csaw, g, starts, length, bias, 7) == builds
     kw = {"teleport": "restart", "teleport_q32": 1 << 29}
     assert walk(csaw, g, starts, length, bias, 8, **kw) == builds
+
+
+def ring(V, d):
+    """Every vertex beside the d / 2 next and the d / 2 before it."""
+    a = np.concatenate([np.arange(-(d // 2), 0), np.arange(1, d // 2 + 1)])
+    col = np.sort((np.arange(V)[:, None] + a) % V, axis=1).astype(np.uint32).ravel()
+    return inputs.CSRGraph((np.arange(V + 1) * d).astype(np.uint64), col,
+                           np.random.default_rng(d).integers(1, 256, size=V * d).astype(np.uint32))
+
+
+@pytest.mark.parametrize("d,V,n,length", [(4, 1 << 18, 16, 80), (4, 1 << 18, 8000, 80), (64, 1 << 14, 16, 80),
+                                          (64, 1 << 14, 30000, 30), (512, 1 << 12, 100, 80)])
+def test_node2vec_streams_regular_rows(csaw, d, V, n, length):
+    """Where both lists of a step are alike, streaming one is quicker than the index."""
+    g = ring(V, d)
+    assert not walk(csaw, g, inputs.uniform_vertices(n, V, 2), length, "node2vec", 9, (1, 2, 4))
