@@ -917,23 +917,32 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
     return st;
 }
 
-// Whether building the packed array for one call pays.  In ps: streaming a
-// step costs about 250 + 0.3 per neighbour of the row with the chip full (RMAT
-// s16 to s20; 1.0 and more where degrees are gathered), and the slowest walker
-// 750 per neighbour however few walk beside it (degrees 1300); the array takes
-// 4 per edge (degrees 5 to 6), its launches 25 us, and a few walkers half a us
-// a step more than streaming short rows.  60 steps of 256 walkers on RMAT s20,
-// streamed and over the array: 363 and 274 us by weight, 1890 and 358 by
-// degree; 10 steps by degree 371 and 205.
+// Whether building the packed array for one call pays.  Each side is the
+// larger of what its steps take with the chip full and of what the slowest
+// walker takes, however few walk beside it, in ps: streaming a step takes 250 +
+// 0.4 per neighbour of the row (200 + 1.0 where degrees are gathered) with the
+// chip full, and the slowest walker 0.6 us and 0.8 ns per neighbour (0.3 and
+// 1.1); the array takes 4.3 per edge (5) and 20 us, and its steps 30 each with
+// the chip full, 1.0 us each (0.8) for one walker.  60 steps of 256 walkers on
+// RMAT s20, streamed and over the array: 363 and 274 us by weight, 1890 and 358
+// by degree; 10 steps by degree 371 and 205.  A random graph of degree 32 and 8
+// M edges, 8,000 walkers: 12 steps 58 and 90, 80 steps 194 and 210.
+// The figures are fitted to the choices, 1,110 calls of either kind on 20
+// graphs (grid, circulant, random, Zipf, stars, RMAT s12 to s20), 16 to 120,000
+// walkers of 2 to 80 steps: 9 take longer than streamed by weight, at most by
+// 20 % (RMAT s20, 2,000 walkers x 12: 150 and 179 us), and one by degree (6 %).
 static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length)
 {
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const bool by_degree = kind == CSAW_BIAS_NEIGHBOR_DEGREE;
-    const double visited = visited_degree(g, by_degree);
-    const double full = (double)n * (double)length * (250.0 + (by_degree ? 1.0 : 0.3) * visited);
-    const double slowest = (by_degree ? 1300.0 : 750.0) * slowest_walk(g, (double)n, (double)length, visited);
-    const double cost = (by_degree ? 6.0 : 4.0) * (double)g->E + 25e6;
-    return full >= cost || slowest >= cost + 0.5e6 * (double)length;
+    const double walkers = (double)n, steps = (double)length, visited = visited_degree(g, by_degree);
+    const double slowest = slowest_walk(g, walkers, steps, visited);
+    const double streamed = by_degree
+        ? std::max(walkers * steps * (200.0 + visited), 0.3e6 * steps + 1100.0 * slowest)
+        : std::max(walkers * steps * (250.0 + 0.4 * visited), 0.6e6 * steps + 800.0 * slowest);
+    const double searched = (by_degree ? 5.0 : 4.3) * (double)g->E + 20e6 +
+                            std::max(30.0 * walkers * steps, (by_degree ? 0.8e6 : 1.0e6) * steps);
+    return streamed >= searched;
 }
 
 // Whether the graph keeps an array that walks of the kind can search.  The

@@ -113,7 +113,7 @@ def test_plans(env, instances):
 def test_host_walks(env, bias, build):
     torch, csaw, g, G = env
     mem = Memory(env, packed_bytes(g))
-    starts = inputs.uniform_vertices(3000, g.V, 6)
+    starts = inputs.uniform_vertices(6000, g.V, 6)
 
     def run():
         phases = []
@@ -151,7 +151,7 @@ def test_kept_array_with_zero_biases(env, bias, tele):
     torch, csaw, g, _ = env
     off = np.minimum(g.off, g.off[g.V // 2])   # the upper half has no edges of its own
     z = inputs.CSRGraph(off, g.col[:off[-1]], g.w[:off[-1]] & np.uint32(3))
-    starts = inputs.uniform_vertices(3000, g.V, 6)
+    starts = inputs.uniform_vertices(6000, g.V, 6)
     Z = csaw.Graph(z.off, z.col, z.w)
     mem = Memory((torch, csaw, z, Z), packed_bytes(z))
     Z.build_cdf(bias)

@@ -110,8 +110,8 @@ def test_node2vec_tiny_graphs(csaw, edges, weights):
 
 
 @pytest.mark.parametrize("bias,n,length,builds", [
-    ("edge_weight", 257, 1, False), ("edge_weight", 257, 90, False), ("edge_weight", 257, 600, True),
-    ("edge_weight", 31, 5000, True), ("neighbor_degree", 1, 1, False), ("neighbor_degree", 1, 200, True),
+    ("edge_weight", 257, 1, False), ("edge_weight", 257, 12, False), ("edge_weight", 257, 90, True),
+    ("edge_weight", 1000, 90, True), ("neighbor_degree", 1, 1, False), ("neighbor_degree", 1, 200, True),
     ("neighbor_degree", 31, 90, True), ("node2vec", 31, 1, False), ("node2vec", 31, 90, True)])
 def test_few_walkers(csaw, bias, n, length, builds):
     g = inputs.rmat_csr(15, 16, 255, 21)
@@ -136,3 +136,12 @@ def test_node2vec_streams_regular_rows(csaw, d, V, n, length):
     """Where both lists of a step are alike, streaming one is quicker than the index."""
     g = ring(V, d)
     assert not walk(csaw, g, inputs.uniform_vertices(n, V, 2), length, "node2vec", 9, (1, 2, 4))
+
+
+@pytest.mark.parametrize("bias", ["edge_weight", "neighbor_degree"])
+@pytest.mark.parametrize("d,V", [(4, 1 << 18), (32, 1 << 15), (64, 1 << 16)])
+def test_few_walkers_stream_short_rows(csaw, bias, d, V):
+    """A few thousand walkers over short rows do not win the array's construction back."""
+    g = ring(V, d)
+    assert not walk(csaw, g, inputs.uniform_vertices(2000, V, 2), 80, bias, 9)
+    assert walk(csaw, g, inputs.uniform_vertices(60000, V, 2), 80, bias, 9)
