@@ -14,8 +14,8 @@
 // Rows that fit one round stay in registers and need one pass.
 //
 // Work distribution: a persistent grid; each warp takes the next walker from
-// a global counter and runs all its steps.  (Uniform walks, and walks over an
-// array of the biases, are in csaw_walk_cdf.cu.)  The path row is buffered one
+// a global counter and runs all its steps.  (Most uniform walks, and walks
+// over an array of the biases, are in csaw_walk_cdf.cu.)  The path row is buffered one
 // 32-entry block per warp (lane j holds entry 32*blk + j) and written with
 // one coalesced store per block.
 #include <atomic>
@@ -575,6 +575,10 @@ __device__ __forceinline__ bool walk_pick(const WalkParams& p, const Row& row, c
             n2v_fast_pays(row.d, (uint32_t)(c.pend - c.pbeg)))
             return n2v_fast_pick(p, row, c, r, lane, s_jpos, s_jw, idx);
     }
+    if constexpr (KIND == CSAW_BIAS_UNIFORM) {
+        *idx = (uint32_t)scale_draw(r, row.d);   // b = 1: S[i] = i + 1, the pick is x itself
+        return true;
+    }
     if constexpr (KIND != CSAW_BIAS_NODE2VEC) {
         if (row.span <= TILE) {
             // One tile: lane l holds positions 4l .. 4l+3; its inclusive
@@ -694,7 +698,8 @@ __device__ __forceinline__ bool walk_pick(const WalkParams& p, const Row& row, c
 template <int KIND, bool WIDE, bool TELE, bool BATCH>
 constexpr int walk_min_blocks()
 {
-    return (KIND == CSAW_BIAS_EDGE_WEIGHT && !WIDE) ? CSAW_WALK_EW_BLOCKS
+    return KIND == CSAW_BIAS_UNIFORM ? 5
+           : (KIND == CSAW_BIAS_EDGE_WEIGHT && !WIDE) ? CSAW_WALK_EW_BLOCKS
            : KIND == CSAW_BIAS_NODE2VEC ? (TELE || BATCH ? 3 : CSAW_WALK_N2V_BLOCKS) : 4;
 }
 
@@ -844,6 +849,8 @@ static csaw_status launch_walk(int kind, uint64_t max_bias, const WalkParams& p,
 {
     const bool wide = max_bias * ROUND >= (1ull << 32);
     switch (kind) {
+    case CSAW_BIAS_UNIFORM:   // teleporting ones alone (uniform_by_warps)
+        return launch_walk_kwt<CSAW_BIAS_UNIFORM, false, true>(p, sm_count, s);
     case CSAW_BIAS_EDGE_WEIGHT:
         return wide ? launch_walk_kw<CSAW_BIAS_EDGE_WEIGHT, true>(p, sm_count, s)
                     : launch_walk_kw<CSAW_BIAS_EDGE_WEIGHT, false>(p, sm_count, s);
@@ -945,6 +952,17 @@ static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t 
     return streamed >= searched;
 }
 
+// Whether teleporting uniform walks take a warp per walker instead of a
+// thread.  A warp of 32 walkers waits for the slowest of their loads in every
+// step, which few and long walks feel; many walkers need the threads.  RMAT
+// s20 ef32 with restarts, by threads and by warps: 500 walkers x 80 steps 122
+// and 79 us, x 30 58 and 50, x 12 37 and 41; 8,000 x 80 141 and 136, x 30 67
+// and 75; smaller graphs 84, 74, 47, 48, 33, 38, 84, 134, 47 and 72.
+static bool uniform_by_warps(int kind, uint32_t tele, uint64_t n, uint32_t length)
+{
+    return kind == CSAW_BIAS_UNIFORM && tele != CSAW_TELEPORT_NONE && n <= 4096 && length > 24;
+}
+
 // Whether the graph keeps an array that walks of the kind can search.  The
 // packed one takes zero biases as they are.
 static bool walk_array_kept(const csaw_graph* g, int kind)
@@ -1033,7 +1051,8 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
     void* tmp = nullptr;   // an array built for this call
     void* a = nullptr;     // device starts and paths of a host call
     void* b = nullptr;
-    bool over_array = kind != CSAW_BIAS_NODE2VEC && (kept || build || pays);
+    bool over_array = kind != CSAW_BIAS_NODE2VEC && (kept || build || pays) &&
+                      !uniform_by_warps(kind, tele, n_walkers, length);
     const bool own = over_array && !kept && kind != CSAW_BIAS_UNIFORM;
     if (over_array && kept && kind != CSAW_BIAS_UNIFORM) {
         if (g->pack[kind]) {

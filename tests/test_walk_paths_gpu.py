@@ -145,3 +145,25 @@ def test_few_walkers_stream_short_rows(csaw, bias, d, V):
     g = ring(V, d)
     assert not walk(csaw, g, inputs.uniform_vertices(2000, V, 2), 80, bias, 9)
     assert walk(csaw, g, inputs.uniform_vertices(60000, V, 2), 80, bias, 9)
+
+
+@pytest.mark.parametrize("tele", ["restart", "jump"])
+@pytest.mark.parametrize("n,length,warps", [(1, 24, False), (1, 25, True), (500, 80, True), (4096, 33, True),
+                                            (4097, 33, False)])
+def test_uniform_teleports(csaw, tele, n, length, warps):
+    """Few and long ones by a warp per walker, which takes walkers by a counter."""
+    g = inputs.rmat_csr(12, 4, 1, 5)   # isolated vertices among them: dead ends
+    starts = inputs.uniform_vertices(n, g.V, 3)
+    G = csaw.Graph(g.off, g.col, None)
+    sizes = []
+    G.use_torch_allocator(lambda p, k: sizes.append(k))
+    import torch
+    d = torch.from_numpy(starts.view(np.int32)).cuda()
+    kw = {"teleport": tele, "teleport_q32": 1 << 29}
+    got = csaw.walk(G, d, length, "uniform", 4, **kw)
+    host = csaw.walk(G, starts, length, "uniform", 4, **kw)
+    G.use_own_allocator()
+    G.close()
+    ref = oracle.walk(g, starts, length, "uniform", 4, **kw)
+    assert np.array_equal(got.cpu().numpy().view(np.uint32), ref) and np.array_equal(host, ref)
+    assert (sizes[:1] == [8]) == warps
