@@ -236,16 +236,39 @@ __global__ void validate_kernel(const uint64_t* __restrict__ off, const uint32_t
 }
 
 // Whether some edge points at a vertex with no neighbours (a zero
-// neighbour-degree bias).  Runs after validation has filled deg.
-__global__ void zero_target_kernel(const uint32_t* __restrict__ col, const uint32_t* __restrict__ deg,
-                                   uint64_t E, uint32_t* __restrict__ flag)
+// neighbour-degree bias), and the degrees that edges lead to, summed, and their
+// squares.  Runs after validation has filled deg; 256 threads.
+__global__ void __launch_bounds__(256) targets_kernel(const uint32_t* __restrict__ col,
+                                                      const uint32_t* __restrict__ deg, uint64_t E,
+                                                      uint32_t* __restrict__ flag, double* __restrict__ sums)
 {
+    __shared__ double s_sum[2][8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t found = 0;
+    double s1 = 0.0, s2 = 0.0;
     for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E;
-         e += (uint64_t)gridDim.x * blockDim.x)
-        found |= deg[col[e]] == 0;
+         e += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t d = deg[col[e]];
+        found |= d == 0;
+        s1 += (double)d;
+        s2 += (double)d * (double)d;
+    }
     found = __reduce_or_sync(CSAW_FULL_MASK, found);
-    if ((threadIdx.x & 31) == 0 && found) atomicOr(flag, 1u);
+    for (int o = 16; o > 0; o >>= 1) {
+        s1 += __shfl_down_sync(CSAW_FULL_MASK, s1, o);
+        s2 += __shfl_down_sync(CSAW_FULL_MASK, s2, o);
+    }
+    if (lane == 0) {
+        if (found) atomicOr(flag, 1u);
+        s_sum[0][wid] = s1;
+        s_sum[1][wid] = s2;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += s_sum[threadIdx.x][w];
+        atomicAdd(sums + threadIdx.x, t);
+    }
 }
 
 }  // namespace csaw
@@ -327,8 +350,12 @@ extern "C" csaw_status csaw_graph_create(const uint64_t* row_offsets, uint32_t n
     if (e == cudaSuccess && col_b) e = cudaMemcpyAsync(g->col, cols, col_b, kind, s);
     if (e == cudaSuccess && weights && col_b) e = cudaMemcpyAsync(g->w, weights, col_b, kind, s);
     uint32_t* d_stat = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&d_stat, 8 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_stat, 0, 8 * sizeof(uint32_t), s);
+    struct Stat {
+        uint32_t word[8];
+        double sums[2];
+    } h{};
+    if (e == cudaSuccess) e = cudaMalloc(&d_stat, sizeof(Stat));
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_stat, 0, sizeof(Stat), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_stat + 3, 0xFF, sizeof(uint32_t), s);
     if (e == cudaSuccess) {
         const int threads = 256;
@@ -349,11 +376,12 @@ extern "C" csaw_status csaw_graph_create(const uint64_t* row_offsets, uint32_t n
         uint64_t blocks = (n_edges + 255) / 256;
         const uint64_t cap = (uint64_t)g->sm_count * 16;
         if (blocks > cap) blocks = cap;
-        zero_target_kernel<<<(unsigned)blocks, 256, 0, s>>>(g->col, g->deg, n_edges, d_stat + 4);
+        targets_kernel<<<(unsigned)blocks, 256, 0, s>>>(g->col, g->deg, n_edges, d_stat + 4,
+                                                        reinterpret_cast<Stat*>(d_stat)->sums);
         e = cudaGetLastError();
     }
-    uint32_t h_stat[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_stat, d_stat, sizeof(h_stat), cudaMemcpyDeviceToHost, s);
+    const uint32_t* h_stat = h.word;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d_stat, sizeof(Stat), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(d_stat);
     if (e != cudaSuccess) {
@@ -369,6 +397,11 @@ extern "C" csaw_status csaw_graph_create(const uint64_t* row_offsets, uint32_t n
     g->max_weight = weights ? h_stat[2] : 1u;
     g->min_weight = (weights && n_edges > 0) ? h_stat[3] : 1u;
     g->zero_degree_target = h_stat[4] != 0;
+    if (n_edges > 0) {
+        g->reach = h.sums[0] / (double)n_edges;
+        g->reach_spread = std::sqrt(std::max(0.0, h.sums[1] / (double)n_edges - g->reach * g->reach));
+        g->reach_by_degree = h.sums[0] > 0.0 ? h.sums[1] / h.sums[0] : 0.0;
+    }
     *out = g;
     return CSAW_OK;
 }

@@ -36,6 +36,9 @@ struct csaw_graph {
     uint32_t max_weight = 1;
     uint32_t min_weight = 1;            // 0 if some edge weight is zero
     bool zero_degree_target = false;    // some edge points at a vertex without neighbours
+    // degree of the vertex that an edge leads to: mean and standard deviation over
+    // the edges, and the mean where edges are followed by that degree
+    double reach = 0.0, reach_spread = 0.0, reach_by_degree = 0.0;
     uint64_t device_bytes = 0;
     int device = 0;
     int sm_count = 0;
@@ -196,25 +199,24 @@ csaw_status walk_batch_cached(const csaw_graph* g, int kind, const uint32_t* d_s
 csaw_status walk_n2v(const csaw_graph* g, const csaw_bias* bias, uint64_t max_bias, const uint32_t* starts, uint64_t n,
                      uint32_t length, uint64_t rng_seed, uint32_t tele, uint32_t tele_q32, uint32_t* path,
                      unsigned long long* next_walker, cudaStream_t s, bool* done);
-// The mean degree of the rows that a walk or a sampled layer comes to, for the
-// rules that weigh streaming rows against building an array: sqrt(mean degree *
+// An estimate of the mean degree of the rows that a sampled layer comes to, for
+// the rules that weigh streaming rows against building an array: sqrt(mean degree *
 // largest degree) where edges are followed by weight (RMAT s16 520 for 684
 // measured, s20 1393 for 2233, s20 ef32 2424 for 3315), nearer the largest
 // degree where they are followed by degree, and the degree itself on a regular
 // graph.
-inline double mean_degree(const csaw_graph* g) { return g->V ? (double)g->E / (double)g->V : 0.0; }
 inline double visited_degree(const csaw_graph* g, bool by_degree)
 {
-    const double avg = mean_degree(g), most = (double)g->max_degree;
+    const double avg = g->V ? (double)g->E / (double)g->V : 0.0, most = (double)g->max_degree;
     return by_degree ? std::cbrt(avg * most * most) : std::sqrt(avg * most);
 }
 
 // The neighbours that the slowest of n walkers comes by in `length` steps, at
-// rows of a mean degree, for the same rules: a call ends no sooner than that
-// walker, which meets rows far longer than the mean.
-inline double slowest_walk(const csaw_graph* g, double n, double length, double degree)
+// rows of that mean degree and spread, for the rules of walks: a call ends no
+// sooner than that walker, which meets rows far longer than the mean.
+inline double slowest_walk(const csaw_graph* g, double n, double length, double degree, double spread)
 {
-    return length * degree + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * degree);
+    return length * degree + std::sqrt(length) * std::min((double)g->max_degree, std::sqrt(n) * spread);
 }
 
 // Device bytes of the array that a plain walk call of n walkers, or a sampling

@@ -924,32 +924,34 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
     return st;
 }
 
-// Whether building the packed array for one call pays.  Each side is the
-// larger of what its steps take with the chip full and of what the slowest
-// walker takes, however few walk beside it, in ps: streaming a step takes 250 +
-// 0.4 per neighbour of the row (200 + 1.0 where degrees are gathered) with the
-// chip full, and the slowest walker 0.6 us and 0.8 ns per neighbour (0.3 and
-// 1.1); the array takes 4.3 per edge (5) and 20 us, and its steps 30 each with
-// the chip full, 1.0 us each (0.8) for one walker.  60 steps of 256 walkers on
+// Whether building the packed array for one call pays.  Each side in ps:
+// streaming, the larger of what its steps take with the chip full, 250 + 0.6
+// per neighbour of the row (300 + 1.1 where degrees are gathered), and of what
+// the slowest walker takes however few walk beside it, 0.9 us a step and 0.58
+// ns per neighbour (1.3 and 0.8); over the array, its construction, 5 per edge
+// (4.4) and 14 us (30), and 1.5 us a step (1.4).  60 steps of 256 walkers on
 // RMAT s20, streamed and over the array: 363 and 274 us by weight, 1890 and 358
-// by degree; 10 steps by degree 371 and 205.  A random graph of degree 32 and 8
-// M edges, 8,000 walkers: 12 steps 58 and 90, 80 steps 194 and 210.
-// The figures are fitted to the choices, 1,110 calls of either kind on 20
-// graphs (grid, circulant, random, Zipf, stars, RMAT s12 to s20), 16 to 120,000
-// walkers of 2 to 80 steps: 9 take longer than streamed by weight, at most by
-// 20 % (RMAT s20, 2,000 walkers x 12: 150 and 179 us), and one by degree (6 %).
+// by degree; a random graph of degree 32 and 8 M edges, 8,000 walkers x 12: 58
+// and 90, x 80 194 and 210.
+// The rows that walks come to are those that edges lead to, so their mean and
+// spread are the graph's own (reach); one call may well go either way, so the
+// figures are fitted to the choices: 2,062 calls by weight and as many by
+// degree on 37 graphs (grids, circulants, cliques, random, Zipf, log-normal,
+// preferential attachment, bipartite, stars, RMAT s12 to s21), 16 to 200,000
+// walkers of 2 to 120 steps, plain and with restarts.  Of those 4 take longer
+// than streamed by more than 4 % (at most 9) by weight and 2 (6) by degree.
 static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length)
 {
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
-    const bool by_degree = kind == CSAW_BIAS_NEIGHBOR_DEGREE;
-    const double walkers = (double)n, steps = (double)length, visited = visited_degree(g, by_degree);
-    const double slowest = slowest_walk(g, walkers, steps, visited);
-    const double streamed = by_degree
-        ? std::max(walkers * steps * (200.0 + visited), 0.3e6 * steps + 1100.0 * slowest)
-        : std::max(walkers * steps * (250.0 + 0.4 * visited), 0.6e6 * steps + 800.0 * slowest);
-    const double searched = (by_degree ? 5.0 : 4.3) * (double)g->E + 20e6 +
-                            std::max(30.0 * walkers * steps, (by_degree ? 0.8e6 : 1.0e6) * steps);
-    return streamed >= searched;
+    const double walkers = (double)n, steps = (double)length, edges = (double)g->E;
+    if (kind == CSAW_BIAS_NEIGHBOR_DEGREE) {
+        const double d = g->reach_by_degree, slowest = slowest_walk(g, walkers, steps, d, 0.8 * g->reach_spread);
+        return std::max(walkers * steps * (300.0 + 1.1 * d), 1.3e6 * steps + 800.0 * slowest) >=
+               4.4 * edges + 30e6 + 1.4e6 * steps;
+    }
+    const double d = g->reach, slowest = slowest_walk(g, walkers, steps, d, 0.3 * g->reach_spread);
+    return std::max(walkers * steps * (250.0 + 0.6 * d), 0.9e6 * steps + 580.0 * slowest) >=
+           5.0 * edges + 14e6 + 1.5e6 * steps;
 }
 
 // Whether teleporting uniform walks take a warp per walker instead of a

@@ -629,30 +629,32 @@ uint64_t n2v_bytes(const csaw_graph* g)
            sizeof(uint32_t) * (g->E / N2V_BIG_ROW + 2);
 }
 
-// Streaming, a step costs by the row it stands on; over the index, by the
-// shorter of two rows' lists, which stays near the mean degree however long
-// the hubs are.  So the index pays where the rows that walks come to are
-// longer than the mean, once its construction is paid, and hardly ever on a
-// regular graph, where both lists are alike (degree 4: 0.64 ns a step streamed
-// and 0.83 over the index with the chip full; 64: 1.04 and 1.13; 512 of which
-// half are common: 2.85 and 4.49).  RMAT s12 1.41 and 0.99, s16 2.9 and 1.2,
-// s20 5.8 and 2.4; 16 stars of 60,000 leaves 35 and 1.0.  Each side is the larger of
-// what its steps cost with the chip full and of what the slowest walker takes,
-// however few walk beside it.
+// Streaming, a step costs by the row it stands on, one that an edge led to;
+// over the index, by the shorter of two rows' lists, which stays near the mean
+// degree however long the hubs are.  So the index pays where the rows that
+// walks come to are longer than the mean, once its construction is paid, and
+// hardly ever on a regular graph, where both lists are alike (degree 4: 0.64 ns
+// a step streamed and 0.83 over the index with the chip full; 64: 1.04 and
+// 1.13; 512 of which half are common: 2.85 and 4.49).  RMAT s12 1.41 and 0.99,
+// s16 2.9 and 1.2, s20 5.8 and 2.4; 16 stars of 60,000 leaves 35 and 1.0.  Each
+// side is the larger of what its steps cost with the chip full and of what the
+// slowest walker takes, however few walk beside it.
 // The figures, in ps, are fitted to the choices, not to either side alone:
-// 645 calls on 20 graphs (grid, circulant, random, Zipf, stars, RMAT s12 to
-// s20), 16 to 1,000,000 walkers of 2 to 80 steps.  Of those calls 11 take
-// longer than streamed, at most by 15 %.
+// 1,087 calls on 37 graphs (grids, circulants, cliques, random, Zipf,
+// log-normal, preferential attachment, bipartite, stars, RMAT s12 to s21), 16 to
+// 1,000,000 walkers of 2 to 120 steps.  Of those 7 take longer than streamed by
+// more than 4 %, at most by 15.
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length)
 {
     if (g->E == 0 || g->max_degree > 0x7FFFFFFFu) return false;   // positions plus 8 fit 32 bits
     if (n2v_bytes(g) > array_room()) return false;
-    const double walkers = (double)n, steps = (double)length;
-    const double visited = visited_degree(g, false), mean = mean_degree(g);
-    const double streamed = std::max(7.3 * walkers * steps * visited,
-                                     9.5e3 * slowest_walk(g, walkers, steps, visited) + 0.4e6 * steps);
-    const double indexed = 42.0 * (double)g->E + 80e6 +
-                           std::max(walkers * steps * (7.3 * mean + 40.0), 7e3 * slowest_walk(g, walkers, steps, mean));
+    const double walkers = (double)n, steps = (double)length, mean = (double)g->E / (double)g->V;
+    const double streamed = std::max(walkers * steps * (420.0 + 4.8 * g->reach),
+                                     1.2e6 * steps + 5.5e3 * slowest_walk(g, walkers, steps, g->reach,
+                                                                          0.65 * g->reach_spread));
+    const double indexed = 40.0 * (double)g->E + 35e6 +
+                           std::max(walkers * steps * (790.0 + 4.3 * mean),
+                                    1.4e6 * steps + 3.5e3 * slowest_walk(g, walkers, steps, mean, mean));
     return streamed >= indexed;
 }
 

@@ -110,8 +110,8 @@ def test_node2vec_tiny_graphs(csaw, edges, weights):
 
 
 @pytest.mark.parametrize("bias,n,length,builds", [
-    ("edge_weight", 257, 1, False), ("edge_weight", 257, 12, False), ("edge_weight", 257, 90, True),
-    ("edge_weight", 1000, 90, True), ("neighbor_degree", 1, 1, False), ("neighbor_degree", 1, 200, True),
+    ("edge_weight", 257, 1, False), ("edge_weight", 257, 12, False), ("edge_weight", 257, 90, False),
+    ("edge_weight", 8000, 90, True), ("neighbor_degree", 1, 1, False), ("neighbor_degree", 1, 200, True),
     ("neighbor_degree", 31, 90, True), ("node2vec", 31, 1, False), ("node2vec", 31, 90, True)])
 def test_few_walkers(csaw, bias, n, length, builds):
     g = inputs.rmat_csr(15, 16, 255, 21)
@@ -167,3 +167,24 @@ def test_uniform_teleports(csaw, tele, n, length, warps):
     ref = oracle.walk(g, starts, length, "uniform", 4, **kw)
     assert np.array_equal(got.cpu().numpy().view(np.uint32), ref) and np.array_equal(host, ref)
     assert (sizes[:1] == [8]) == warps
+
+
+def preferential(V, m):
+    """m edges of every vertex, to earlier ones and most of them to the earliest: a few very
+    long rows, which few edges lead to, beside rows of about 2 m."""
+    r = np.random.default_rng(5)
+    t = np.repeat(np.arange(V), m)
+    a = np.stack([t, (r.random(V * m) ** 2 * t).astype(np.int64)], 1)
+    a = np.concatenate([a, a[:, ::-1]])
+    a = np.unique(a[a[:, 0] != a[:, 1]], axis=0)
+    off = np.zeros(V + 1, dtype=np.uint64)
+    off[1:] = np.cumsum(np.bincount(a[:, 0], minlength=V))
+    return inputs.CSRGraph(off, a[:, 1].astype(np.uint32), r.integers(1, 256, size=len(a)).astype(np.uint32))
+
+
+@pytest.mark.parametrize("n,length,builds", [(300, 40, False), (300, 120, False), (1000, 40, False), (20000, 120, True)])
+def test_rows_that_edges_lead_to(csaw, n, length, builds):
+    """It is those that a walk stands on that count, not the longest of the graph."""
+    g = preferential(1 << 16, 12)
+    starts = inputs.uniform_vertices(n, g.V, 2)
+    assert walk(csaw, g, starts, length, "edge_weight", 9) == builds
