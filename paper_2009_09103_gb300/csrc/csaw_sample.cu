@@ -2290,30 +2290,38 @@ struct Pipeline {
 };
 
 // Whether a run should build the packed array and draw long rows from it (and
-// read degrees from it).  The array takes about 4.3 ps per edge of the graph
-// and 20 us.  Against it, in ps: with several instances, the grouping of hub
-// items and the hubs' own prefix sums (150 us in small runs, and 150 per
-// frontier entry in large ones: RMAT s12 to s22); with one, whose long rows a
-// block each would scan, about 2 per neighbour of a row reached by an edge
-// (see visited_degree).  A frontier is taken as eight times the one before,
-// most rows being short.  The batched s22 plan (2048 instances, 32 M edges of
-// frontier) draws its long rows in 4.9 ms, with 0.6 for the array, against 8.3
-// over shared hub arrays.
+// read degrees from it).  With several instances the array stands against the
+// grouping of hub items and the hubs' own prefix sums; with one, whose long
+// rows a block each scans, against the longest of them in each layer, which
+// the layer waits for.  The rows of later layers are those that edges lead to
+// (reach), the longest of f of them about the mean and sqrt(f) times their
+// spread; a frontier is taken as eight times the one before, most rows being
+// short.  The batched s22 plan (2048 instances, 32 M edges of frontier) draws
+// its long rows in 4.9 ms, with 0.6 for the array, against 8.3 over shared hub
+// arrays.
+// The figures are fitted to the choices: 3,204 calls and plan runs on 27 graphs
+// (grids, circulants, cliques, random, Zipf, log-normal, preferential
+// attachment, bipartite, stars, RMAT s12 to s21), 10 to 135,000 seeds, one to
+// three layers.  Of those 9 take longer than without the array by more than 4 %
+// with several instances, at most by 10, and one (5) with one.
 static bool sample_array_pays(const Pipeline& P, uint64_t n_seeds)
 {
     const csaw_graph* g = P.g;
     if (P.kind == CSAW_BIAS_UNIFORM || P.cached || P.zero_bias || !pack_fits(g, P.kind) || n_seeds == 0) return false;
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
-    const double visited = visited_degree(g, false);
-    double entries = 0, reached = 0, f = (double)n_seeds;
+    double entries = 0, reached = 0, longest = 0, f = (double)n_seeds;
     for (uint32_t l = 0; l < P.depth; ++l) {
         entries += f;
-        if (l) reached += f;
+        if (l) {
+            reached += f;
+            longest += std::min((double)g->max_degree, g->reach + std::sqrt(f) * g->reach_spread);
+        }
         f *= std::min<double>(P.fanout[l], 8.0);
         f = std::min(f, (double)P.n_inst * (double)g->V);
     }
-    const double cost = 4.3 * (double)g->E + 20e6;
-    return P.n_inst > 1 ? 150e6 + 150.0 * entries >= cost : 2.0 * reached * visited >= cost + 40e6;
+    const double edges = (double)g->E;   // all in ps
+    if (P.n_inst > 1) return 30e6 * P.depth + 350.0 * entries + 30e3 * longest >= 2.5 * edges + 20e6;
+    return std::max(0.2 * reached * g->reach, 1100.0 * longest) >= 4.5 * edges + 55e6;
 }
 
 uint64_t sample_array_bytes(csaw_graph* g, int kind, uint32_t n_inst, uint64_t n_seeds, uint32_t depth,
