@@ -925,33 +925,35 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
 }
 
 // Whether building the packed array for one call pays.  Each side in ps:
-// streaming, the larger of what its steps take with the chip full, 250 + 0.6
-// per neighbour of the row (300 + 1.1 where degrees are gathered), and of what
-// the slowest walker takes however few walk beside it, 0.9 us a step and 0.58
-// ns per neighbour (1.3 and 0.8); over the array, its construction, 5 per edge
-// (4.4) and 14 us (30), and 1.5 us a step (1.4).  60 steps of 256 walkers on
-// RMAT s20, streamed and over the array: 363 and 274 us by weight, 1890 and 358
-// by degree; a random graph of degree 32 and 8 M edges, 8,000 walkers x 12: 58
-// and 90, x 80 194 and 210.
+// streaming, the larger of what its steps take with the chip full, 257 + 0.85
+// per neighbour of the row (255 + 0.81 where degrees are gathered), and of what
+// the slowest walker takes however few walk beside it, 0.83 us a step and 0.68
+// ns per neighbour (1.23 and 0.76); over the array, its construction, 4.0 per
+// edge (4.2) and 20 us (18), and 1.4 us a step, 0.8 more where walks jump to
+// any vertex, whose record is then cold.  60 steps of 256 walkers on RMAT s20,
+// streamed and over the array: 363 and 274 us by weight, 1890 and 358 by
+// degree; a random graph of degree 32 and 8 M edges, 8,000 walkers x 12: 58 and
+// 90, x 80 194 and 210.
 // The rows that walks come to are those that edges lead to, so their mean and
 // spread are the graph's own (reach); one call may well go either way, so the
 // figures are fitted to the choices: 2,062 calls by weight and as many by
 // degree on 37 graphs (grids, circulants, cliques, random, Zipf, log-normal,
 // preferential attachment, bipartite, stars, RMAT s12 to s21), 16 to 200,000
-// walkers of 2 to 120 steps, plain and with restarts.  Of those 4 take longer
-// than streamed by more than 4 % (at most 9) by weight and 2 (6) by degree.
-static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length)
+// walkers of 2 to 120 steps, plain and with restarts.  Of those 12 take longer
+// than streamed by more than 4 % (at most 24) by weight and 7 (14) by degree.
+static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length, uint32_t tele)
 {
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const double walkers = (double)n, steps = (double)length, edges = (double)g->E;
+    const double jump = tele == CSAW_TELEPORT_JUMP ? 0.8e6 : 0.0;
     if (kind == CSAW_BIAS_NEIGHBOR_DEGREE) {
-        const double d = g->reach_by_degree, slowest = slowest_walk(g, walkers, steps, d, 0.8 * g->reach_spread);
-        return std::max(walkers * steps * (300.0 + 1.1 * d), 1.3e6 * steps + 800.0 * slowest) >=
-               4.4 * edges + 30e6 + 1.4e6 * steps;
+        const double d = g->reach_by_degree, slowest = slowest_walk(g, walkers, steps, d, 0.633 * g->reach_spread);
+        return std::max(walkers * steps * (255.0 + 0.807 * d), 1.23e6 * steps + 764.0 * slowest) >=
+               4.21 * edges + 18.1e6 + (1.43e6 + jump) * steps;
     }
-    const double d = g->reach, slowest = slowest_walk(g, walkers, steps, d, 0.3 * g->reach_spread);
-    return std::max(walkers * steps * (250.0 + 0.6 * d), 0.9e6 * steps + 580.0 * slowest) >=
-           5.0 * edges + 14e6 + 1.5e6 * steps;
+    const double d = g->reach, slowest = slowest_walk(g, walkers, steps, d, 0.225 * g->reach_spread);
+    return std::max(walkers * steps * (257.0 + 0.852 * d), 0.831e6 * steps + 678.0 * slowest) >=
+           4.03 * edges + 20.4e6 + (1.38e6 + jump) * steps;
 }
 
 // Whether teleporting uniform walks take a warp per walker instead of a
@@ -977,7 +979,7 @@ uint64_t walk_array_bytes(const csaw_graph* g, const csaw_bias* bias, uint64_t n
     int kind;
     if (check_bias(g, bias, true, &kind) != CSAW_OK) return 0;
     if (kind == CSAW_BIAS_NODE2VEC) return n2v_index_pays(g, n, length) ? n2v_bytes(g) : 0;
-    const bool builds = !walk_array_kept(g, kind) && pack_fits(g, kind) && walk_array_pays(g, kind, n, length);
+    const bool builds = !walk_array_kept(g, kind) && pack_fits(g, kind) && walk_array_pays(g, kind, n, length, CSAW_TELEPORT_NONE);
     return builds ? sizeof(uint64_t) * pack_layout(g->E, g->V).words : 0;
 }
 
@@ -1046,7 +1048,7 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
     const bool kept = walk_array_kept(g, kind);
     const bool build = !kept && tele == CSAW_TELEPORT_NONE && opts && opts->build_cdf && cdf_kind_positive(g, kind);
     const bool pays = !kept && !build && kind != CSAW_BIAS_NODE2VEC && pack_fits(g, kind) &&
-                      walk_array_pays(g, kind, n_walkers, length);
+                      walk_array_pays(g, kind, n_walkers, length, tele);
     WalkArray arr;
     arr.tele = tele;
     arr.tele_q32 = tele != CSAW_TELEPORT_NONE ? opts->teleport_q32 : 0u;

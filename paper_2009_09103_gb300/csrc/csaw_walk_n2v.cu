@@ -637,24 +637,23 @@ uint64_t n2v_bytes(const csaw_graph* g)
 // a step streamed and 0.83 over the index with the chip full; 64: 1.04 and
 // 1.13; 512 of which half are common: 2.85 and 4.49).  RMAT s12 1.41 and 0.99,
 // s16 2.9 and 1.2, s20 5.8 and 2.4; 16 stars of 60,000 leaves 35 and 1.0.  Each
-// side is the larger of what its steps cost with the chip full and of what the
-// slowest walker takes, however few walk beside it.
-// The figures, in ps, are fitted to the choices, not to either side alone:
-// 1,087 calls on 37 graphs (grids, circulants, cliques, random, Zipf,
-// log-normal, preferential attachment, bipartite, stars, RMAT s12 to s21), 16 to
-// 1,000,000 walkers of 2 to 120 steps.  Of those 7 take longer than streamed by
-// more than 4 %, at most by 15.
+// side is what its steps cost with the chip full and what the slowest walker
+// takes besides, however few walk beside it.
+// The figures, in ps, are fitted to the choices, not to either side alone (a
+// neighbour held to cost the index 1.4 to 1.6 times as much as streaming, as on
+// the regular rows of 512): 1,087 calls on 37 graphs (grids, circulants,
+// cliques, random, Zipf, log-normal, preferential attachment, bipartite, stars,
+// RMAT s12 to s21), 16 to 1,000,000 walkers of 2 to 120 steps.  Of those 10
+// take longer than streamed by more than 4 %, at most by 21.
 bool n2v_index_pays(const csaw_graph* g, uint64_t n, uint32_t length)
 {
     if (g->E == 0 || g->max_degree > 0x7FFFFFFFu) return false;   // positions plus 8 fit 32 bits
     if (n2v_bytes(g) > array_room()) return false;
     const double walkers = (double)n, steps = (double)length, mean = (double)g->E / (double)g->V;
-    const double streamed = std::max(walkers * steps * (420.0 + 4.8 * g->reach),
-                                     1.2e6 * steps + 5.5e3 * slowest_walk(g, walkers, steps, g->reach,
-                                                                          0.65 * g->reach_spread));
-    const double indexed = 40.0 * (double)g->E + 35e6 +
-                           std::max(walkers * steps * (790.0 + 4.3 * mean),
-                                    1.4e6 * steps + 3.5e3 * slowest_walk(g, walkers, steps, mean, mean));
+    const double slowest = slowest_walk(g, walkers, steps, g->reach, 0.638 * g->reach_spread);
+    const double streamed = walkers * steps * (15.6 + 4.42 * g->reach) + 0.938e6 * steps + 5.14e3 * slowest;
+    const double indexed = 38.9 * (double)g->E + 46.3e6 + walkers * steps * (410.0 + 6.26 * mean) +
+                           (0.466e6 + 8.2e3 * mean) * steps;
     return streamed >= indexed;
 }
 
