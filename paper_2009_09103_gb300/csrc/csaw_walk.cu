@@ -925,46 +925,50 @@ csaw_status walk_batch(const csaw_graph* g, const csaw_bias* bias, const uint32_
 }
 
 // Whether building the packed array for one call pays.  Each side in ps:
-// streaming, the larger of what its steps take with the chip full, 257 + 0.85
-// per neighbour of the row (255 + 0.81 where degrees are gathered), and of what
-// the slowest walker takes however few walk beside it, 0.83 us a step and 0.68
-// ns per neighbour (1.23 and 0.76); over the array, its construction, 4.0 per
-// edge (4.2) and 20 us (18), and 1.4 us a step, 0.8 more where walks jump to
-// any vertex, whose record is then cold.  60 steps of 256 walkers on RMAT s20,
-// streamed and over the array: 363 and 274 us by weight, 1890 and 358 by
-// degree; a random graph of degree 32 and 8 M edges, 8,000 walkers x 12: 58 and
-// 90, x 80 194 and 210.
+// streaming, the larger of what its steps take with the chip full, 338 + 0.39
+// per neighbour of the row (302 + 0.61 where degrees are gathered), and of what
+// the slowest walker takes however few walk beside it, 1.5 us a step and 0.62
+// ns per neighbour (1.1 and 0.82); over the array, its construction, 3.2 per
+// edge (4.7) and 17 us, and 1.7 us a step (1.3).  A step waits the longer the
+// larger the graph: for every doubling past 2^19 edges 0.05 us more streamed
+// (0.23) and 0.12 over the array (0.13), and 0.06 more there where walks jump to
+// any vertex.  60 steps of 256 walkers on RMAT s20, streamed and over the array:
+// 363 and 274 us by weight, 1890 and 358 by degree; a random graph of degree 32
+// and 8 M edges, 8,000 walkers x 12: 58 and 90, x 80 194 and 210.
 // The rows that walks come to are those that edges lead to, so their mean and
 // spread are the graph's own (reach); one call may well go either way, so the
 // figures are fitted to the choices: 2,062 calls by weight and as many by
 // degree on 37 graphs (grids, circulants, cliques, random, Zipf, log-normal,
 // preferential attachment, bipartite, stars, RMAT s12 to s21), 16 to 200,000
-// walkers of 2 to 120 steps, plain and with restarts.  Of those 12 take longer
-// than streamed by more than 4 % (at most 24) by weight and 7 (14) by degree.
+// walkers of 2 to 120 steps, plain and with restarts.  Of those 8 take longer
+// than streamed by more than 4 % (at most 9) by weight and 6 (14) by degree.
 static bool walk_array_pays(const csaw_graph* g, int kind, uint64_t n, uint32_t length, uint32_t tele)
 {
     if (sizeof(uint64_t) * pack_layout(g->E, g->V).words > array_room()) return false;
     const double walkers = (double)n, steps = (double)length, edges = (double)g->E;
-    const double jump = tele == CSAW_TELEPORT_JUMP ? 0.8e6 : 0.0;
+    const double doublings = std::max(0.0, std::log2(edges) - 19.0);
+    const double jump = tele == CSAW_TELEPORT_JUMP ? 0.06e6 * doublings : 0.0;
     if (kind == CSAW_BIAS_NEIGHBOR_DEGREE) {
-        const double d = g->reach_by_degree, slowest = slowest_walk(g, walkers, steps, d, 0.633 * g->reach_spread);
-        return std::max(walkers * steps * (255.0 + 0.807 * d), 1.23e6 * steps + 764.0 * slowest) >=
-               4.21 * edges + 18.1e6 + (1.43e6 + jump) * steps;
+        const double d = g->reach_by_degree, slowest = slowest_walk(g, walkers, steps, d, 0.617 * g->reach_spread);
+        return std::max(walkers * steps * (302.0 + 0.608 * d), (1.1e6 + 0.233e6 * doublings) * steps + 819.0 * slowest) >=
+               4.73 * edges + 17.3e6 + 3.4 * walkers * steps + (1.33e6 + 0.13e6 * doublings + jump) * steps;
     }
-    const double d = g->reach, slowest = slowest_walk(g, walkers, steps, d, 0.225 * g->reach_spread);
-    return std::max(walkers * steps * (257.0 + 0.852 * d), 0.831e6 * steps + 678.0 * slowest) >=
-           4.03 * edges + 20.4e6 + (1.38e6 + jump) * steps;
+    const double d = g->reach, slowest = slowest_walk(g, walkers, steps, d, 0.183 * g->reach_spread);
+    return std::max(walkers * steps * (338.0 + 0.385 * d), (1.48e6 + 0.0469e6 * doublings) * steps + 624.0 * slowest) >=
+           3.15 * edges + 17.5e6 + 11.3 * walkers * steps + (1.68e6 + 0.123e6 * doublings + jump) * steps;
 }
 
 // Whether teleporting uniform walks take a warp per walker instead of a
 // thread.  A warp of 32 walkers waits for the slowest of their loads in every
-// step, which few and long walks feel; many walkers need the threads.  RMAT
-// s20 ef32 with restarts, by threads and by warps: 500 walkers x 80 steps 122
-// and 79 us, x 30 58 and 50, x 12 37 and 41; 8,000 x 80 141 and 136, x 30 67
-// and 75; smaller graphs 84, 74, 47, 48, 33, 38, 84, 134, 47 and 72.
-static bool uniform_by_warps(int kind, uint32_t tele, uint64_t n, uint32_t length)
+// step, which few and long walks feel, and longer walks of a few thousand on a
+// large graph; many walkers need the threads.  With restarts, by threads and by
+// warps: RMAT s20 ef32 500 walkers x 80 steps 122 and 79 us, x 30 58 and 50,
+// 2,000 x 80 139 and 92, 8,000 x 80 141 and 136; RMAT s14 84 and 76, 47 and 48,
+// 84 and 92, 84 and 138.
+static bool uniform_by_warps(const csaw_graph* g, int kind, uint32_t tele, uint64_t n, uint32_t length)
 {
-    return kind == CSAW_BIAS_UNIFORM && tele != CSAW_TELEPORT_NONE && n <= 4096 && length > 24;
+    return kind == CSAW_BIAS_UNIFORM && tele != CSAW_TELEPORT_NONE && length > 32 &&
+           n <= (g->E >= (1ull << 23) ? 4096 : 1024);
 }
 
 // Whether the graph keeps an array that walks of the kind can search.  The
@@ -1056,7 +1060,7 @@ extern "C" csaw_status csaw_walk_ex(csaw_graph* g, const uint32_t* starts, uint6
     void* a = nullptr;     // device starts and paths of a host call
     void* b = nullptr;
     bool over_array = kind != CSAW_BIAS_NODE2VEC && (kept || build || pays) &&
-                      !uniform_by_warps(kind, tele, n_walkers, length);
+                      !uniform_by_warps(g, kind, tele, n_walkers, length);
     const bool own = over_array && !kept && kind != CSAW_BIAS_UNIFORM;
     if (over_array && kept && kind != CSAW_BIAS_UNIFORM) {
         if (g->pack[kind]) {

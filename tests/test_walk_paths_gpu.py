@@ -148,8 +148,8 @@ def test_few_walkers_stream_short_rows(csaw, bias, d, V):
 
 
 @pytest.mark.parametrize("tele", ["restart", "jump"])
-@pytest.mark.parametrize("n,length,warps", [(1, 24, False), (1, 25, True), (500, 80, True), (4096, 33, True),
-                                            (4097, 33, False)])
+@pytest.mark.parametrize("n,length,warps", [(1, 32, False), (1, 33, True), (500, 80, True), (1024, 33, True),
+                                            (1025, 33, False)])
 def test_uniform_teleports(csaw, tele, n, length, warps):
     """Few and long ones by a warp per walker, which takes walkers by a counter."""
     g = inputs.rmat_csr(12, 4, 1, 5)   # isolated vertices among them: dead ends
