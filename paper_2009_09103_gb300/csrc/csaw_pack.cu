@@ -5,7 +5,7 @@
 // One pass over the edges writes the packed groups, their sums inside 64-edge
 // blocks and the block ends relative to the thread block's chunk; the chunk
 // totals are scanned by one block, then added to the block ends.  Bound by
-// memory: 8 bytes read and 8.6 written per edge (neighbour degree adds its
+// memory: 8 bytes read and 8.67 written per edge (neighbour degree adds its
 // gathers, once).  RMAT s20, 31 M edges: 0.077 ms for the edges (6.7 TB/s),
 // 0.11 in all, against 0.15 for the segmented scan of the summaries.
 #include "csaw_internal.cuh"

@@ -319,7 +319,7 @@ __device__ __forceinline__ void sector_biases(const SelParams& p, uint64_t beg, 
 // WARP_MAX_DEG neighbours with S in this warp's shared slot.  A lane holds
 // eight consecutive neighbours (one 32-byte load), so that the row takes one
 // warp scan of lane totals, of 32-bit sums where they fit (A).  Bound by
-// instruction issue (70 %): RMAT s22, 2048 instances, neighbour degree, both
+// instruction issue: RMAT s22, 2048 instances, neighbour degree, both
 // layers 4.5 ms, against 5.1 with eight 64-bit scans of strided tiles and 5.7
 // with the degrees gathered and whole rows among the items.
 template <int KIND, class A>
@@ -2259,7 +2259,7 @@ struct Pipeline {
         // long rows take the CTA path without the grouping kernels
         hub_path = !cached && n_inst > 1 && (kind == CSAW_BIAS_EDGE_WEIGHT || kind == CSAW_BIAS_NEIGHBOR_DEGREE);
         // vertex order pays only when several instances can hold the same hub,
-        // and over the packed array only where its rows do not stay in L2 (8.6
+        // and over the packed array only where its rows do not stay in L2 (8.67
         // bytes per edge) and there are items enough: RMAT s20, 1024 instances,
         // 1 M seeds 3.56 ms in order, 3.67 without; 64 K seeds 0.68 and 0.63;
         // s16, 1 M seeds 2.67 and 2.63; the s22 plan 14.4 and 15.5

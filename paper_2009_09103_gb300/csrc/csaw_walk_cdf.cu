@@ -34,7 +34,7 @@ namespace csaw {
 // summaries and weights: 133 DRAM bytes a step instead of 276 (a missing
 // sector is fetched as 64 bytes, so what one pick needs lies in one such
 // line), four dependent loads instead of ten.  Bound by scattered sectors (six
-// a step; a seventh cost 0.1 ms; DRAM 4.5 TB/s, L2 65 % busy), not by lanes:
+// a step; a seventh cost 0.1 ms; DRAM 4.8 TB/s, on s19 L2 62 % busy), not by lanes:
 // leaving out the walkers that cannot move (38 %) made it slower.  Six blocks
 // per SM; seven spill (1.90 ms), five are even.
 constexpr int WC_THREADS = 256;

@@ -28,8 +28,8 @@
 //
 // Measured (RMAT s20 ef32, 1 M walkers, 40 steps): 150 ms with the index's
 // construction (2.6 ms) against 459 ms for the streaming kernel.  Bound by
-// instruction issue and dependent loads together (issue active 59 %, DRAM 35 %
-// at 32 warps per SM; 24 or 40 warps are 7-9 % slower).
+// instruction issue and dependent loads together (24 or 40 warps per SM instead
+// of 32 are 7-9 % slower).
 #include <atomic>
 #include <cmath>
 
