@@ -1266,7 +1266,8 @@ def main():
     ap.add_argument("--no-variant", action="store_true",
                     help="walks: skip the default call measured after the main line")
     ap.add_argument("--streaming", action="store_true",
-                    help="walks: the main line streams each step's row (no cumulative array)")
+                    help="walks: the main line is the default call (without build_cdf), which builds the packed array by "
+                         "itself where that pays")
     ap.add_argument("--cdf", action="store_true",
                     help="build the cached per-edge cumulative array of the static bias first")
     ap.add_argument("--plain-instances", type=int, default=4096,

@@ -133,12 +133,12 @@ csaw_status csaw_graph_get_info(const csaw_graph* g, csaw_graph_info* out);
  * Sec. II-B computed once instead of at every selection -- and a summary of
  * every 8th sum (9.1 bytes per edge in all), and for walks, where the biases
  * are below 2^26 and memory allows, the biases packed beside their columns
- * with running sums (8.6 bytes per edge + 16 per vertex).
+ * with running sums (8.67 bytes per edge + 16 per vertex).
  * Afterwards csaw_walk, csaw_sample and plans created later use it for that
  * kind: a walk step or a draw is a binary search (O(log d)) instead of a pass
- * over the row.  Picks are identical (same prefix sums, same draws).  Graphs
- * where some bias of the kind is zero keep the streaming path.  Waits on
- * `stream`.  Errors: CSAW_ERR_INVALID (dynamic or unweighted kind),
+ * over the row.  Picks are identical (same prefix sums, same draws).  Where
+ * some bias of the kind is zero, sampling keeps the streaming path and walks
+ * search the packed array alone.  Waits on `stream`.  Errors: CSAW_ERR_INVALID (dynamic or unweighted kind),
  * CSAW_ERR_NOMEM, CSAW_ERR_CUDA. */
 csaw_status csaw_graph_build_cdf(csaw_graph* g, int32_t bias_kind, void* stream);
 
@@ -208,17 +208,19 @@ csaw_status csaw_walk(csaw_graph* g, const uint32_t* starts, uint64_t n_walkers,
  * kind over the whole graph into a temporary (stream-ordered, freed by the
  * call), and every step is then a search of it instead of a pass over the row:
  * the same paths, with the array's construction inside the call.  Ignored
- * otherwise.  Biases below 2^26: the packed array (8.6 bytes per edge + 16 per
- * vertex).  Larger ones: for edge weights the summaries of the prefix sums
+ * otherwise.  Biases below 2^26: the packed array (8.67 bytes per edge + 16 per
+ * vertex).  Larger ones, and where that does not fit in memory beside the
+ * call's buffers: for edge weights the summaries of the prefix sums
  * (every 8th and 64th) and per-vertex records {start, end, total}, about 1.14
  * bytes per edge + 32 per vertex, and a step forms its 8-edge group's sums
  * from the weights; for neighbour degree the whole cumulative array (9 bytes
  * per edge + 32 per vertex).
  * phase_ms (not NULL): the call records CUDA events on `stream` around its
  * phases, waits for the stream, and stores the device time of the array's
- * construction in phase_ms[0] (0 without build_cdf; what a plain call builds
- * by itself counts as walking) and of the walk kernels in phase_ms[1].  Errors: those of csaw_walk, and CSAW_ERR_INVALID
- * for an unknown teleport mode. */
+ * construction in phase_ms[0] (next to 0 without build_cdf; what a plain call
+ * builds by itself counts as walking) and of the walk kernels in phase_ms[1].
+ * Errors: those of csaw_walk, and CSAW_ERR_INVALID for an unknown teleport
+ * mode. */
 #define CSAW_TELEPORT_NONE 0
 #define CSAW_TELEPORT_RESTART 1
 #define CSAW_TELEPORT_JUMP 2
